@@ -42,8 +42,8 @@
 // columns.  The token operand lives in a second ring whose entries are sized by the
 // segment's row count and never wrap.
 //
-// CTA = 11 warps.  warp 0: weight producer (one lane issues TMA), warp 1: MMA issuer (one
-// lane) and owner of the TMEM allocation, warp 2: token-operand producer, warps 3..10:
+// CTA = 11 warps.  warp 0: weight producer (one lane issues TMA), warp 1: MMA issuer (the
+// warp in step, one elected lane issues) and owner of the TMEM allocation, warp 2: token-operand producer, warps 3..10:
 // epilogue, two warps per TMEM lane quarter that take alternate 16-token chunks (tcgen05.ld,
 // SwiGLU, transposition, 16-byte bf16 stores): where no second set of accumulators exists the
 // epilogue is not hidden behind the next tile, and two warps per scheduler hide its latencies.  Rings and the
@@ -745,8 +745,15 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
-            ItemWalk walk(args, claims, false, true, false, !GATED);
+        // All lanes walk, wait and compute, and the values of an item that came through shared
+        // memory are made warp-uniform for the compiler; one elected lane issues.  With the whole
+        // loop in one lane's branch the operands of every instruction had to be moved to the
+        // uniform registers the tensor pipe reads, and the issue bounded the pass: about 140
+        // cycles per instruction where N / 2 = 80 to 128 are its time (Qwen2 shape, T = 1280).
+        // Layer, before -> after: Qwen1.5 shape T = 5 77.4 -> 71.0 us, T = 640 270 -> 258,
+        // Mixtral shape T = 1280 1256 -> 1218, DeepSeek-V3 shape T = 128 3261 -> 3178.
+        {
+            ItemWalk walk(args, claims, false, lane == 0, true, !GATED);
             XRingWalk ring(args.x_units);
             int sw = 0;
             uint32_t pw = 0;
@@ -759,60 +766,61 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                 const int set = n_items % acc_sets;
                 const uint32_t acc_par = ((uint32_t)(n_items / acc_sets) & 1u) ^ 1u;
                 ++n_items;
-                bool acc_ready = false;
                 const uint32_t d0 = tmem_base + (uint32_t)set * 2u * acc_block;
-                const uint32_t tile_bytes = (uint32_t)it.h * 128u;
-                const int pieces = pieces16(it.n);
-                const uint32_t idesc = umma_idesc_bf16(pieces << 4);  // M = 128, N = token rows
+                const int hc = warp_uniform(it.h);
+                const uint32_t tile_bytes = (uint32_t)hc * 128u;
+                const int pieces = pieces16(warp_uniform(it.n));
+                // M = 128, N = token rows
+                const uint32_t idesc = umma_idesc_bf16(pieces << 4);
                 // weight blocks of the tile: gate and up, or the 128-row halves of a down tile
-                const int nblk = GATED ? 2 : (it.h + 127) >> 7;
+                const int nblk = GATED ? 2 : (hc + 127) >> 7;
                 // descriptor steps in 16-byte units: to the next block, to the next k box
                 const uint32_t blk16 = (GATED ? tile_bytes : 128u * 128u) >> 4;
                 const uint64_t w_box16 = (uint64_t)((NW * tile_bytes) >> 4);
                 const uint64_t x_box16 = (uint64_t)((pieces * FF_X_UNIT) >> 4);
-                const int K = it.k1;
-                for (int k0 = it.k0; ok && k0 < K; k0 += 64 * kb) {
-                    const int nbox = min(kb, (K - k0 + 63) >> 6);
+                const int n_box = warp_uniform((it.k1 - it.k0 + 63) >> 6);  // k boxes of the item
+                uint32_t accum = 0;
+                for (int box = 0; box < n_box; box += kb) {
+                    const int nbox = min(kb, n_box - box);
                     const int j = ring.count;
                     int pad;
                     const int at = ring.place(pieces * kb, pad);
                     const int xe = j % FF_X_ENTRIES;
                     const uint32_t xpar = (uint32_t)(j / FF_X_ENTRIES) & 1u;
                     const uint32_t xbase = ring_x + (uint32_t)at * FF_X_UNIT;
-                    if (!mbar_wait(w_full(sw), pw, abortp, args.status) ||
-                        !mbar_wait(x_full(xe), xpar, abortp, args.status)) {
+                    bool ready = mbar_wait(w_full(sw), pw, abortp, args.status) &&
+                                 mbar_wait(x_full(xe), xpar, abortp, args.status);
+                    if (box == 0)
+                        ready = ready && mbar_wait(acc_empty(set), acc_par, abortp, args.status);
+                    if (!__all_sync(0xffffffffu, ready)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    if (!acc_ready) {
-                        if (!mbar_wait(acc_empty(set), acc_par, abortp, args.status)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        acc_ready = true;
-                    }
                     uint64_t w_desc = umma_desc_sw128(ring_w + sw * args.w_slot_bytes);
                     uint64_t x_desc = umma_desc_sw128(xbase);
-                    for (int b = 0; b < nbox; ++b) {
-                        const uint32_t accum = ((k0 - it.k0) | b) != 0 ? 1u : 0u;
-                        if (nblk == 2)
-                            issue_k_box<2>(d0, acc_block, w_desc, blk16, x_desc, idesc, accum);
-                        else
-                            issue_k_box<1>(d0, acc_block, w_desc, blk16, x_desc, idesc, accum);
-                        w_desc += w_box16;
-                        x_desc += x_box16;
+                    if (elect_one()) {
+                        for (int b = 0; b < nbox; ++b) {
+                            if (nblk == 2)
+                                issue_k_box<2>(d0, acc_block, w_desc, blk16, x_desc, idesc, accum);
+                            else
+                                issue_k_box<1>(d0, acc_block, w_desc, blk16, x_desc, idesc, accum);
+                            w_desc += w_box16;
+                            x_desc += x_box16;
+                            accum = 1u;
+                        }
+                        umma_commit(x_empty(xe));
+                        umma_commit(w_empty(sw));  // reusable once these MMAs have read it
+                        if (box + kb >= n_box)
+                            umma_commit(acc_full(set));  // accumulators complete
                     }
-                    umma_commit(x_empty(xe));
-                    umma_commit(w_empty(sw));  // reusable once these MMAs have read it
+                    __syncwarp();
+                    accum = 1u;
                     if (++sw == NS) {
                         sw = 0;
                         pw ^= 1u;
                     }
                 }
-                if (ok)
-                    umma_commit(acc_full(set));  // accumulators complete
             }
             if (!walk.synced)
                 walk.sync(true);

@@ -52,6 +52,21 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
+// A value that is the same in all lanes of a converged warp, in a form the compiler knows to be.
+__device__ __forceinline__ int warp_uniform(int v) { return __reduce_max_sync(0xffffffffu, v); }
+
 // Bounded wait.  Returns false (and raises the abort flag) if the phase did not complete within
 // the wait limit or another role already aborted.  abort_flag[0] is the CTA's abort flag,
 // abort_flag[1] the limit in microseconds (FF_WAIT_NS unless the host shortened it).
