@@ -263,6 +263,8 @@ int geometry_override();
 // From MOE_SMALL_FUSED: 0 keeps calls of a few tokens on the chain of kernels every other call
 // uses, -1 (unset) lets them take the one-launch kernel.
 int small_layer_override();
+// From MOE_FF_PAIR: 0 / 1 forces the FFN kernels to run on single CTAs / on CTA pairs.
+int pair_override();
 // Token rows per segment of the routed groups for a call with T tokens: 128 or 256 (the plan and
 // the FFN kernels of one call must agree on it).
 int ffn_segment_rows(const moe_config_t &c, int T);
@@ -297,7 +299,8 @@ void prefer_max_shared_carveout(const void *kernel);
 // Launch with the programmatic-stream-serialization attribute: the kernel may begin while its
 // predecessor in the stream is still running and must execute griddepcontrol.wait before it
 // touches anything the predecessor produces.
-template <typename... KArgs, typename... Args>
+// CLUSTER > 1: clusters of that many consecutive CTAs.
+template <int CLUSTER = 1, typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t s, Args &&...args)
 {
@@ -307,11 +310,15 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = CLUSTER;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = CLUSTER > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 

@@ -37,19 +37,29 @@
 // producer/consumer hand-shake moves enough bytes to keep HBM busy and every weight row is
 // requested in 256 contiguous bytes; two sets of accumulators, so the epilogue of one tile
 // runs under the instructions of the next.  Contraction (segments of up to 256 rows, for
-// groups in the hundreds of rows): one k box per slot (32 KB) and per token entry (up to
-// 32 KB), four weight slots and three token entries, one set of accumulators of 2 x 256
-// columns.  The token operand lives in a second ring whose entries are sized by the
-// segment's row count and never wrap.
+// groups in the hundreds of rows): one k box per slot (32 KB) and per token entry, one set of
+// accumulators of 2 x 256 columns.  The token operand lives in a second ring whose entries are
+// sized by the segment's row count and never wrap.
+//
+// CTA pairs.  In the contraction geometry a cluster of two CTAs works on a tile of twice the
+// features with tcgen05 cta_group::2: each CTA loads its half of the weight rows and half of
+// the token rows, the tensor cores of both read both halves of the tokens, and each CTA's
+// TMEM and epilogue get its half of the features for all tokens.  What bounds this regime is
+// bytes: each SM is filled at no more than about 44 bytes per clock, a 256 x 256 tile of a single
+// CTA wants 64 at the full instruction rate and 256 x 160 wants 81; a pair's CTA wants 47 and 66.
+// The leader (even CTA) claims the work for both, its barriers count the bytes of both and its
+// commits release the slots of both.  Layer, single CTAs -> pairs: Qwen2 shape T = 1280
+// 1298 -> 1208 us, Mixtral shape T = 1280 1082 -> 1004.
 //
 // CTA = 11 warps.  warp 0: weight producer (one lane issues TMA), warp 1: MMA issuer (the
-// warp in step, one elected lane issues) and owner of the TMEM allocation, warp 2: token-operand producer, warps 3..10:
+// warp in step, one elected lane issues; idle in a pair's second CTA) and owner of the TMEM
+// allocation, warp 2: token-operand producer, warps 3..10:
 // epilogue, two warps per TMEM lane quarter that take alternate 16-token chunks (tcgen05.ld,
 // SwiGLU, transposition, 16-byte bf16 stores): where no second set of accumulators exists the
 // epilogue is not hidden behind the next tile, and two warps per scheduler hide its latencies.  Rings and the
 // accumulator sets are handed over through mbarriers.  Every wait is bounded: when one
 // gives up it raises the CTA's abort flag and the device status word, all roles leave their
-// loops, TMEM is freed and the kernel returns.
+// loops (the other CTA of a pair by its own limits), TMEM is freed and the kernel returns.
 //
 // Programmatic dependent launch: the kernels may start while their predecessor in the stream
 // is still running.  Work that depends only on the caller's inputs (shared-expert tiles in the
@@ -102,7 +112,7 @@ struct FfnArgs {
     int shared_tiles;  // tiles of the shared expert's rows; (tile, k chunk, segment) units are dealt
                        // round-robin to the CTAs; the first (units % tiles) tiles have one
                        // 16-row unit more
-    int max_tile;      // weight rows per tile: 128 (gate + up stacked) or 256 (down)
+    int max_tile;      // weight rows per tile and CTA: 128 (gate + up stacked) or 256 (down)
     int kboxes;        // 64-element k boxes per weight slot
     int w_slot_bytes;  // capacity of a weight slot
     int n_w_slots;
@@ -128,7 +138,7 @@ struct Item {
     int grp;     // 0 routed, 1 shared
     int expert;  // routed expert id (0 for the shared expert)
     int f0;      // first output feature (weight row inside the expert), multiple of 16
-    int h;       // output features of the tile, multiple of 16
+    int h;       // output features of the tile, multiple of 16 (pair: of 32, half of them per CTA)
     int row0;    // first token row (sorted row for routed groups, token for the shared expert)
     int n;       // token rows, 1..seg_rows
     int seg;     // index of the segment's progress counter (plan index; shared: segment number)
@@ -141,7 +151,9 @@ struct Item {
 // producer) claims chunks from a grid-wide counter and publishes them in a small ring; the
 // other roles read the same sequence, so all roles walk identical items.
 constexpr int FF_CLAIMS = 4;      // ring entries
-constexpr int FF_CLAIM_READERS = 2 + FF_EPI_WARPS;  // token producer, MMA issuer, epilogue warps
+// token producer, MMA issuer, epilogue warps; in the second CTA of a pair the weight producer
+// reads as well and nothing is issued
+constexpr int FF_CLAIM_READERS = 2 + FF_EPI_WARPS;
 
 constexpr int FF_CLAIM_WORDS = 8;  // lo, hi, and (round-robin mode) the item's group, decoded
 struct ClaimRing {
@@ -149,6 +161,9 @@ struct ClaimRing {
     uint32_t full0, empty0;    // shared addresses of the barrier arrays [FF_CLAIMS]
     volatile int *abort_flag;
     int32_t *status;
+    // a pair's ring: the leader claims for both CTAs and writes both copies of an entry; the
+    // readers of both CTAs arrive on the leader's empty barriers (cluster addresses)
+    uint32_t peer_data, peer_full0, leader_empty0;
 };
 
 // Walks the items of one CTA: its units of the shared expert first (dealt round-robin: they
@@ -173,13 +188,18 @@ __device__ __forceinline__ int balanced_segment_rows(int n, int nseg)
     return (((n + nseg - 1) / nseg) + 15) & ~15;
 }
 
+// PAIR: the worker is a CTA pair that walks the items together, each CTA computing half of a
+// tile's features; row units are then 32 weight rows, so that the halves are whole 16-row units.
+template <bool PAIR>
 struct ItemWalk {
+    static constexpr int USH = PAIR ? 5 : 4;  // log2 of the weight rows of a unit
     const FfnArgs &a;
     const ClaimRing &ring;
     const bool claimer;    // this thread claims; all others follow the ring
     const bool lead;       // this thread arrives on the ring's barriers for its role
     const bool warp_wide;  // the role is run by all 32 lanes in lock step (epilogue warps)
     const int max_units;
+    const int worker, workers;
     int n_claims;
     // shared expert: units (tile, k chunk, segment) sj, sj + grid, ...
     int sj, Us, s_base, s_rem, nseg_s, s_units;
@@ -202,18 +222,19 @@ struct ItemWalk {
     __device__ ItemWalk(const FfnArgs &args, const ClaimRing &r, bool is_claimer, bool is_lead,
                         bool is_warp_wide, bool already_synced)
         : a(args), ring(r), claimer(is_claimer), lead(is_lead), warp_wide(is_warp_wide),
-          max_units(args.max_tile >> 4),
+          max_units(args.max_tile >> 4),  // a pair's tile is twice as high, as is its unit
+          worker(PAIR ? blockIdx.x >> 1 : blockIdx.x), workers(PAIR ? gridDim.x >> 1 : gridDim.x),
           n_claims(0), synced(false), group_loaded(false), have_chunk(false), finished(false),
           end_published(false), n_pub(0),
           have_tile(false)
     {
-        Us = a.with_shared ? a.rows[1] >> 4 : 0;
+        Us = a.with_shared ? a.rows[1] >> USH : 0;
         s_base = a.shared_tiles ? Us / a.shared_tiles : 0;
         s_rem = a.shared_tiles ? Us % a.shared_tiles : 0;
-        sj = blockIdx.x;
+        sj = worker;
         nseg_s = (a.T + a.shared_seg - 1) / a.shared_seg;
         s_units = a.shared_tiles * a.shared_ksplit * nseg_s;
-        R0 = a.rows[0] >> 4;
+        R0 = a.rows[0] >> USH;
         nseg_total = fs = u = fs_hi = u_hi = 0;
         ntiles = (R0 + max_units - 1) / max_units;
         P = 0;
@@ -243,18 +264,17 @@ struct ItemWalk {
         synced = true;
     }
     // Claims the next chunk from the grid-wide counter (claimer only).  In round-robin mode
-    // the first item of every CTA is fixed -- item gridDim.x - 1 - blockIdx.x, so that the CTAs
+    // the first item of every worker is fixed -- item workers - 1 - worker, so that the workers
     // without a shared-expert tile (the high ones) take the first routed items -- and costs no
-    // round trip to the counter; the counter hands out the items from gridDim.x on.
+    // round trip to the counter; the counter hands out the items from `workers` on.
     __device__ void claim(int &lo, int &hi)
     {
         if (a.round_robin) {
-            lo = n_pub == 0 ? (int)(gridDim.x - 1 - blockIdx.x)
-                            : (int)gridDim.x + atomicAdd(a.claim_counter, 1);
+            lo = n_pub == 0 ? workers - 1 - worker : workers + atomicAdd(a.claim_counter, 1);
             hi = lo + 1;
         } else {
             const long long left = P - *reinterpret_cast<volatile int32_t *>(a.claim_counter);
-            const long long guided = left / (3 * (long long)gridDim.x);
+            const long long guided = left / (3 * (long long)workers);
             const int size = (int)(guided > max_units ? guided : max_units);
             lo = atomicAdd(a.claim_counter, size);
             hi = (int)(lo + (long long)size < P ? lo + size : P);
@@ -281,8 +301,14 @@ struct ItemWalk {
             grp.n = g.z;
             grp.first_seg = g.w;
         }
-        if (!mbar_wait(ring.empty0 + 8u * slot, par ^ 1u, ring.abort_flag, ring.status))
+        if (!mbar_wait<PAIR>(ring.empty0 + 8u * slot, par ^ 1u, ring.abort_flag, ring.status))
             return false;
+        if (PAIR) {
+            const uint32_t pe = ring.peer_data + slot * FF_CLAIM_WORDS * 4;
+            st_cluster_v4(pe, lo, hi, sidx, grp.expert);
+            st_cluster_v4(pe + 16, grp.row0, grp.n, grp.first_seg, 0);
+            mbar_arrive_cluster(ring.peer_full0 + 8u * slot);
+        }
         int *e = ring.data + slot * FF_CLAIM_WORDS;
         e[0] = lo;
         e[1] = hi;
@@ -311,7 +337,7 @@ struct ItemWalk {
         if (claimer) {
             for (;;) {
                 // (the counter is only read where the answer can be yes)
-                const long long ample = 4 * (long long)gridDim.x * (a.round_robin ? 1 : max_units);
+                const long long ample = 4 * (long long)workers * (a.round_robin ? 1 : max_units);
                 const bool plenty =
                     P > ample && P - *reinterpret_cast<volatile int32_t *>(a.claim_counter) > ample;
                 if (end_published || n_pub >= n_claims + (plenty ? 2 : 1))
@@ -319,7 +345,7 @@ struct ItemWalk {
                 if (!publish_one())
                     return false;
             }
-        } else if (!mbar_wait(ring.full0 + 8u * slot, par, ring.abort_flag, ring.status)) {
+        } else if (!mbar_wait<PAIR>(ring.full0 + 8u * slot, par, ring.abort_flag, ring.status)) {
             return false;
         }
         ++n_claims;
@@ -333,8 +359,12 @@ struct ItemWalk {
         if (!claimer) {
             if (warp_wide)
                 __syncwarp();  // every lane has read the entry before it is released
-            if (lead)
-                mbar_arrive(ring.empty0 + 8u * slot);
+            if (lead) {
+                if (PAIR)
+                    mbar_arrive_cluster(ring.leader_empty0 + 8u * slot);
+                else
+                    mbar_arrive(ring.empty0 + 8u * slot);
+            }
         }
         return lo >= 0;
     }
@@ -346,8 +376,8 @@ struct ItemWalk {
                 if (t_s < t_s_end) {
                     it.grp = t_grp;
                     it.expert = t_expert;
-                    it.f0 = t_u0 << 4;
-                    it.h = t_h << 4;
+                    it.f0 = t_u0 << USH;
+                    it.h = t_h << USH;
                     it.row0 = t_row0 + t_s * t_seg_rows;
                     it.n = min(t_seg_rows, t_n - t_s * t_seg_rows);
                     it.seg = t_seg0 + t_s;
@@ -377,7 +407,7 @@ struct ItemWalk {
                 t_s = q;
                 t_s_end = q + 1;
                 t_once = nseg_s <= 1;
-                sj += gridDim.x;
+                sj += workers;
                 have_tile = true;
                 continue;
             }
@@ -477,6 +507,14 @@ struct XRingWalk {
 
 __device__ __forceinline__ int pieces16(int n) { return (n + 15) >> 4; }
 
+// 16-row pieces of a segment's n token rows that one CTA loads: all, or half of them (rounded
+// up) for each CTA of a pair.
+template <bool PAIR>
+__device__ __forceinline__ int token_pieces(int n)
+{
+    return PAIR ? (n + 31) >> 5 : pieces16(n);
+}
+
 // One output value of an epilogue thread: h = silu(g) * u (GATED) or the plain sum, as bf16.
 template <bool GATED>
 __device__ __forceinline__ __nv_bfloat16 epilogue_value(uint32_t g, uint32_t u)
@@ -531,7 +569,7 @@ __device__ __forceinline__ void transpose_16x32(const uint32_t (&w)[16], int lan
 }
 
 // GATED: W_gate and W_up tiles -> h = silu(g) * u.   !GATED: W_down tiles -> y.
-template <bool GATED>
+template <bool GATED, bool PAIR>
 __global__ void __launch_bounds__(FF_THREADS, 1)
 ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
 {
@@ -541,7 +579,7 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
     __shared__ uint64_t bars[2 * FF_MAX_W_SLOTS + 2 * FF_X_ENTRIES + 4 + 2 * FF_CLAIMS];
     __shared__ uint32_t tmem_base_holder;
     __shared__ int abort_flag[2];  // [0] raised by the first wait that gives up, [1] wait limit (us)
-    __shared__ int claim_data[FF_CLAIMS * FF_CLAIM_WORDS];
+    __shared__ __align__(16) int claim_data[FF_CLAIMS * FF_CLAIM_WORDS];
 
     const int NS = args.n_w_slots;
     const int kb = args.kboxes;
@@ -564,6 +602,11 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
     const uint32_t claim_empty0 = claim_full0 + 8u * FF_CLAIMS;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // pair: the leader's barriers count the bytes that land in both CTAs, its issuer feeds both
+    // tensor pipes and releases the slots of both
+    const int rank = PAIR ? (int)(blockIdx.x & 1) : 0;
+    constexpr int CTAS = PAIR ? 2 : 1;
+    auto leader_bar = [&](uint32_t bar) { return PAIR ? map_to_rank(bar, 0) : bar; };
 
     if (threadIdx.x == 0) {
         abort_flag[0] = 0;
@@ -578,28 +621,40 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(acc_full(b), 1);
-            mbar_init(acc_empty(b), FF_EPI_WARPS);
+            mbar_init(acc_empty(b), CTAS * FF_EPI_WARPS);
         }
         for (int i = 0; i < FF_CLAIMS; ++i) {
             mbar_init(claim_full0 + 8u * i, 1);
-            mbar_init(claim_empty0 + 8u * i, FF_CLAIM_READERS);
+            mbar_init(claim_empty0 + 8u * i, CTAS * FF_CLAIM_READERS);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(&tmem_base_holder)),
-                     "r"(FF_TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             smem_u32(&tmem_base_holder)),
+                         "r"(FF_TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                             smem_u32(&tmem_base_holder)),
+                         "r"(FF_TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
     tc_fence_before();
     __syncthreads();
+    if (PAIR)
+        cluster_barrier();  // the other CTA's barriers are initialised, its TMEM is allocated
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_holder;
     volatile int *abortp = abort_flag;
-    const ClaimRing claims{claim_data, claim_full0, claim_empty0, abortp, args.status};
+    const ClaimRing claims{claim_data, claim_full0, claim_empty0, abortp, args.status,
+                           PAIR ? map_to_rank(smem_u32(claim_data), rank ^ 1) : 0u,
+                           PAIR ? map_to_rank(claim_full0, rank ^ 1) : 0u, leader_bar(claim_empty0)};
 
     if (warp == 0) {
         // ---------------- weight producer ----------------
@@ -607,7 +662,7 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
             // gate/up pass: the shared expert's weights and x are the caller's inputs, so those
             // items run before the wait.  Down pass: every weight tile may be fetched ahead --
             // the launch order guarantees that the plan is complete when this kernel starts.
-            ItemWalk walk(args, claims, true, false, false, !GATED);
+            ItemWalk<PAIR> walk(args, claims, rank == 0, rank != 0, false, !GATED);
             const uint64_t pol_once = l2_policy_evict_first();
             bool launched = !GATED;
             if (!GATED)
@@ -622,8 +677,9 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                     launched = true;
                 }
                 const int K = it.k1;
-                const uint32_t tile_bytes = (uint32_t)it.h * 128u;
-                const int wrow = it.expert * args.rows[0] + it.f0;  // expert = 0 for the shared kind
+                const int hc = it.h / CTAS;  // this CTA's rows of the tile
+                const uint32_t tile_bytes = (uint32_t)hc * 128u;
+                const int wrow = it.expert * args.rows[0] + it.f0 + rank * hc;  // expert = 0 for the shared kind
                 for (int k0 = it.k0; k0 < K; k0 += 64 * kb) {
                     const int nbox = min(kb, (K - k0 + 63) >> 6);
                     if (!mbar_wait(w_empty(slot), phase ^ 1u, abortp, args.status)) {
@@ -631,21 +687,27 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                         break;
                     }
                     const uint32_t base = ring_w + slot * args.w_slot_bytes;
-                    mbar_expect_tx(w_full(slot), nbox * NW * tile_bytes);
+                    const uint32_t full = leader_bar(w_full(slot));
+                    if (rank == 0)
+                        mbar_expect_tx(w_full(slot), CTAS * nbox * NW * tile_bytes);
                     for (int b = 0; b < nbox; ++b) {
 #pragma unroll
                         for (int m = 0; m < NW; ++m) {
                             // the tile as boxes of 128, 64, 32 and 16 rows, stacked
                             uint32_t dst = base + (uint32_t)(b * NW + m) * tile_bytes;
-                            int row = wrow, rem = it.h;
+                            int row = wrow, rem = hc;
                             while (rem > 0) {
                                 const int hi = rem >= 128 ? 0 : (rem >= 64 ? 1 : (rem >= 32 ? 2 : 3));
                                 const int bh = 128 >> hi;
-                                if (it.w_once)
-                                    tma_load_2d_hint(dst, &maps.w[it.grp][m][hi], w_full(slot), k0 + 64 * b,
-                                                     row, pol_once);
+                                const CUtensorMap *map = &maps.w[it.grp][m][hi];
+                                if (PAIR && it.w_once)
+                                    tma_load_2d_pair_hint(dst, map, full, k0 + 64 * b, row, pol_once);
+                                else if (PAIR)
+                                    tma_load_2d_pair(dst, map, full, k0 + 64 * b, row);
+                                else if (it.w_once)
+                                    tma_load_2d_hint(dst, map, full, k0 + 64 * b, row, pol_once);
                                 else
-                                    tma_load_2d(dst, &maps.w[it.grp][m][hi], w_full(slot), k0 + 64 * b, row);
+                                    tma_load_2d(dst, map, full, k0 + 64 * b, row);
                                 dst += (uint32_t)bh * 128u;
                                 row += bh;
                                 rem -= bh;
@@ -658,6 +720,14 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                     }
                 }
             }
+            if (PAIR)  // the leader's last releases have arrived before this CTA may exit
+                for (int i = 0; ok && i < NS; ++i) {
+                    ok = mbar_wait(w_empty(slot), phase ^ 1u, abortp, args.status);
+                    if (++slot == NS) {
+                        slot = 0;
+                        phase ^= 1u;
+                    }
+                }
             if (!walk.synced)
                 walk.sync(true);
             if (!launched)
@@ -668,7 +738,7 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
         if (lane == 0) {
             // down pass: h is written by the preceding kernel, which may still be running; a
             // segment's rows are fetched once its progress counter says they are complete
-            ItemWalk walk(args, claims, false, true, false, !GATED);
+            ItemWalk<PAIR> walk(args, claims, false, true, false, !GATED);
             XRingWalk ring(args.x_units);
             int seen = -1;  // (group kind, segment) key last found complete
             const uint64_t pol_keep = l2_policy_evict_last();
@@ -693,8 +763,9 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                         asm volatile("fence.proxy.async.global;" ::: "memory");
                     }
                 }
-                const int pieces = pieces16(it.n);
+                const int pieces = token_pieces<PAIR>(it.n);  // this CTA's share of the rows
                 const int m = pieces * kb;
+                const int xrow = it.row0 + rank * (pieces << 4);
                 for (int k0 = it.k0; ok && k0 < K; k0 += 64 * kb) {
                     const int nbox = min(kb, (K - k0 + 63) >> 6);
                     const int j = ring.count;
@@ -721,16 +792,22 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                     v_start_of[e] = v_start;
                     v_cur = v_end;
                     const uint32_t base = ring_x + (uint32_t)at * FF_X_UNIT;
-                    mbar_expect_tx(x_full(e), (uint32_t)(nbox * pieces) * FF_X_UNIT);
+                    const uint32_t full = leader_bar(x_full(e));
+                    if (rank == 0)
+                        mbar_expect_tx(x_full(e), (uint32_t)(CTAS * nbox * pieces) * FF_X_UNIT);
                     for (int b = 0; b < nbox; ++b) {
                         // the entry's rows as boxes of 128, 64, 32 and 16 rows
                         uint32_t dst = base + (uint32_t)(b * pieces) * FF_X_UNIT;
-                        int row = it.row0, rem = pieces << 4;
+                        int row = xrow, rem = pieces << 4;
                         while (rem > 0) {
                             const int hi = rem >= 128 ? 0 : (rem >= 64 ? 1 : (rem >= 32 ? 2 : 3));
                             const int bh = 128 >> hi;
-                            tma_load_2d_hint(dst, &maps.x[it.grp][hi], x_full(e), k0 + 64 * b, row,
-                                             pol_keep);
+                            if (PAIR)
+                                tma_load_2d_pair_hint(dst, &maps.x[it.grp][hi], full, k0 + 64 * b, row,
+                                                      pol_keep);
+                            else
+                                tma_load_2d_hint(dst, &maps.x[it.grp][hi], full, k0 + 64 * b, row,
+                                                 pol_keep);
                             dst += (uint32_t)bh * 128u;
                             row += bh;
                             rem -= bh;
@@ -738,6 +815,10 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                     }
                 }
             }
+            if (PAIR)  // as for the weight slots
+                for (; ok && released < ring.count; ++released)
+                    ok = mbar_wait(x_empty(released % FF_X_ENTRIES),
+                                   (uint32_t)(released / FF_X_ENTRIES) & 1u, abortp, args.status);
             if (!walk.synced)
                 walk.sync(true);
             if (!GATED)
@@ -752,8 +833,8 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
         // cycles per instruction where N / 2 = 80 to 128 are its time (Qwen2 shape, T = 1280).
         // Layer, before -> after: Qwen1.5 shape T = 5 77.4 -> 71.0 us, T = 640 270 -> 258,
         // Mixtral shape T = 1280 1256 -> 1218, DeepSeek-V3 shape T = 128 3261 -> 3178.
-        {
-            ItemWalk walk(args, claims, false, lane == 0, true, !GATED);
+        if (rank == 0) {
+            ItemWalk<PAIR> walk(args, claims, false, lane == 0, true, !GATED);
             XRingWalk ring(args.x_units);
             int sw = 0;
             uint32_t pw = 0;
@@ -767,11 +848,11 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                 const uint32_t acc_par = ((uint32_t)(n_items / acc_sets) & 1u) ^ 1u;
                 ++n_items;
                 const uint32_t d0 = tmem_base + (uint32_t)set * 2u * acc_block;
-                const int hc = warp_uniform(it.h);
+                const int hc = warp_uniform(it.h) / CTAS;
                 const uint32_t tile_bytes = (uint32_t)hc * 128u;
-                const int pieces = pieces16(warp_uniform(it.n));
-                // M = 128, N = token rows
-                const uint32_t idesc = umma_idesc_bf16(pieces << 4);
+                const int pieces = token_pieces<PAIR>(warp_uniform(it.n));
+                // M = 128 per CTA, N = token rows
+                const uint32_t idesc = umma_idesc_bf16(CTAS * (pieces << 4), CTAS * 128);
                 // weight blocks of the tile: gate and up, or the 128-row halves of a down tile
                 const int nblk = GATED ? 2 : (hc + 127) >> 7;
                 // descriptor steps in 16-byte units: to the next block, to the next k box
@@ -791,7 +872,7 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                     bool ready = mbar_wait(w_full(sw), pw, abortp, args.status) &&
                                  mbar_wait(x_full(xe), xpar, abortp, args.status);
                     if (box == 0)
-                        ready = ready && mbar_wait(acc_empty(set), acc_par, abortp, args.status);
+                        ready = ready && mbar_wait<PAIR>(acc_empty(set), acc_par, abortp, args.status);
                     if (!__all_sync(0xffffffffu, ready)) {
                         ok = false;
                         break;
@@ -802,17 +883,17 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                     if (elect_one()) {
                         for (int b = 0; b < nbox; ++b) {
                             if (nblk == 2)
-                                issue_k_box<2>(d0, acc_block, w_desc, blk16, x_desc, idesc, accum);
+                                issue_k_box<2, PAIR>(d0, acc_block, w_desc, blk16, x_desc, idesc, accum);
                             else
-                                issue_k_box<1>(d0, acc_block, w_desc, blk16, x_desc, idesc, accum);
+                                issue_k_box<1, PAIR>(d0, acc_block, w_desc, blk16, x_desc, idesc, accum);
                             w_desc += w_box16;
                             x_desc += x_box16;
                             accum = 1u;
                         }
-                        umma_commit(x_empty(xe));
-                        umma_commit(w_empty(sw));  // reusable once these MMAs have read it
+                        umma_commit<PAIR>(x_empty(xe));
+                        umma_commit<PAIR>(w_empty(sw));  // reusable once these MMAs have read it
                         if (box + kb >= n_box)
-                            umma_commit(acc_full(set));  // accumulators complete
+                            umma_commit<PAIR>(acc_full(set));  // accumulators complete
                     }
                     __syncwarp();
                     accum = 1u;
@@ -831,7 +912,7 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
         // stores need not wait for the preceding kernel (the token producer does, per segment)
         const int quarter = warp & 3;  // TMEM lanes 32*quarter .. +31 belong to this warp
         const int chunk0 = warp >= 7 ? 16 : 0;  // the quarter's second warp takes the odd chunks
-        ItemWalk walk(args, claims, false, lane == 0, true, !GATED);
+        ItemWalk<PAIR> walk(args, claims, false, lane == 0, true, !GATED);
         int n_items = 0;
         Item it;
         for (;;) {
@@ -849,11 +930,12 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                 break;
             tc_fence_after();
             // a thread owns one weight row (output feature) of a block and walks the tokens
-            const int nblk = GATED ? 1 : (it.h + 127) >> 7;  // gate and up are read together
+            const int hc = it.h / CTAS;
+            const int nblk = GATED ? 1 : (hc + 127) >> 7;  // gate and up are read together
             const int ld = args.out_ld[it.grp];
             const int npad = pieces16(it.n) << 4;
             for (int m = 0; m < nblk; ++m) {
-                const int rows_blk = GATED ? it.h : min(128, it.h - 128 * m);
+                const int rows_blk = GATED ? hc : min(128, hc - 128 * m);
                 if (quarter * 32 >= rows_blk)
                     break;  // this warp's lanes lie beyond the tile (uniform)
                 // after the transposition this lane stores features 8 * (lane >> 3) .. + 7 of
@@ -861,7 +943,7 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                 const int fgrp = quarter * 32 + 8 * (lane >> 3);
                 const bool grp_ok = fgrp < rows_blk;
                 __nv_bfloat16 *out = args.out[it.grp] + it.out_off + (size_t)it.row0 * ld + it.f0 +
-                                     128 * m + fgrp;
+                                     rank * hc + 128 * m + fgrp;
                 const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) +
                                     (uint32_t)set * 2u * acc_block + (uint32_t)m * acc_block;
                 // two register buffers: the TMEM load of this warp's next 16 tokens is in flight
@@ -906,12 +988,15 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                 asm volatile("fence.proxy.async.global;" ::: "memory");
             __syncwarp();
             if (lane == 0) {
-                mbar_arrive(acc_empty(set));
+                if (PAIR)
+                    mbar_arrive_cluster(leader_bar(acc_empty(set)));
+                else
+                    mbar_arrive(acc_empty(set));
                 if (GATED) {
                     // publish: this warp's part of the tile is in h (a releasing reduction: the
                     // warp does not wait for its stores to become visible, the counter does)
                     asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(args.done[it.grp] + it.seg),
-                                 "r"(it.h >> 4)
+                                 "r"(hc >> 4)
                                  : "memory");
                 }
             }
@@ -931,12 +1016,19 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
     }
     tc_fence_before();
     __syncthreads();
+    if (PAIR)
+        cluster_barrier();  // nothing of the other CTA refers to this one's memory any more
     if (warp == 1) {
         __syncwarp();  // lane 0 arrived from the issue loop: reconverge for the aligned dealloc
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
-                     "r"(FF_TMEM_COLS)
-                     : "memory");
+        if (PAIR)
+            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
+                         "r"(FF_TMEM_COLS)
+                         : "memory");
+        else
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
+                         "r"(FF_TMEM_COLS)
+                         : "memory");
     }
 }
 
@@ -1135,6 +1227,28 @@ static double expected_active_experts(int E, int k, int T)
 
 static int ffn_grid() { return sm_count(); }
 
+// Whether the FFN kernels of a call run on CTA pairs: in the contraction geometry.  In the
+// streaming geometry the token rows are a small part of what an SM loads (4 rows per group on the
+// DeepSeek-V3 shape at T = 128: 3172 us on single CTAs, 3248 on pairs; Mixtral shape T = 80 443
+// and 450), and a pair waits for the slower of its two streams.
+static bool ffn_pairs(const moe_config_t &c, int T)
+{
+    const int force = pair_override();
+    if (force >= 0)
+        return force == 1;
+    return ffn_segment_rows(c, T) > FF_SEG;
+}
+
+// What pulls work items: a CTA, or a pair of CTAs whose tiles are twice as high.
+struct FfnWorkers {
+    int ctas, count;
+};
+static FfnWorkers ffn_workers(const moe_config_t &c, int T)
+{
+    const int ctas = ffn_pairs(c, T) ? 2 : 1;
+    return FfnWorkers{ctas, ffn_grid() / ctas};
+}
+
 // Segment size of a call (the N limit of its tensor-core instructions).  Groups in the hundreds
 // of rows want the contraction geometry: segments of 256 rows, so that a weight tile is fetched
 // once per 256 tokens and the instruction runs at its full rate.  Small groups want the
@@ -1186,17 +1300,18 @@ static int shared_segment_rows(const moe_config_t &c, int T)
 // pass (or less), with the tile height within [min_tile, max_tile] rows (a weight block
 // costs the same instruction time whether it holds 16 rows or 128).
 static int shared_tile_count(const moe_config_t &c, int T, int rows_routed, int rows_shared,
-                             int K_routed, int K_shared, int ksplit, int min_tile, int max_tile,
-                             int grid)
+                             int K_routed, int K_shared, int ksplit, int min_tile, int max_tile)
 {
+    const FfnWorkers wk = ffn_workers(c, T);
+    const int unit = 16 * wk.ctas;  // (a pair's tiles: twice the height, units of 32 rows)
     const int seg_s = shared_segment_rows(c, T), seg_r = ffn_segment_rows(c, T);
     const int nseg_s = (T + seg_s - 1) / seg_s;
-    const int units = rows_shared >> 4;
+    const int units = rows_shared / unit;
     const double k_ratio = (double)K_shared / K_routed;  // cost of a shared row unit per segment
     const double n_act = expected_active_experts(c.n_experts, c.top_k, T);
     const double segs_r = n_act * ceil((double)T * c.top_k / n_act / seg_r);
-    const double total = units * k_ratio * nseg_s + segs_r * (rows_routed >> 4);
-    int tu = (int)ceil(total / grid / (k_ratio / ksplit));
+    const double total = units * k_ratio * nseg_s + segs_r * (rows_routed / unit);
+    int tu = (int)ceil(total / wk.count / (k_ratio / ksplit));
     if (tu < (min_tile >> 4))
         tu = min_tile >> 4;
     if (tu > (max_tile >> 4))
@@ -1216,7 +1331,9 @@ static void ffn_geometry(const moe_config_t &c, int T, FfnArgs &a)
     a.kboxes = wide ? 1 : 2;
     a.acc_sets = wide ? 1 : 2;
     a.w_slot_bytes = 256 * 128 * a.kboxes;  // a full tile: 256 rows per k box
-    const int x_ring_bytes = (!wide && small_token_ring(c, T)) ? 32 * 1024 : 96 * 1024;
+    // (a CTA of a pair holds half of a segment's rows: entries of at most 16 KB in both geometries)
+    const int x_ring_bytes = ffn_pairs(c, T) ? (wide ? 64 * 1024 : 32 * 1024)
+                             : (!wide && small_token_ring(c, T)) ? 32 * 1024 : 96 * 1024;
     a.x_units = x_ring_bytes / FF_X_UNIT;
     const int avail = FF_SMEM_LIMIT - 1024 - 512;  // alignment slack, static shared memory
     int ns = (avail - x_ring_bytes) / a.w_slot_bytes;
@@ -1235,8 +1352,7 @@ static void ffn_geometry(const moe_config_t &c, int T, FfnArgs &a)
 // Then, and when there are so many tiles per CTA that the last wave hardly matters, the routed
 // work is dealt round-robin as (segment, tile) items: full tiles only, and the CTAs work on a
 // few groups at a time.
-static bool use_round_robin(const moe_config_t &c, int T, int rows_routed, int K_routed, int max_tile,
-                            int grid)
+static bool use_round_robin(const moe_config_t &c, int T, int rows_routed, int K_routed, int max_tile)
 {
     const int force = schedule_override();
     if (force >= 0)
@@ -1244,12 +1360,14 @@ static bool use_round_robin(const moe_config_t &c, int T, int rows_routed, int K
     const double n_act = expected_active_experts(c.n_experts, c.top_k, T);
     const double rows_per_group = (double)T * c.top_k / n_act;
     const double segs = n_act * ceil(rows_per_group / ffn_segment_rows(c, T));
-    const double tiles_per_cta = segs * ((rows_routed + max_tile - 1) / max_tile) / grid;
-    const double token_bytes = rows_per_group * K_routed * 2.0 * grid;
+    const FfnWorkers wk = ffn_workers(c, T);
+    const int tile = max_tile * wk.ctas;
+    const double tiles_per_cta = segs * ((rows_routed + tile - 1) / tile) / wk.count;
+    const double token_bytes = rows_per_group * K_routed * 2.0 * wk.count;
     return tiles_per_cta < 3.0 || tiles_per_cta >= 12.0 || token_bytes > 200.0 * 1024 * 1024;
 }
 
-template <bool GATED>
+template <bool GATED, bool PAIR>
 static cudaError_t launch_ffn(FfnArgs &a, const FfnMaps &maps, cudaStream_t s)
 {
     // the opt-in to large dynamic shared memory is a per-device attribute of the kernel
@@ -1258,7 +1376,7 @@ static cudaError_t launch_ffn(FfnArgs &a, const FfnMaps &maps, cudaStream_t s)
     if (cudaGetDevice(&dev) != cudaSuccess)
         return cudaErrorInvalidDevice;
     if (!configured.done(dev)) {
-        cudaError_t e = cudaFuncSetAttribute(ffn_fused_kernel<GATED>,
+        cudaError_t e = cudaFuncSetAttribute(ffn_fused_kernel<GATED, PAIR>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              FF_SMEM_LIMIT - 512);
         if (e != cudaSuccess)
@@ -1268,7 +1386,9 @@ static cudaError_t launch_ffn(FfnArgs &a, const FfnMaps &maps, cudaStream_t s)
     const size_t smem = (size_t)a.x_units * FF_X_UNIT + (size_t)a.n_w_slots * a.w_slot_bytes + 1024;
     if (a.n_w_slots < 2 || smem > FF_SMEM_LIMIT - 512)
         return cudaErrorInvalidConfiguration;
-    return launch_pdl(ffn_fused_kernel<GATED>, dim3(ffn_grid()), dim3(FF_THREADS), smem, s, a, maps);
+    const int grid = PAIR ? ffn_grid() & ~1 : ffn_grid();
+    return launch_pdl<PAIR ? 2 : 1>(ffn_fused_kernel<GATED, PAIR>, dim3(grid), dim3(FF_THREADS), smem, s, a,
+                                    maps);
 }
 
 cudaError_t launch_ffn_gateup(const moe_config_t &c, const moe_weights_t &w, const __nv_bfloat16 *x,
@@ -1285,7 +1405,7 @@ cudaError_t launch_ffn_gateup(const moe_config_t &c, const moe_weights_t &w, con
     a.shared_ksplit = 1;
     a.shared_kchunk = (c.hidden + 127) / 128 * 128;
     a.shared_tiles = with_shared ? shared_tile_count(c, T, c.inter, c.shared_inter, c.hidden, c.hidden,
-                                                     1, 64, 128, ffn_grid())
+                                                     1, 64, 128)
                                  : 0;
     ffn_geometry(c, T, a);
     FfnMaps maps;
@@ -1316,13 +1436,13 @@ cudaError_t launch_ffn_gateup(const moe_config_t &c, const moe_weights_t &w, con
     a.claim_counter = plan.header + 2;
     a.done[0] = plan.done_routed;
     a.done[1] = plan.done_shared;
-    a.round_robin = use_round_robin(c, T, c.inter, c.hidden, a.max_tile, ffn_grid()) ? 1 : 0;
+    a.round_robin = use_round_robin(c, T, c.inter, c.hidden, a.max_tile) ? 1 : 0;
     a.routed_ksplit = 1;
     a.routed_kchunk = c.hidden;
     a.status = status;
     a.T = T;
     a.with_shared = with_shared ? 1 : 0;
-    return launch_ffn<true>(a, maps, s);
+    return ffn_pairs(c, T) ? launch_ffn<true, true>(a, maps, s) : launch_ffn<true, false>(a, maps, s);
 }
 
 // Length of a k chunk when K is cut into about `parts` pieces (a multiple of the 128-column
@@ -1346,7 +1466,7 @@ static double routed_down_items(const moe_config_t &c, int T)
 // adds the planes.  (Fewer than three items per CTA also means the pass deals single items.)
 int routed_down_parts(const moe_config_t &c, int T)
 {
-    if (!use_round_robin(c, T, c.hidden, c.inter, 256, ffn_grid()))
+    if (!use_round_robin(c, T, c.hidden, c.inter, 256))
         return 1;
     int parts = (int)ceil(3.0 * ffn_grid() / routed_down_items(c, T));
     const int cap = c.inter / 1024;  // chunks below half a megabyte cost more than they level
@@ -1404,7 +1524,7 @@ cudaError_t launch_ffn_down(const moe_config_t &c, const moe_weights_t &w, int T
     a.shared_kchunk = with_shared ? split_chunk(c.shared_inter, a.shared_ksplit) : 128;
     a.shared_part_stride = (long long)T * c.hidden;
     a.shared_tiles = with_shared ? shared_tile_count(c, T, c.hidden, c.hidden, c.inter, c.shared_inter,
-                                                     a.shared_ksplit, 128, 256, ffn_grid())
+                                                     a.shared_ksplit, 128, 256)
                                  : 0;
     ffn_geometry(c, T, a);
     FfnMaps maps;
@@ -1432,7 +1552,7 @@ cudaError_t launch_ffn_down(const moe_config_t &c, const moe_weights_t &w, int T
     a.claim_counter = plan.header + 3;
     a.done[0] = plan.done_routed;
     a.done[1] = plan.done_shared;
-    a.round_robin = use_round_robin(c, T, c.hidden, c.inter, a.max_tile, ffn_grid()) ? 1 : 0;
+    a.round_robin = use_round_robin(c, T, c.hidden, c.inter, a.max_tile) ? 1 : 0;
     if (routed_parts > 1 && !a.round_robin)
         return cudaErrorInvalidValue;  // planes exist only where single items are dealt
     a.routed_ksplit = routed_parts;
@@ -1444,7 +1564,7 @@ cudaError_t launch_ffn_down(const moe_config_t &c, const moe_weights_t &w, int T
     a.status = status;
     a.T = T;
     a.with_shared = with_shared ? 1 : 0;
-    return launch_ffn<false>(a, maps, s);
+    return ffn_pairs(c, T) ? launch_ffn<false, true>(a, maps, s) : launch_ffn<false, false>(a, maps, s);
 }
 
 }  // namespace moe

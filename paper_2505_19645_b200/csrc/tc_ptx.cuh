@@ -39,17 +39,58 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
                  : "memory");
 }
 
+// CLUSTER: the arrivals come from (or cover stores of) the other CTA of a pair.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
+    if (CLUSTER)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
     return ok != 0;
+}
+
+// ---- CTA pairs (a cluster of two) ---------------------------------------------------------
+
+// Address of `smem` (a shared-memory address of this CTA) in the cluster's CTA `rank`.
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t smem, uint32_t rank)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem), "r"(rank));
+    return a;
+}
+
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar)
+                 : "memory");
+}
+
+__device__ __forceinline__ void st_cluster_v4(uint32_t cluster_addr, int a, int b, int c, int d)
+{
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b),
+                 "r"(c), "r"(d)
+                 : "memory");
+}
+
+// Every thread of both CTAs (warps need not be converged).
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // One lane of a converged warp.
@@ -70,16 +111,17 @@ __device__ __forceinline__ int warp_uniform(int v) { return __reduce_max_sync(0x
 // Bounded wait.  Returns false (and raises the abort flag) if the phase did not complete within
 // the wait limit or another role already aborted.  abort_flag[0] is the CTA's abort flag,
 // abort_flag[1] the limit in microseconds (FF_WAIT_NS unless the host shortened it).
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag,
                                           int32_t *status)
 {
-    if (mbar_try_wait(bar, parity))
+    if (mbar_try_wait<CLUSTER>(bar, parity))
         return true;
     const uint64_t t0 = global_ns();
     for (;;) {
 #pragma unroll 1
         for (int i = 0; i < 64; ++i)
-            if (mbar_try_wait(bar, parity))
+            if (mbar_try_wait<CLUSTER>(bar, parity))
                 return true;
         if (*abort_flag)
             return false;
@@ -144,6 +186,29 @@ __device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const CUtensorMap
         : "memory");
 }
 
+// The same loads into this CTA's shared memory from a CTA of a pair: the mbarrier (a cluster
+// address) may be the other CTA's.
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, uint32_t cluster_bar,
+                                                 int c0, int c1)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2 "
+        "[%0], [%1, {%3, %4}], [%2];"
+        :
+        : "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(cluster_bar), "r"(c0), "r"(c1)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_2d_pair_hint(uint32_t dst, const CUtensorMap *map,
+                                                      uint32_t cluster_bar, int c0, int c1, uint64_t policy)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2"
+        ".L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
+        :
+        : "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(cluster_bar), "r"(c0), "r"(c1), "l"(policy)
+        : "memory");
+}
+
 // L2 policies: weights that are read once should leave L2 first, the token rows (re-read for
 // every weight tile of their group) last -- otherwise the weight stream, which is larger than
 // L2, evicts them between two tiles.
@@ -168,29 +233,52 @@ __device__ __forceinline__ void prefetch_map(const CUtensorMap *map)
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+// PAIR: one instruction for both CTAs of a pair, issued by its leader.  Each CTA's shared memory
+// holds, at the same offsets, its 128 rows of A and half of the rows of B; each CTA's TMEM gets
+// its 128 rows of D with all N columns.
+template <bool PAIR>
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                           uint32_t idesc, uint32_t accumulate)
 {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        :
-        : "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
+    if (PAIR)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+            :
+            : "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+            :
+            : "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+            : "memory");
 }
 
 // The same, always accumulating (no predicate to derive from a register).
+template <bool PAIR>
 __device__ __forceinline__ void umma_bf16_acc(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                               uint32_t idesc)
 {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.eq.b32 p, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        :
-        : "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc)
-        : "memory");
+    if (PAIR)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.eq.b32 p, 0, 0;\n\t"
+            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+            :
+            : "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.eq.b32 p, 0, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+            :
+            : "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc)
+            : "memory");
 }
 
 // The instructions of one 64-element k box: four k steps of 16, each against NBLK weight blocks
@@ -198,27 +286,36 @@ __device__ __forceinline__ void umma_bf16_acc(uint32_t d_tmem, uint64_t a_desc, 
 // pipe, so this is straight-line code: descriptors advance by adding to their address field
 // (16-byte units; a 32-byte k step is +2), and only the very first instruction of an item
 // carries a run-time accumulate flag.
-template <int NBLK>
+template <int NBLK, bool PAIR = false>
 __device__ __forceinline__ void issue_k_box(uint32_t d0, uint32_t acc_block, uint64_t w_desc,
                                             uint32_t w_blk16, uint64_t x_desc, uint32_t idesc,
                                             uint32_t accum_first)
 {
 #pragma unroll
     for (int m = 0; m < NBLK; ++m)
-        umma_bf16(d0 + m * acc_block, w_desc + (uint64_t)(m * w_blk16), x_desc, idesc, accum_first);
+        umma_bf16<PAIR>(d0 + m * acc_block, w_desc + (uint64_t)(m * w_blk16), x_desc, idesc, accum_first);
 #pragma unroll
     for (int q = 1; q < 4; ++q)
 #pragma unroll
         for (int m = 0; m < NBLK; ++m)
-            umma_bf16_acc(d0 + m * acc_block, w_desc + (uint64_t)(m * w_blk16 + 2 * q),
-                          x_desc + (uint64_t)(2 * q), idesc);
+            umma_bf16_acc<PAIR>(d0 + m * acc_block, w_desc + (uint64_t)(m * w_blk16 + 2 * q),
+                                x_desc + (uint64_t)(2 * q), idesc);
 }
 
-// Arrives on the mbarrier when every MMA issued so far by this thread has completed.
+// Arrives on the mbarrier when every MMA issued so far by this thread has completed; for a pair
+// on the barrier at this offset in both CTAs.
+template <bool PAIR = false>
 __device__ __forceinline__ void umma_commit(uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
+    if (PAIR)
+        asm volatile(
+            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 "
+            "[%0], %1;" ::"r"(bar),
+            "h"((uint16_t)3)
+            : "memory");
+    else
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+                     : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16])
@@ -252,11 +349,11 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr)
            (1ull << 46) | (2ull << 61);
 }
 
-// kind::f16 instruction descriptor: D fp32, A and B bf16, both K-major, M = 128, N = n
-// (a multiple of 16, at most 256).
-__device__ __forceinline__ uint32_t umma_idesc_bf16(int n)
+// kind::f16 instruction descriptor: D fp32, A and B bf16, both K-major, M = m (128, or 256 for a
+// CTA pair), N = n (a multiple of 16, of 32 for a pair, at most 256).
+__device__ __forceinline__ uint32_t umma_idesc_bf16(int n, int m = 128)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
 

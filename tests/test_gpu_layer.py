@@ -209,6 +209,28 @@ def test_row_permutation_equivariance():
     assert torch.equal(out_p, out[p])
 
 
+PAIR_CASES = [
+    ("pair-tile-edges", 288, 5, 2, 352, 1408, 150, 1),   # last tiles of 32 and 96 features, 2 shared segments
+    ("pair-few-rows", 160, 6, 3, 224, 96, 1, 5),         # groups of 1..6 rows: the second CTA's rows are all padding
+    ("pair-segments", 256, 2, 1, 544, 0, 259, 1),        # groups of about 259 rows: two segments, ragged tile ends
+    ("pair-half-box", 544, 4, 4, 96, 32, 33, 0),         # reductions that end in half a k box; 33 rows: 17 per CTA
+]
+
+
+@pytest.mark.parametrize("name,H,E,k,I,Is,B,gamma", PAIR_CASES)
+def test_cta_pair_case(name, H, E, k, I, Is, B, gamma):
+    """One case of the CTA-pair test below (in this process: the host's own choice)."""
+    test_scheduling_mode_case(name, H, E, k, I, Is, B, gamma)
+
+
+@pytest.mark.parametrize("wide", ["0", "1"])
+def test_layer_parity_on_cta_pairs(wide):
+    """The FFN kernels on CTA pairs (MOE_FF_PAIR, a test hook read once per process) in either
+    ring geometry, at the edges of their tiles and of the token halves."""
+    _run_child({"MOE_FF_PAIR": "1", "MOE_FF_WIDE": wide, "MOE_SMALL_FUSED": "0"},
+               "cta_pair_case or scheduling_mode_case or test_layer_parity_small_shapes")
+
+
 @pytest.mark.parametrize("wide", ["0", "1"])
 def test_layer_parity_in_both_ring_geometries(wide):
     """The FFN kernels run with segments of up to 128 token rows (two k boxes per weight slot,
