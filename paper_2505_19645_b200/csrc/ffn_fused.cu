@@ -51,9 +51,9 @@
 // commits release the slots of both.  Layer, single CTAs -> pairs: Qwen2 shape T = 1280
 // 1298 -> 1208 us, Mixtral shape T = 1280 1082 -> 1004.
 //
-// CTA = 11 warps.  warp 0: weight producer (one lane issues TMA), warp 1: MMA issuer (the
-// warp in step, one elected lane issues; idle in a pair's second CTA) and owner of the TMEM
-// allocation, warp 2: token-operand producer, warps 3..10:
+// CTA = 11 warps.  warp 0: weight producer, warp 1: MMA issuer (idle in a pair's second CTA) and
+// owner of the TMEM allocation, warp 2: token-operand producer (in all three the warp runs in
+// step and one elected lane issues), warps 3..10:
 // epilogue, two warps per TMEM lane quarter that take alternate 16-token chunks (tcgen05.ld,
 // SwiGLU, transposition, 16-byte bf16 stores): where no second set of accumulators exists the
 // epilogue is not hidden behind the next tile, and two warps per scheduler hide its latencies.  Rings and the
@@ -77,8 +77,7 @@ namespace moe {
 
 constexpr int FF_EPI_WARPS = 8;
 constexpr int FF_THREADS = 32 * (3 + FF_EPI_WARPS);
-constexpr int FF_MAX_W_SLOTS = 8;
-constexpr int FF_X_ENTRIES = 8;                               // token-ring entries in flight
+constexpr int FF_STEPS = 8;  // k steps in flight: barrier pairs, token-ring entries, weight slots at most
 constexpr int FF_SEG = SEG_TOKENS;        // token rows per segment in the streaming geometry
 constexpr int FF_SEG_WIDE = 2 * SEG_TOKENS;  // ... in the contraction geometry (the MMA's N limit)
 constexpr int FF_TMEM_COLS = 512;
@@ -166,7 +165,7 @@ struct ClaimRing {
     uint32_t peer_data, peer_full0, leader_empty0;
 };
 
-// Walks the items of one CTA: its units of the shared expert first (dealt round-robin: they
+// Walks the items of one CTA, in every lane of the role's warp: its units of the shared expert first (dealt round-robin: they
 // depend on nothing the layer computes), then chunks of the routed groups' work, claimed from
 // a grid-wide counter so that a CTA that is late or slow simply takes less.  The routed part
 // needs the segment plan, which the preceding kernels write: next() calls
@@ -195,9 +194,8 @@ struct ItemWalk {
     static constexpr int USH = PAIR ? 5 : 4;  // log2 of the weight rows of a unit
     const FfnArgs &a;
     const ClaimRing &ring;
-    const bool claimer;    // this thread claims; all others follow the ring
-    const bool lead;       // this thread arrives on the ring's barriers for its role
-    const bool warp_wide;  // the role is run by all 32 lanes in lock step (epilogue warps)
+    const bool claimer;    // this warp's first lane claims; all others follow the ring
+    const bool lead;       // first lane: claims, or arrives on the ring's barriers for its role
     const int max_units;
     const int worker, workers;
     int n_claims;
@@ -219,9 +217,8 @@ struct ItemWalk {
     int t_k0, t_k1;
     long long t_out_off;
 
-    __device__ ItemWalk(const FfnArgs &args, const ClaimRing &r, bool is_claimer, bool is_lead,
-                        bool is_warp_wide, bool already_synced)
-        : a(args), ring(r), claimer(is_claimer), lead(is_lead), warp_wide(is_warp_wide),
+    __device__ ItemWalk(const FfnArgs &args, const ClaimRing &r, bool is_claimer, bool already_synced)
+        : a(args), ring(r), claimer(is_claimer), lead((threadIdx.x & 31) == 0),
           max_units(args.max_tile >> 4),  // a pair's tile is twice as high, as is its unit
           worker(PAIR ? blockIdx.x >> 1 : blockIdx.x), workers(PAIR ? gridDim.x >> 1 : gridDim.x),
           n_claims(0), synced(false), group_loaded(false), have_chunk(false), finished(false),
@@ -335,16 +332,21 @@ struct ItemWalk {
         const uint32_t par = (uint32_t)(n_claims / FF_CLAIMS) & 1u;
         int *e = ring.data + slot * FF_CLAIM_WORDS;
         if (claimer) {
-            for (;;) {
+            bool published = true;
+            while (lead) {
                 // (the counter is only read where the answer can be yes)
                 const long long ample = 4 * (long long)workers * (a.round_robin ? 1 : max_units);
                 const bool plenty =
                     P > ample && P - *reinterpret_cast<volatile int32_t *>(a.claim_counter) > ample;
                 if (end_published || n_pub >= n_claims + (plenty ? 2 : 1))
                     break;
-                if (!publish_one())
-                    return false;
+                if (!publish_one()) {
+                    published = false;
+                    break;
+                }
             }
+            if (!__all_sync(0xffffffffu, published))
+                return false;
         } else if (!mbar_wait<PAIR>(ring.full0 + 8u * slot, par, ring.abort_flag, ring.status)) {
             return false;
         }
@@ -357,8 +359,7 @@ struct ItemWalk {
         grp.n = e[5];
         grp.first_seg = e[6];
         if (!claimer) {
-            if (warp_wide)
-                __syncwarp();  // every lane has read the entry before it is released
+            __syncwarp();  // every lane has read the entry before it is released
             if (lead) {
                 if (PAIR)
                     mbar_arrive_cluster(ring.leader_empty0 + 8u * slot);
@@ -576,7 +577,7 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
     constexpr int NW = GATED ? 2 : 1;  // weight matrices per tile (gate and up: one block each)
 
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bars[2 * FF_MAX_W_SLOTS + 2 * FF_X_ENTRIES + 4 + 2 * FF_CLAIMS];
+    __shared__ uint64_t bars[2 * FF_STEPS + 4 + 2 * FF_CLAIMS];
     __shared__ uint32_t tmem_base_holder;
     __shared__ int abort_flag[2];  // [0] raised by the first wait that gives up, [1] wait limit (us)
     __shared__ __align__(16) int claim_data[FF_CLAIMS * FF_CLAIM_WORDS];
@@ -592,13 +593,15 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
     const uint32_t ring_x = (smem_u32(smem_raw) + 1023u) & ~1023u;  // swizzle needs 1 KB alignment
     const uint32_t ring_w = ring_x + (uint32_t)args.x_units * FF_X_UNIT;
     const uint32_t bar0 = smem_u32(bars);
-    auto w_full = [&](int s) { return bar0 + 8u * s; };
-    auto w_empty = [&](int s) { return bar0 + 8u * (FF_MAX_W_SLOTS + s); };
-    auto x_full = [&](int s) { return bar0 + 8u * (2 * FF_MAX_W_SLOTS + s); };
-    auto x_empty = [&](int s) { return bar0 + 8u * (2 * FF_MAX_W_SLOTS + FF_X_ENTRIES + s); };
-    auto acc_full = [&](int b) { return bar0 + 8u * (2 * FF_MAX_W_SLOTS + 2 * FF_X_ENTRIES + b); };
-    auto acc_empty = [&](int b) { return bar0 + 8u * (2 * FF_MAX_W_SLOTS + 2 * FF_X_ENTRIES + 2 + b); };
-    const uint32_t claim_full0 = bar0 + 8u * (2 * FF_MAX_W_SLOTS + 2 * FF_X_ENTRIES + 4);
+    // One barrier pair per k step in flight (a weight slot and a token entry, consumed together),
+    // step j on pair j % FF_STEPS.  full: both producers' bytes; empty: the step's instructions
+    // have read them.  The weight producer refills slot j % NS once step j - NS is consumed.
+    auto full = [&](int j) { return bar0 + 8u * (j % FF_STEPS); };
+    auto empty = [&](int j) { return bar0 + 8u * (FF_STEPS + j % FF_STEPS); };
+    auto parity = [](int j) { return (uint32_t)(j / FF_STEPS) & 1u; };
+    auto acc_full = [&](int b) { return bar0 + 8u * (2 * FF_STEPS + b); };
+    auto acc_empty = [&](int b) { return bar0 + 8u * (2 * FF_STEPS + 2 + b); };
+    const uint32_t claim_full0 = bar0 + 8u * (2 * FF_STEPS + 4);
     const uint32_t claim_empty0 = claim_full0 + 8u * FF_CLAIMS;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -611,13 +614,9 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
     if (threadIdx.x == 0) {
         abort_flag[0] = 0;
         abort_flag[1] = args.wait_us;
-        for (int s = 0; s < NS; ++s) {
-            mbar_init(w_full(s), 1);
-            mbar_init(w_empty(s), 1);
-        }
-        for (int s = 0; s < FF_X_ENTRIES; ++s) {
-            mbar_init(x_full(s), 1);
-            mbar_init(x_empty(s), 1);
+        for (int j = 0; j < FF_STEPS; ++j) {
+            mbar_init(full(j), 2);
+            mbar_init(empty(j), 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(acc_full(b), 1);
@@ -658,38 +657,46 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
 
     if (warp == 0) {
         // ---------------- weight producer ----------------
-        if (lane == 0) {
-            // gate/up pass: the shared expert's weights and x are the caller's inputs, so those
-            // items run before the wait.  Down pass: every weight tile may be fetched ahead --
-            // the launch order guarantees that the plan is complete when this kernel starts.
-            ItemWalk<PAIR> walk(args, claims, rank == 0, rank != 0, false, !GATED);
-            const uint64_t pol_once = l2_policy_evict_first();
-            bool launched = !GATED;
-            if (!GATED)
-                griddep_launch();
-            int slot = 0;
-            uint32_t phase = 0;
-            bool ok = true;
-            Item it;
-            while (ok && walk.next(it)) {
-                if (!launched && walk.synced) {
-                    griddep_launch();  // after the wait: dependents may rely on the plan
-                    launched = true;
+        // As in the issuer, all lanes in step with uniform values and one elected lane issues the
+        // copies.  With the loop in one lane's branch the issue of a copy cost several hundred
+        // cycles: tiles of 32 rows, whose passes that bounds, took 361 us at T = 77 on the Qwen1.5
+        // shape against 303; with the tiles in use 182 -> 180, T = 32 162 -> 158, the Qwen2 shape
+        // with skewed routing at T = 320 778 -> 760 (one barrier per k step included).
+        //
+        // gate/up pass: the shared expert's weights and x are the caller's inputs, so those
+        // items run before the wait.  Down pass: every weight tile may be fetched ahead --
+        // the launch order guarantees that the plan is complete when this kernel starts.
+        ItemWalk<PAIR> walk(args, claims, rank == 0, !GATED);
+        const uint64_t pol_once = l2_policy_evict_first();
+        bool launched = !GATED;
+        if (!GATED)
+            griddep_launch();
+        int slot = 0, step = 0;
+        bool ok = true;
+        Item it;
+        while (ok && walk.next(it)) {
+            if (!launched && walk.synced) {
+                griddep_launch();  // after the wait: dependents may rely on the plan
+                launched = true;
+            }
+            const int grp = warp_uniform(it.grp), w_once = warp_uniform(it.w_once);
+            const int hc = warp_uniform(it.h) / CTAS;  // this CTA's rows of the tile
+            const uint32_t tile_bytes = (uint32_t)hc * 128u;
+            // expert = 0 for the shared kind
+            const int wrow = warp_uniform(it.expert * args.rows[0] + it.f0) + rank * hc;
+            const int k_begin = warp_uniform(it.k0), k_end = warp_uniform(it.k1);
+            for (int k0 = k_begin; k0 < k_end; k0 += 64 * kb) {
+                const int nbox = min(kb, (k_end - k0 + 63) >> 6);
+                const bool free = step < NS || mbar_wait(empty(step - NS), parity(step - NS), abortp, args.status);
+                if (!__all_sync(0xffffffffu, free)) {
+                    ok = false;
+                    break;
                 }
-                const int K = it.k1;
-                const int hc = it.h / CTAS;  // this CTA's rows of the tile
-                const uint32_t tile_bytes = (uint32_t)hc * 128u;
-                const int wrow = it.expert * args.rows[0] + it.f0 + rank * hc;  // expert = 0 for the shared kind
-                for (int k0 = it.k0; k0 < K; k0 += 64 * kb) {
-                    const int nbox = min(kb, (K - k0 + 63) >> 6);
-                    if (!mbar_wait(w_empty(slot), phase ^ 1u, abortp, args.status)) {
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t base = ring_w + slot * args.w_slot_bytes;
-                    const uint32_t full = leader_bar(w_full(slot));
+                const uint32_t base = ring_w + slot * args.w_slot_bytes;
+                const uint32_t bar = leader_bar(full(step));
+                if (elect_one()) {
                     if (rank == 0)
-                        mbar_expect_tx(w_full(slot), CTAS * nbox * NW * tile_bytes);
+                        mbar_expect_tx(full(step), CTAS * nbox * NW * tile_bytes);
                     for (int b = 0; b < nbox; ++b) {
 #pragma unroll
                         for (int m = 0; m < NW; ++m) {
@@ -699,102 +706,90 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                             while (rem > 0) {
                                 const int hi = rem >= 128 ? 0 : (rem >= 64 ? 1 : (rem >= 32 ? 2 : 3));
                                 const int bh = 128 >> hi;
-                                const CUtensorMap *map = &maps.w[it.grp][m][hi];
-                                if (PAIR && it.w_once)
-                                    tma_load_2d_pair_hint(dst, map, full, k0 + 64 * b, row, pol_once);
+                                const CUtensorMap *map = &maps.w[grp][m][hi];
+                                if (PAIR && w_once)
+                                    tma_load_2d_pair_hint(dst, map, bar, k0 + 64 * b, row, pol_once);
                                 else if (PAIR)
-                                    tma_load_2d_pair(dst, map, full, k0 + 64 * b, row);
-                                else if (it.w_once)
-                                    tma_load_2d_hint(dst, map, full, k0 + 64 * b, row, pol_once);
+                                    tma_load_2d_pair(dst, map, bar, k0 + 64 * b, row);
+                                else if (w_once)
+                                    tma_load_2d_hint(dst, map, bar, k0 + 64 * b, row, pol_once);
                                 else
-                                    tma_load_2d(dst, map, full, k0 + 64 * b, row);
+                                    tma_load_2d(dst, map, bar, k0 + 64 * b, row);
                                 dst += (uint32_t)bh * 128u;
                                 row += bh;
                                 rem -= bh;
                             }
                         }
                     }
-                    if (++slot == NS) {
-                        slot = 0;
-                        phase ^= 1u;
-                    }
                 }
+                __syncwarp();
+                ++step;
+                if (++slot == NS)
+                    slot = 0;
             }
-            if (PAIR)  // the leader's last releases have arrived before this CTA may exit
-                for (int i = 0; ok && i < NS; ++i) {
-                    ok = mbar_wait(w_empty(slot), phase ^ 1u, abortp, args.status);
-                    if (++slot == NS) {
-                        slot = 0;
-                        phase ^= 1u;
-                    }
-                }
-            if (!walk.synced)
-                walk.sync(true);
-            if (!launched)
-                griddep_launch();
         }
+        if (!walk.synced)
+            walk.sync(true);
+        if (!launched)
+            griddep_launch();
     } else if (warp == 2) {
         // ---------------- token-operand producer ----------------
-        if (lane == 0) {
-            // down pass: h is written by the preceding kernel, which may still be running; a
-            // segment's rows are fetched once its progress counter says they are complete
-            ItemWalk<PAIR> walk(args, claims, false, true, false, !GATED);
-            XRingWalk ring(args.x_units);
-            int seen = -1;  // (group kind, segment) key last found complete
-            const uint64_t pol_keep = l2_policy_evict_last();
-            int released = 0;          // entries known to have been consumed
-            int v_cur = 0, v_rel = 0;  // virtual unit positions: issued up to / free up to
-            int v_start_of[FF_X_ENTRIES];  // where each entry's rows begin (after its padding)
-            bool ok = true;
-            Item it;
-            while (ok && walk.next(it)) {
-                const int K = it.k1;
-                if (!GATED) {
-                    const int key = (it.grp << 30) | it.seg;
-                    if (key != seen) {
-                        // every epilogue warp of the gate/up pass counts the 16-column units
-                        // of h it has finished for the segment
-                        ok = counter_wait(args.done[it.grp] + it.seg, (args.K[it.grp] >> 4) * FF_EPI_WARPS, abortp,
-                                          args.status);
-                        seen = key;
-                        if (!ok)
-                            break;
-                        // rows written through the generic proxy, read below by the async proxy
-                        asm volatile("fence.proxy.async.global;" ::: "memory");
-                    }
-                }
-                const int pieces = token_pieces<PAIR>(it.n);  // this CTA's share of the rows
-                const int m = pieces * kb;
-                const int xrow = it.row0 + rank * (pieces << 4);
-                for (int k0 = it.k0; ok && k0 < K; k0 += 64 * kb) {
-                    const int nbox = min(kb, (K - k0 + 63) >> 6);
-                    const int j = ring.count;
-                    int pad;
-                    const int at = ring.place(m, pad);
-                    const int v_start = v_cur + pad, v_end = v_start + m;
-                    // the entry's units (and its barrier pair) must have been released:
-                    // everything before the oldest entry still in use is free, the
-                    // padding in front of it included
-                    while (released < j &&
-                           (j - released >= FF_X_ENTRIES || v_end - v_rel > args.x_units)) {
-                        const int r = released % FF_X_ENTRIES;
-                        if (!mbar_wait(x_empty(r), (uint32_t)(released / FF_X_ENTRIES) & 1u, abortp,
-                                       args.status)) {
-                            ok = false;
-                            break;
-                        }
-                        ++released;
-                        v_rel = released < j ? v_start_of[released % FF_X_ENTRIES] : v_start;
-                    }
+        // down pass: h is written by the preceding kernel, which may still be running; a
+        // segment's rows are fetched once its progress counter says they are complete
+        ItemWalk<PAIR> walk(args, claims, false, !GATED);
+        XRingWalk ring(args.x_units);
+        int seen = -1;  // (group kind, segment) key last found complete
+        const uint64_t pol_keep = l2_policy_evict_last();
+        int released = 0;          // entries known to have been consumed
+        int v_cur = 0, v_rel = 0;  // virtual unit positions: issued up to / free up to
+        int v_start_of[FF_STEPS];  // where each entry's rows begin (after its padding)
+        bool ok = true;
+        Item it;
+        while (ok && walk.next(it)) {
+            const int grp = warp_uniform(it.grp);
+            if (!GATED) {
+                const int key = (it.grp << 30) | it.seg;
+                if (key != seen) {
+                    // every epilogue warp of the gate/up pass counts the 16-column units
+                    // of h it has finished for the segment
+                    const bool done = counter_wait(args.done[it.grp] + it.seg,
+                                                   (args.K[it.grp] >> 4) * FF_EPI_WARPS, abortp, args.status);
+                    seen = key;
+                    ok = __all_sync(0xffffffffu, done);
                     if (!ok)
                         break;
-                    const int e = j % FF_X_ENTRIES;
-                    v_start_of[e] = v_start;
-                    v_cur = v_end;
-                    const uint32_t base = ring_x + (uint32_t)at * FF_X_UNIT;
-                    const uint32_t full = leader_bar(x_full(e));
+                    // rows written through the generic proxy, read below by the async proxy
+                    asm volatile("fence.proxy.async.global;" ::: "memory");
+                }
+            }
+            const int pieces = token_pieces<PAIR>(warp_uniform(it.n));  // this CTA's share of the rows
+            const int m = pieces * kb;
+            const int xrow = warp_uniform(it.row0) + rank * (pieces << 4);
+            const int k_begin = warp_uniform(it.k0), k_end = warp_uniform(it.k1);
+            for (int k0 = k_begin; k0 < k_end; k0 += 64 * kb) {
+                const int nbox = min(kb, (k_end - k0 + 63) >> 6);
+                const int j = ring.count;
+                int pad;
+                const int at = ring.place(m, pad);
+                const int v_start = v_cur + pad, v_end = v_start + m;
+                // the entry's units (and its barrier pair) must have been released:
+                // everything before the oldest entry still in use is free, the
+                // padding in front of it included
+                while (ok && released < j && (j - released >= FF_STEPS || v_end - v_rel > args.x_units)) {
+                    const bool free = mbar_wait(empty(released), parity(released), abortp, args.status);
+                    ok = __all_sync(0xffffffffu, free);
+                    ++released;
+                    v_rel = released < j ? v_start_of[released % FF_STEPS] : v_start;
+                }
+                if (!ok)
+                    break;
+                v_start_of[j % FF_STEPS] = v_start;
+                v_cur = v_end;
+                const uint32_t base = ring_x + (uint32_t)at * FF_X_UNIT;
+                const uint32_t bar = leader_bar(full(j));
+                if (elect_one()) {
                     if (rank == 0)
-                        mbar_expect_tx(x_full(e), (uint32_t)(CTAS * nbox * pieces) * FF_X_UNIT);
+                        mbar_expect_tx(full(j), (uint32_t)(CTAS * nbox * pieces) * FF_X_UNIT);
                     for (int b = 0; b < nbox; ++b) {
                         // the entry's rows as boxes of 128, 64, 32 and 16 rows
                         uint32_t dst = base + (uint32_t)(b * pieces) * FF_X_UNIT;
@@ -803,27 +798,25 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                             const int hi = rem >= 128 ? 0 : (rem >= 64 ? 1 : (rem >= 32 ? 2 : 3));
                             const int bh = 128 >> hi;
                             if (PAIR)
-                                tma_load_2d_pair_hint(dst, &maps.x[it.grp][hi], full, k0 + 64 * b, row,
-                                                      pol_keep);
+                                tma_load_2d_pair_hint(dst, &maps.x[grp][hi], bar, k0 + 64 * b, row, pol_keep);
                             else
-                                tma_load_2d_hint(dst, &maps.x[it.grp][hi], full, k0 + 64 * b, row,
-                                                 pol_keep);
+                                tma_load_2d_hint(dst, &maps.x[grp][hi], bar, k0 + 64 * b, row, pol_keep);
                             dst += (uint32_t)bh * 128u;
                             row += bh;
                             rem -= bh;
                         }
                     }
                 }
+                __syncwarp();
             }
-            if (PAIR)  // as for the weight slots
-                for (; ok && released < ring.count; ++released)
-                    ok = mbar_wait(x_empty(released % FF_X_ENTRIES),
-                                   (uint32_t)(released / FF_X_ENTRIES) & 1u, abortp, args.status);
-            if (!walk.synced)
-                walk.sync(true);
-            if (!GATED)
-                griddep_wait();  // no kernel of the chain completes before its predecessor
         }
+        if (PAIR)  // the leader's last releases have arrived before this CTA may exit
+            for (; ok && released < ring.count; ++released)
+                ok = __all_sync(0xffffffffu, mbar_wait(empty(released), parity(released), abortp, args.status));
+        if (!walk.synced)
+            walk.sync(true);
+        if (!GATED)
+            griddep_wait();  // no kernel of the chain completes before its predecessor
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
         // All lanes walk, wait and compute, and the values of an item that came through shared
@@ -834,10 +827,9 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
         // Layer, before -> after: Qwen1.5 shape T = 5 77.4 -> 71.0 us, T = 640 270 -> 258,
         // Mixtral shape T = 1280 1256 -> 1218, DeepSeek-V3 shape T = 128 3261 -> 3178.
         if (rank == 0) {
-            ItemWalk<PAIR> walk(args, claims, false, lane == 0, true, !GATED);
+            ItemWalk<PAIR> walk(args, claims, false, !GATED);
             XRingWalk ring(args.x_units);
             int sw = 0;
-            uint32_t pw = 0;
             bool ok = true;
             int n_items = 0;
             Item it;
@@ -866,11 +858,8 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                     const int j = ring.count;
                     int pad;
                     const int at = ring.place(pieces * kb, pad);
-                    const int xe = j % FF_X_ENTRIES;
-                    const uint32_t xpar = (uint32_t)(j / FF_X_ENTRIES) & 1u;
                     const uint32_t xbase = ring_x + (uint32_t)at * FF_X_UNIT;
-                    bool ready = mbar_wait(w_full(sw), pw, abortp, args.status) &&
-                                 mbar_wait(x_full(xe), xpar, abortp, args.status);
+                    bool ready = mbar_wait(full(j), parity(j), abortp, args.status);
                     if (box == 0)
                         ready = ready && mbar_wait<PAIR>(acc_empty(set), acc_par, abortp, args.status);
                     if (!__all_sync(0xffffffffu, ready)) {
@@ -890,17 +879,14 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                             x_desc += x_box16;
                             accum = 1u;
                         }
-                        umma_commit<PAIR>(x_empty(xe));
-                        umma_commit<PAIR>(w_empty(sw));  // reusable once these MMAs have read it
+                        umma_commit<PAIR>(empty(j));  // reusable once these MMAs have read them
                         if (box + kb >= n_box)
                             umma_commit<PAIR>(acc_full(set));  // accumulators complete
                     }
                     __syncwarp();
                     accum = 1u;
-                    if (++sw == NS) {
+                    if (++sw == NS)
                         sw = 0;
-                        pw ^= 1u;
-                    }
                 }
             }
             if (!walk.synced)
@@ -912,7 +898,7 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
         // stores need not wait for the preceding kernel (the token producer does, per segment)
         const int quarter = warp & 3;  // TMEM lanes 32*quarter .. +31 belong to this warp
         const int chunk0 = warp >= 7 ? 16 : 0;  // the quarter's second warp takes the odd chunks
-        ItemWalk<PAIR> walk(args, claims, false, lane == 0, true, !GATED);
+        ItemWalk<PAIR> walk(args, claims, false, !GATED);
         int n_items = 0;
         Item it;
         for (;;) {
@@ -1337,8 +1323,8 @@ static void ffn_geometry(const moe_config_t &c, int T, FfnArgs &a)
     a.x_units = x_ring_bytes / FF_X_UNIT;
     const int avail = FF_SMEM_LIMIT - 1024 - 512;  // alignment slack, static shared memory
     int ns = (avail - x_ring_bytes) / a.w_slot_bytes;
-    if (ns > FF_MAX_W_SLOTS)
-        ns = FF_MAX_W_SLOTS;
+    if (ns > FF_STEPS)
+        ns = FF_STEPS;
     a.n_w_slots = ns;
     a.wait_us = (int)(FF_WAIT_NS / 1000ull);
     a.shared_seg = shared_segment_rows(c, T);
