@@ -78,6 +78,7 @@ namespace moe {
 constexpr int FF_EPI_WARPS = 8;
 constexpr int FF_THREADS = 32 * (3 + FF_EPI_WARPS);
 constexpr int FF_STEPS = 8;  // k steps in flight: barrier pairs, token-ring entries, weight slots at most
+static_assert(SEG_TOKENS == 128, "n_segments() divides by shifts");
 constexpr int FF_SEG = SEG_TOKENS;        // token rows per segment in the streaming geometry
 constexpr int FF_SEG_WIDE = 2 * SEG_TOKENS;  // ... in the contraction geometry (the MMA's N limit)
 constexpr int FF_TMEM_COLS = 512;
@@ -93,9 +94,11 @@ struct FfnArgs {
     const int32_t *plan_header;  // [0] = [1] = number of segments
     const Segment *seg;
     const PairEntry *pairs;      // one entry per segment, with its group
+    int max_pairs;               // capacity of the table
     int32_t *claim_counter;      // grid-wide: next unclaimed routed position / item of this pass
     int32_t *done[2];            // per segment of each group kind: 16-column units of h finished
                                  // by the gate/up pass, summed over its four epilogue warps
+    int first_fixed;             // round-robin mode: every worker's first item is fixed
     int round_robin;             // routed work dealt as (pair, tile) items instead of ranges
     int32_t *status;
     int T;             // token rows (the shared expert's group)
@@ -184,7 +187,7 @@ struct ClaimRing {
 // 160 + 160 than as 256 + 64.
 __device__ __forceinline__ int balanced_segment_rows(int n, int nseg)
 {
-    return (((n + nseg - 1) / nseg) + 15) & ~15;
+    return nseg == 1 ? (n + 15) & ~15 : (((n + nseg - 1) / nseg) + 15) & ~15;
 }
 
 // PAIR: the worker is a CTA pair that walks the items together, each CTA computing half of a
@@ -208,6 +211,8 @@ struct ItemWalk {
     int ntiles;
     bool synced, group_loaded, have_chunk, finished, end_published;
     int n_pub;  // claimer: chunks published so far
+    int4 pair_group;  // claimer: the plan entry looked up last
+    int pair_seg;
     // current group and tile
     Segment sg;
     int g_nseg, g_u_end;
@@ -238,6 +243,8 @@ struct ItemWalk {
         if (already_synced)
             sync(false);
     }
+    // segments of a group of n rows (seg_rows is 128 or 256)
+    __device__ int n_segments(int n) const { return (n + a.seg_rows - 1) >> (a.seg_rows == SEG_TOKENS ? 7 : 8); }
     // position p -> (group, row unit rounded down to a tile boundary of the group)
     __device__ void boundary(long long p, int &fs_out, int &u_out) const
     {
@@ -247,7 +254,7 @@ struct ItemWalk {
             return;
         }
         const Segment s = a.seg[(int)(p / R0)];
-        const int ns = (s.n + a.seg_rows - 1) / a.seg_rows;
+        const int ns = n_segments(s.n);
         fs_out = s.first_seg;
         u_out = (int)((p - (long long)s.first_seg * R0) / ns) / max_units * max_units;
     }
@@ -255,19 +262,36 @@ struct ItemWalk {
     {
         if (wait)
             griddep_wait();
-        nseg_total = a.plan_header[0];
-        P = a.round_robin ? (long long)a.plan_header[1] * ntiles * a.routed_ksplit
-                          : (long long)nseg_total * R0;
+        // (the entry of a fixed first item is requested with the header, not after it)
+        const int4 hdr = *reinterpret_cast<const int4 *>(a.plan_header);
+        if (claimer && lead && a.first_fixed)
+            load_pair(min((workers - 1 - worker) / (ntiles * a.routed_ksplit), a.max_pairs - 1));
+        nseg_total = hdr.x;
+        P = a.round_robin ? (long long)hdr.y * ntiles * a.routed_ksplit : (long long)nseg_total * R0;
         synced = true;
     }
+    // The plan's entry of a segment, with its group: one load level between a claim and its tile.
+    __device__ void load_pair(int i)
+    {
+        const int4 *pe = reinterpret_cast<const int4 *>(a.pairs + i);
+        pair_group = pe[0];
+        pair_seg = pe[1].x;
+    }
     // Claims the next chunk from the grid-wide counter (claimer only).  In round-robin mode
+    // of the gate/up pass, whose workers all start together,
     // the first item of every worker is fixed -- item workers - 1 - worker, so that the workers
     // without a shared-expert tile (the high ones) take the first routed items -- and costs no
-    // round trip to the counter; the counter hands out the items from `workers` on.
+    // round trip to the counter; the counter hands out the items from `workers` on.  The workers
+    // of the down pass start as the gate/up pass leaves their SMs, so all its items are handed
+    // out in that order: with few items (8 at T = 16 on the tiny shape) a fixed share went to
+    // the SMs that were busy longest (26.0 -> 20.8 us with the shorter path from the plan to the
+    // first tile; Qwen1.5 shape T = 5 69.0 -> 66.1).
     __device__ void claim(int &lo, int &hi)
     {
         if (a.round_robin) {
-            lo = n_pub == 0 ? workers - 1 - worker : workers + atomicAdd(a.claim_counter, 1);
+            lo = !a.first_fixed  ? atomicAdd(a.claim_counter, 1)
+                 : n_pub == 0 ? workers - 1 - worker
+                              : workers + atomicAdd(a.claim_counter, 1);
             hi = lo + 1;
         } else {
             const long long left = P - *reinterpret_cast<volatile int32_t *>(a.claim_counter);
@@ -289,14 +313,13 @@ struct ItemWalk {
         Segment grp = sg;
         claim(lo, hi);
         if (lo >= 0 && a.round_robin) {
-            // the pair entry carries its group: one load level between the claim and the tile
-            const int4 *pe = reinterpret_cast<const int4 *>(a.pairs + lo / (ntiles * a.routed_ksplit));
-            const int4 g = pe[0];
-            sidx = pe[1].x;
-            grp.expert = g.x;
-            grp.row0 = g.y;
-            grp.n = g.z;
-            grp.first_seg = g.w;
+            if (n_pub > 0 || !a.first_fixed)
+                load_pair(lo / (ntiles * a.routed_ksplit));
+            sidx = pair_seg;
+            grp.expert = pair_group.x;
+            grp.row0 = pair_group.y;
+            grp.n = pair_group.z;
+            grp.first_seg = pair_group.w;
         }
         if (!mbar_wait<PAIR>(ring.empty0 + 8u * slot, par ^ 1u, ring.abort_flag, ring.status))
             return false;
@@ -424,9 +447,10 @@ struct ItemWalk {
                 }
                 if (a.round_robin) {
                     // one (segment, tile, k chunk) item
-                    const int chunk = lo % a.routed_ksplit;
-                    const int tile = (lo / a.routed_ksplit) % ntiles;
-                    g_nseg = (sg.n + a.seg_rows - 1) / a.seg_rows;
+                    const int st = a.routed_ksplit == 1 ? lo : lo / a.routed_ksplit;
+                    const int chunk = lo - st * a.routed_ksplit;
+                    const int tile = st % ntiles;
+                    g_nseg = n_segments(sg.n);
                     t_u0 = tile * max_units;
                     t_h = min(max_units, R0 - t_u0);
                     t_grp = 0;
@@ -455,7 +479,7 @@ struct ItemWalk {
             }
             if (!group_loaded) {
                 sg = a.seg[fs];
-                g_nseg = (sg.n + a.seg_rows - 1) / a.seg_rows;
+                g_nseg = n_segments(sg.n);
                 g_u_end = fs == fs_hi ? u_hi : R0;
                 group_loaded = true;
             }
@@ -1419,6 +1443,8 @@ cudaError_t launch_ffn_gateup(const moe_config_t &c, const moe_weights_t &w, con
     a.plan_header = plan.header;
     a.seg = plan.seg;
     a.pairs = plan.pairs;
+    a.max_pairs = max_segments(c.n_experts, T * c.top_k);
+    a.first_fixed = 1;
     a.claim_counter = plan.header + 2;
     a.done[0] = plan.done_routed;
     a.done[1] = plan.done_shared;
@@ -1535,6 +1561,7 @@ cudaError_t launch_ffn_down(const moe_config_t &c, const moe_weights_t &w, int T
     a.plan_header = plan.header;
     a.seg = plan.seg;
     a.pairs = plan.pairs;
+    a.max_pairs = max_segments(c.n_experts, T * c.top_k);
     a.claim_counter = plan.header + 3;
     a.done[0] = plan.done_routed;
     a.done[1] = plan.done_shared;
