@@ -284,8 +284,8 @@ struct ItemWalk {
     // round trip to the counter; the counter hands out the items from `workers` on.  The workers
     // of the down pass start as the gate/up pass leaves their SMs, so all its items are handed
     // out in that order: with few items (8 at T = 16 on the tiny shape) a fixed share went to
-    // the SMs that were busy longest (26.0 -> 20.8 us with the shorter path from the plan to the
-    // first tile; Qwen1.5 shape T = 5 69.0 -> 66.1).
+    // the SMs that were busy longest (26.0 -> 22.4 us with the shorter path from the plan to the
+    // first tile; Qwen1.5 shape T = 5 69.6 -> 68.5).
     __device__ void claim(int &lo, int &hi)
     {
         if (a.round_robin) {

@@ -249,7 +249,7 @@ route_group_small_kernel(const float *__restrict__ logits, const __nv_bfloat16 *
     __shared__ int tmp[MOE_MAX_EXPERTS];
     __shared__ int flag[MOE_MAX_EXPERTS];
     __shared__ uint16_t wcount[ROUTE_SMALL_ASSIGN / 32][MOE_MAX_EXPERTS];
-    __shared__ int expert_of[ROUTE_SMALL_ASSIGN];  // by assignment t * k + j
+    __shared__ __align__(16) int expert_of[ROUTE_SMALL_ASSIGN];  // by assignment t * k + j
     __shared__ int token_of[ROUTE_SMALL_ASSIGN];   // by sorted row
     __shared__ int total;
     griddep_launch();
@@ -259,6 +259,8 @@ route_group_small_kernel(const float *__restrict__ logits, const __nv_bfloat16 *
         hist[tid] = 0;
     for (int i = tid; i < (ROUTE_SMALL_ASSIGN / 32) * MOE_MAX_EXPERTS / 2; i += PERM_THREADS)
         reinterpret_cast<uint32_t *>(&wcount[0][0])[i] = 0u;
+    if (tid >= A && tid < 32)
+        expert_of[tid] = 0x7fffffff;  // (up to a warp's worth of assignments: none)
     griddep_wait();  // the logits come from the preceding kernel
 
     // top-k: warp w selects for token w
@@ -278,20 +280,23 @@ route_group_small_kernel(const float *__restrict__ logits, const __nv_bfloat16 *
     __syncthreads();
 
     if (A <= 32) {
-        // At most a warp's worth of assignments: one warp sorts them with shuffles and every
-        // thread derives its expert's table entries from the (few) assignments directly --
-        // two barriers in all instead of the scans below.
+        // At most a warp's worth of assignments: one warp sorts them with shuffles and writes
+        // the plan, every thread derives its expert's table entries from the (few) assignments
+        // directly -- two barriers in all instead of the scans below.
         if (warp == 0) {
             const int e = lane < A ? expert_of[lane] : -1;
             const uint32_t peers = __match_any_sync(0xffffffffu, e);
+            const bool first = e >= 0 && lane == __ffs(peers) - 1;  // of its expert
+            const uint32_t firsts = __ballot_sync(0xffffffffu, first);
             const int rank = __popc(peers & ((1u << lane) - 1u));
-            int less = 0;
+            int less = 0, arank = 0;  // assignments, activated experts below this one
 #pragma unroll
             for (int src = 0; src < 32; ++src) {
                 const int other = __shfl_sync(0xffffffffu, e, src);
-                less += (other >= 0 && other < e) ? 1 : 0;
+                const int below = (other >= 0 && other < e) ? 1 : 0;
+                less += below;
+                arank += below & (int)(firsts >> src);
             }
-            flag[lane] = (e >= 0 && lane == __ffs(peers) - 1) ? 1 : 0;  // first of its expert
             if (e >= 0) {
                 const int pos = less + rank;  // stable: ascending assignment id inside an expert
                 token_of[pos] = lane / k;
@@ -300,42 +305,44 @@ route_group_small_kernel(const float *__restrict__ logits, const __nv_bfloat16 *
                     inv_perm[lane] = pos;
                 }
             }
+            if (lane == 0)
+                total = __popc(firsts);
+            if (blockIdx.x == 1 && first) {
+                active[arank] = e;
+                if (plan.header != nullptr) {  // one segment and one pair per activated expert
+                    Segment sg;
+                    sg.expert = e;
+                    sg.row0 = less;
+                    sg.n = __popc(peers);
+                    sg.first_seg = arank;
+                    plan.seg[arank] = sg;
+                    plan.done_routed[arank] = 0;
+                    PairEntry pe;
+                    pe.expert = e;
+                    pe.row0 = less;
+                    pe.n = sg.n;
+                    pe.first_seg = arank;
+                    pe.seg = arank;
+                    pe.pad[0] = pe.pad[1] = pe.pad[2] = 0;
+                    plan.pairs[arank] = pe;
+                }
+            }
         }
         __syncthreads();
         if (blockIdx.x == 1) {
-            int cnt = 0, off = 0, arank = 0, n_act = 0;
-            for (int a = 0; a < A; ++a) {
-                const int ea = expert_of[a];
-                cnt += ea == tid ? 1 : 0;
-                off += ea < tid ? 1 : 0;
-                arank += (flag[a] && ea < tid) ? 1 : 0;  // activated experts below this one
-                n_act += flag[a];
-            }
+            const int n_act = total;
             if (tid < E) {
+                int cnt = 0, off = 0;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int4 v = reinterpret_cast<const int4 *>(expert_of)[q];
+                    cnt += (v.x == tid) + (v.y == tid) + (v.z == tid) + (v.w == tid);
+                    off += (v.x < tid) + (v.y < tid) + (v.z < tid) + (v.w < tid);
+                }
                 counts[tid] = cnt;
                 offsets[tid] = off;
                 if (tid >= n_act)
                     active[tid] = -1;
-                if (cnt > 0) {
-                    active[arank] = tid;
-                    if (plan.header != nullptr) {  // one segment and one pair per activated expert
-                        Segment sg;
-                        sg.expert = tid;
-                        sg.row0 = off;
-                        sg.n = cnt;
-                        sg.first_seg = arank;
-                        plan.seg[arank] = sg;
-                        plan.done_routed[arank] = 0;
-                        PairEntry pe;
-                        pe.expert = tid;
-                        pe.row0 = off;
-                        pe.n = cnt;
-                        pe.first_seg = arank;
-                        pe.seg = arank;
-                        pe.pad[0] = pe.pad[1] = pe.pad[2] = 0;
-                        plan.pairs[arank] = pe;
-                    }
-                }
             }
             if (tid == 0) {
                 offsets[E] = A;
