@@ -41,10 +41,10 @@
 // accumulators of 2 x 256 columns.  The token operand lives in a second ring whose entries are
 // sized by the segment's row count and never wrap.
 //
-// CTA pairs.  In the contraction geometry a cluster of two CTAs works on a tile of twice the
-// features with tcgen05 cta_group::2: each CTA loads its half of the weight rows and half of
-// the token rows, the tensor cores of both read both halves of the tokens, and each CTA's
-// TMEM and epilogue get its half of the features for all tokens.  What bounds this regime is
+// CTA pairs.  In the contraction geometry, and in the streaming one beyond 128 tokens
+// (ffn_pairs), a cluster of two CTAs works on a tile of twice the features with tcgen05
+// cta_group::2: each CTA loads its half of the weight rows and half of the token rows, the
+// tensor cores of both read both halves of the tokens, and each CTA's TMEM and epilogue get its half of the features for all tokens.  What bounds the contraction is
 // bytes: each SM is filled at no more than about 44 bytes per clock, a 256 x 256 tile of a single
 // CTA wants 64 at the full instruction rate and 256 x 160 wants 81; a pair's CTA wants 47 and 66.
 // The leader (even CTA) claims the work for both, its barriers count the bytes of both and its
@@ -1237,16 +1237,21 @@ static double expected_active_experts(int E, int k, int T)
 
 static int ffn_grid() { return sm_count(); }
 
-// Whether the FFN kernels of a call run on CTA pairs: in the contraction geometry.  In the
-// streaming geometry the token rows are a small part of what an SM loads (4 rows per group on the
-// DeepSeek-V3 shape at T = 128: 3172 us on single CTAs, 3248 on pairs; Mixtral shape T = 80 443
-// and 450), and a pair waits for the slower of its two streams.
+// Whether the FFN kernels of a call run on CTA pairs: always in the contraction geometry (see the
+// top of the file), in the streaming one beyond 128 tokens.  There a pair's token entries are half
+// as large, so that three weight slots fit where a single CTA has two (96 KB of token ring for
+// segments of 128 rows).  Layer on single CTAs -> pairs: DeepSeek-V3 shape T = 256 3367 -> 3287 us,
+// T = 1024 3647 -> 3560, T = 2048 4075 -> 3944, T = 3072 4428 -> 4374; Mixtral shape T = 192
+// 488 -> 474, T = 384 537 -> 527; Qwen1.5 shape T = 192 to 640 within 1 %.  Up to 128 tokens the
+// token rows are a small part of what an SM loads, single CTAs have three slots too, and a pair
+// waits for the slower of its two streams (DeepSeek-V3 shape T = 128 3172 on single CTAs, 3248 on
+// pairs; Mixtral shape T = 80 443 and 450).
 static bool ffn_pairs(const moe_config_t &c, int T)
 {
+    if (ffn_segment_rows(c, T) > FF_SEG)
+        return true;
     const int force = pair_override();
-    if (force >= 0)
-        return force == 1;
-    return ffn_segment_rows(c, T) > FF_SEG;
+    return force >= 0 ? force == 1 : T > FF_SEG;
 }
 
 // What pulls work items: a CTA, or a pair of CTAs whose tiles are twice as high.
@@ -1331,9 +1336,11 @@ static int shared_tile_count(const moe_config_t &c, int T, int rows_routed, int 
 
 // Ring geometry.  Streaming: two k boxes per weight slot (64 KB for a full tile: every row is
 // fetched in 256 contiguous bytes, which both HBM and L2 serve markedly faster than 128); the
-// token ring holds two entries of the largest possible segment while no group can exceed 64
-// rows (32 KB, three weight slots), three 128-row entries otherwise (96 KB, two slots).
-// Contraction: one k box per slot and per entry, three 256-row entries (96 KB), four slots.
+// token ring holds two entries of the largest possible segment on CTA pairs and while no group
+// can exceed 64 rows (32 KB, three weight slots), three 128-row entries otherwise (96 KB, two
+// slots).  (One k box per slot, five slots, measured 3-4 % slower on pairs as well.)
+// Contraction: pairs, one k box per slot and per entry, four entries of half a 256-row segment
+// (64 KB), five slots.
 static void ffn_geometry(const moe_config_t &c, int T, FfnArgs &a)
 {
     a.seg_rows = ffn_segment_rows(c, T);
@@ -1342,8 +1349,8 @@ static void ffn_geometry(const moe_config_t &c, int T, FfnArgs &a)
     a.acc_sets = wide ? 1 : 2;
     a.w_slot_bytes = 256 * 128 * a.kboxes;  // a full tile: 256 rows per k box
     // (a CTA of a pair holds half of a segment's rows: entries of at most 16 KB in both geometries)
-    const int x_ring_bytes = ffn_pairs(c, T) ? (wide ? 64 * 1024 : 32 * 1024)
-                             : (!wide && small_token_ring(c, T)) ? 32 * 1024 : 96 * 1024;
+    const int x_ring_bytes = wide ? 64 * 1024
+                             : ffn_pairs(c, T) || small_token_ring(c, T) ? 32 * 1024 : 96 * 1024;
     a.x_units = x_ring_bytes / FF_X_UNIT;
     const int avail = FF_SMEM_LIMIT - 1024 - 512;  // alignment slack, static shared memory
     int ns = (avail - x_ring_bytes) / a.w_slot_bytes;
