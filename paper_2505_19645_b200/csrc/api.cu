@@ -456,6 +456,7 @@ moe_status_t moe_verify_layer(const moe_config_t *cfg, const moe_weights_t *w, c
     // the grouping kernel also writes the FFN segment plan (one launch fewer); for a small
     // batch it selects the experts and gathers the token rows as well (three fewer)
     const bool small = route_group_small_applies(*cfg, T);
+    const bool grouped = !small && group_gather_applies(*cfg, T);
     if (small) {
         MOE_STAGE(MOE_STAGE_PERMUTE,
                   launch_route_group_small(*cfg, logits, xb, T, topk_idx, topk_w, counts, offsets,
@@ -470,14 +471,20 @@ moe_status_t moe_verify_layer(const moe_config_t *cfg, const moe_weights_t *w, c
                                             topk_idx, topk_w, s));
         else
             MOE_STAGE(MOE_STAGE_ROUTE_TOPK, launch_route_topk(*cfg, logits, T, topk_idx, topk_w, s));
-        MOE_STAGE(MOE_STAGE_PERMUTE,
-                  launch_permute(*cfg, topk_idx, T, counts, offsets, perm, inv_perm, active,
-                                 n_active, s, &plan, status));
+        if (grouped)
+            MOE_STAGE(MOE_STAGE_PERMUTE,
+                      launch_group_gather(*cfg, topk_idx, xb, T, counts, offsets, perm, inv_perm, active,
+                                          n_active, status, plan,
+                                          reinterpret_cast<__nv_bfloat16 *>(base + L.x_sorted), s));
+        else
+            MOE_STAGE(MOE_STAGE_PERMUTE,
+                      launch_permute(*cfg, topk_idx, T, counts, offsets, perm, inv_perm, active,
+                                     n_active, s, &plan, status));
     }
     const int shared_parts = has_shared ? shared_down_parts(*cfg) : 1;
     const int routed_parts = routed_down_parts(*cfg, T);
     st = run_ffn(*cfg, *w, xb, T, offsets, perm, y, ys, base, L, s, launches, true, shared_parts,
-                 routed_parts, small);
+                 routed_parts, small || grouped);
     if (st != MOE_OK)
         return st;
     MOE_STAGE(MOE_STAGE_COMBINE,

@@ -230,6 +230,13 @@ cudaError_t launch_route_group_small(const moe_config_t &c, const float *logits,
                                      int32_t *inv_perm, int32_t *active, int32_t *n_active,
                                      int32_t *status, PlanView plan, __nv_bfloat16 *x_sorted,
                                      cudaStream_t s);
+// grouping, tables, plan and row gather of a larger batch in one launch (replaces launch_permute +
+// launch_gather_rows where it applies)
+bool group_gather_applies(const moe_config_t &c, int T);
+cudaError_t launch_group_gather(const moe_config_t &c, const int32_t *idx, const __nv_bfloat16 *x, int T,
+                                int32_t *counts, int32_t *offsets, int32_t *perm, int32_t *inv_perm,
+                                int32_t *active, int32_t *n_active, int32_t *status, PlanView plan,
+                                __nv_bfloat16 *x_sorted, cudaStream_t s);
 // one bounded wait on a word nothing sets (moe_selftest_wait_limit)
 cudaError_t launch_wait_limit_selftest(int32_t *status, int32_t *never_set, int limit_us,
                                        cudaStream_t s);

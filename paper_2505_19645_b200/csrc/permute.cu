@@ -225,6 +225,143 @@ cudaError_t launch_permute(const moe_config_t &c, const int32_t *idx, int T, int
                       counts, offsets, perm, inv_perm, active, n_active, status, pv);
 }
 
+// Grouping and row gather of a larger batch in one launch: permute_kernel's counting sort with
+// smaller chunks, so that as many CTAs as the copy wants share it, each then copying its own
+// tokens' rows to their sorted places (a token's row is read once and written top_k times).  Two
+// launches had a boundary between two short kernels, and the gather read every row top_k times.
+// Bound by latencies (A / 4096 rounds of counting, the scans, one pass over the rows).  CTA b owns `tokens` tokens (at most PERM_THREADS assignments); the last CTA writes the tables.
+__global__ void __launch_bounds__(PERM_THREADS)
+group_gather_kernel(const int32_t *__restrict__ topk_idx, const __nv_bfloat16 *__restrict__ x, int T, int H,
+                    int E, int k, int tokens, int32_t *__restrict__ counts, int32_t *__restrict__ offsets,
+                    int32_t *__restrict__ perm, int32_t *__restrict__ inv_perm,
+                    int32_t *__restrict__ active, int32_t *__restrict__ n_active,
+                    int32_t *__restrict__ status, PlanView plan, __nv_bfloat16 *__restrict__ x_sorted)
+{
+    __shared__ int hist[MOE_MAX_EXPERTS];    // all assignments
+    __shared__ int before[MOE_MAX_EXPERTS];  // assignments of earlier chunks
+    __shared__ int offs[MOE_MAX_EXPERTS];
+    __shared__ int tmp[MOE_MAX_EXPERTS];
+    __shared__ uint8_t wcount[PERM_THREADS / 32][MOE_MAX_EXPERTS];  // per warp of this chunk
+    __shared__ int pos_of[PERM_THREADS];                            // by assignment of this chunk
+    __shared__ int total;
+    griddep_launch();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int A = T * k;
+    const bool tables_cta = blockIdx.x == gridDim.x - 1;
+    const int t0 = tables_cta ? 0 : blockIdx.x * tokens;
+    const int nt = tables_cta ? 0 : min(tokens, T - t0);
+    const int chunk0 = t0 * k, chunk = nt * k;
+    if (tid < MOE_MAX_EXPERTS) {
+        hist[tid] = 0;
+        before[tid] = 0;
+    }
+    for (int i = tid; i < (PERM_THREADS / 32) * MOE_MAX_EXPERTS / 4; i += PERM_THREADS)
+        reinterpret_cast<uint32_t *>(&wcount[0][0])[i] = 0u;
+    griddep_wait();  // the expert indices come from the preceding kernel
+    __syncthreads();
+    const bool few = E <= 32;
+    constexpr int U = 4;  // loads in flight
+    for (int a0 = 0; a0 < A; a0 += U * PERM_THREADS) {
+        int e[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int a = a0 + u * PERM_THREADS + tid;
+            e[u] = a < A ? topk_idx[a] : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int a = a0 + u * PERM_THREADS + tid;
+            if (a0 + u * PERM_THREADS >= A)
+                break;
+            const bool valid = e[u] >= 0 && e[u] < E;
+            warp_histogram_add(hist, e[u], valid, few);
+            if (a0 + u * PERM_THREADS < chunk0)
+                warp_histogram_add(before, e[u], valid && a < chunk0, few);
+        }
+    }
+    // this thread's assignment: rank inside its warp, and its warp's counts
+    const int my_a = chunk0 + tid;
+    const int my_e = tid < chunk ? topk_idx[my_a] : -1;
+    const bool my_valid = my_e >= 0 && my_e < E;
+    const uint32_t peers = __match_any_sync(0xffffffffu, my_valid ? my_e : -1);
+    const int rank_in_warp = __popc(peers & ((1u << lane) - 1u));
+    if (my_valid && lane == __ffs(peers) - 1)
+        wcount[warp][my_e] = (uint8_t)__popc(peers);
+    __syncthreads();
+    if (tid < MOE_MAX_EXPERTS)
+        offs[tid] = tid < E ? hist[tid] : 0;
+    __syncthreads();
+    block_exclusive_scan(offs, tmp, E, &total);
+    if (tables_cta) {  // it counted no earlier chunk: `before` is free (all zero)
+        write_tables(hist, offs, before, tmp, &total, E, counts, offsets, active, n_active, status, plan);
+        return;
+    }
+    int pos = -1;
+    if (my_valid) {
+        pos = offs[my_e] + before[my_e] + rank_in_warp;
+        for (int w = 0; w < warp; ++w)
+            pos += wcount[w][my_e];
+        perm[pos] = my_a;
+        inv_perm[my_a] = pos;
+    }
+    pos_of[tid] = pos;
+    __syncthreads();
+    const int vec_per_row = H >> 3;
+    const int total_vec = nt * vec_per_row;
+    const uint4 *src = reinterpret_cast<const uint4 *>(x) + (size_t)t0 * vec_per_row;
+    uint4 *dst = reinterpret_cast<uint4 *>(x_sorted);
+    constexpr int V = 2;
+    for (int v0 = tid; v0 < total_vec; v0 += V * PERM_THREADS) {
+        uint4 d[V];
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+            if (v0 + u * PERM_THREADS < total_vec)
+                d[u] = src[v0 + u * PERM_THREADS];
+#pragma unroll
+        for (int u = 0; u < V; ++u) {
+            const int v = v0 + u * PERM_THREADS;
+            if (v < total_vec) {
+                const int t = v / vec_per_row, c = v - t * vec_per_row;
+                for (int j = 0; j < k; ++j) {
+                    const int p = pos_of[t * k + j];
+                    if (p >= 0)
+                        dst[(size_t)p * vec_per_row + c] = d[u];
+                }
+            }
+        }
+    }
+}
+
+// Every CTA counts all assignments, so the CTAs' reading grows with their number times A.  Layer,
+// two launches -> one: tiny shape T = 640 36.4 -> 34.3 us, Qwen1.5 shape T = 40 166.3 -> 165.0,
+// T = 192 202 -> 198, T = 640 250 -> 247, Mixtral shape T = 80 445 -> 443, Qwen2 shape T = 64 593 -> 590,
+// DeepSeek-V3 shape T = 512 (4096 assignments) equal; T = 3072 (24576) 4461 -> 4507.
+constexpr int GROUP_GATHER_ASSIGN = 8192;
+
+bool group_gather_applies(const moe_config_t &c, int T) { return T * c.top_k <= GROUP_GATHER_ASSIGN; }
+
+cudaError_t launch_group_gather(const moe_config_t &c, const int32_t *idx, const __nv_bfloat16 *x, int T,
+                                int32_t *counts, int32_t *offsets, int32_t *perm, int32_t *inv_perm,
+                                int32_t *active, int32_t *n_active, int32_t *status, PlanView plan,
+                                __nv_bfloat16 *x_sorted, cudaStream_t s)
+{
+    if (!group_gather_applies(c, T))
+        return cudaErrorInvalidValue;
+    // about 96 KB of rows per CTA, as few assignments as a chunk holds, and one CTA per SM at most
+    // (the FFN kernel's CTAs start on the SMs these leave alone)
+    const size_t bytes = (size_t)T * c.top_k * c.hidden * 2;
+    int want = (int)(bytes / (96 * 1024)) + 1;
+    if (want > sm_count() - 1)
+        want = sm_count() - 1;
+    int tokens = (T + want - 1) / want;
+    if (tokens > PERM_THREADS / c.top_k)
+        tokens = PERM_THREADS / c.top_k;
+    const int blocks = (T + tokens - 1) / tokens + 1;  // + the tables CTA
+    return launch_pdl(group_gather_kernel, dim3(blocks), dim3(PERM_THREADS), 0, s, idx, x, T, c.hidden,
+                      c.n_experts, c.top_k, tokens, counts, offsets, perm, inv_perm, active, n_active, status,
+                      plan, x_sorted);
+}
+
 // Routing of a small batch in one launch: top-k, grouping, segment plan and the gather of
 // the token rows into sorted order, for T <= ROUTE_SMALL_TOKENS tokens and at most
 // ROUTE_SMALL_ASSIGN assignments.  Every CTA repeats the (tiny) top-k and counting sort for
