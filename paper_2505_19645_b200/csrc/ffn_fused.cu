@@ -15,12 +15,12 @@
 // instruction at its full rate.  In TMEM a lane is a weight row (an output feature) and a
 // column a token: an epilogue thread owns one feature and walks the tokens.
 //
-// Work partition.  Output features are independent, so the weight rows of all routed
-// groups are laid end to end (one position = 16 rows of one group for one of its segments)
-// and the CTAs of the persistent grid claim chunks of positions at run time from a grid-wide
-// counter (chunk ends on tile boundaries, sizes shrinking as the work runs out), or, where
-// chunks would be too short or too many, single (segment, tile, k chunk) items: a CTA that
-// starts late or runs slowly takes less, there is no tile-count quantisation and no tail wave.
+// Work partition.  Output features are independent, so the routed work is cut into (segment,
+// tile, k chunk) items which the workers of the persistent grid claim at run time from a
+// grid-wide counter: one that starts late or runs slowly takes less.  (The kernels can also deal
+// ranges: the weight rows of all routed groups laid end to end, one position = 16 rows of one
+// group for one of its segments, chunk ends on tile boundaries, sizes shrinking as the work runs
+// out; see use_round_robin.)
 // The shared expert's rows are cut into (tile, k chunk, segment) units that are dealt
 // round-robin to the CTAs; they depend on nothing the layer computes, so they run before the
 // routing result exists.  Tiles have at most 128 features (gate/up: two blocks, gate and up)
@@ -1361,27 +1361,17 @@ static void ffn_geometry(const moe_config_t &c, int T, FfnArgs &a)
     a.shared_seg = shared_segment_rows(c, T);
 }
 
-// Range mode keeps every CTA alone on "its" groups, perfectly levelled.  It loses when
-//  - a range is shorter than a few tiles: its two ends are partial tiles, and a weight block
-//    costs K/16 tensor-core instructions whatever its height, so short ranges turn issue-bound;
-//  - the token rows of `grid` groups do not fit in L2 beside the weight stream (large T): every
-//    tile would fetch its group's rows from HBM again.
-// Then, and when there are so many tiles per CTA that the last wave hardly matters, the routed
-// work is dealt round-robin as (segment, tile) items: full tiles only, and the CTAs work on a
-// few groups at a time.
-static bool use_round_robin(const moe_config_t &c, int T, int rows_routed, int K_routed, int max_tile)
+// The routed work is dealt as single (segment, tile, k chunk) items.  Ranges of consecutive tiles,
+// the other way the kernels know (a test hook chooses it), keep a worker on "its" groups' token
+// rows, but their ends are uneven and their chunks coarse; since a copy and an instruction cost
+// little to issue, items are the faster way throughout: layer, ranges -> items, Qwen1.5 shape T = 77
+// 180.2 -> 177.6 us, T = 128 189 -> 186, T = 192 199.4 -> 195.1; Qwen2 shape T = 64 589.6 -> 586.9;
+// Mixtral and DeepSeek-V3 shapes equal.  (Items of half the tile height for the last round of every
+// worker: 1-6 % slower.)
+static bool use_round_robin()
 {
     const int force = schedule_override();
-    if (force >= 0)
-        return force == 1;
-    const double n_act = expected_active_experts(c.n_experts, c.top_k, T);
-    const double rows_per_group = (double)T * c.top_k / n_act;
-    const double segs = n_act * ceil(rows_per_group / ffn_segment_rows(c, T));
-    const FfnWorkers wk = ffn_workers(c, T);
-    const int tile = max_tile * wk.ctas;
-    const double tiles_per_cta = segs * ((rows_routed + tile - 1) / tile) / wk.count;
-    const double token_bytes = rows_per_group * K_routed * 2.0 * wk.count;
-    return tiles_per_cta < 3.0 || tiles_per_cta >= 12.0 || token_bytes > 200.0 * 1024 * 1024;
+    return force >= 0 ? force == 1 : true;
 }
 
 template <bool GATED, bool PAIR>
@@ -1455,7 +1445,7 @@ cudaError_t launch_ffn_gateup(const moe_config_t &c, const moe_weights_t &w, con
     a.claim_counter = plan.header + 2;
     a.done[0] = plan.done_routed;
     a.done[1] = plan.done_shared;
-    a.round_robin = use_round_robin(c, T, c.inter, c.hidden, a.max_tile) ? 1 : 0;
+    a.round_robin = use_round_robin() ? 1 : 0;
     a.routed_ksplit = 1;
     a.routed_kchunk = c.hidden;
     a.status = status;
@@ -1485,7 +1475,7 @@ static double routed_down_items(const moe_config_t &c, int T)
 // adds the planes.  (Fewer than three items per CTA also means the pass deals single items.)
 int routed_down_parts(const moe_config_t &c, int T)
 {
-    if (!use_round_robin(c, T, c.hidden, c.inter, 256))
+    if (!use_round_robin())
         return 1;
     int parts = (int)ceil(3.0 * ffn_grid() / routed_down_items(c, T));
     const int cap = c.inter / 1024;  // chunks below half a megabyte cost more than they level
@@ -1572,7 +1562,7 @@ cudaError_t launch_ffn_down(const moe_config_t &c, const moe_weights_t &w, int T
     a.claim_counter = plan.header + 3;
     a.done[0] = plan.done_routed;
     a.done[1] = plan.done_shared;
-    a.round_robin = use_round_robin(c, T, c.hidden, c.inter, a.max_tile) ? 1 : 0;
+    a.round_robin = use_round_robin() ? 1 : 0;
     if (routed_parts > 1 && !a.round_robin)
         return cudaErrorInvalidValue;  // planes exist only where single items are dealt
     a.routed_ksplit = routed_parts;
