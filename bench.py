@@ -21,6 +21,7 @@ import hashlib
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -467,8 +468,8 @@ def record_traffic(csv_path, workload, command):
                                        head.index("Metric Unit"), head.index("Metric Value"))
     scale = {"byte": 1, "Kbyte": 1e3, "Mbyte": 1e6, "Gbyte": 1e9}
     for r in rows[1:]:
-        if "ffn_fused_kernel<1>" not in r[i_name] and "ffn_fused_kernel<true>" not in r[i_name] \
-                and "(bool)1" not in r[i_name]:
+        # first template argument: the gate/up pass
+        if not re.search(r"ffn_fused_kernel<(1|true|\(bool\)1)[,>]", r[i_name]):
             continue
         v = float(r[i_val].replace(",", "")) * scale[r[i_unit]]
         (rd if r[i_metric] == "dram__bytes_read.sum" else wr).append(v)

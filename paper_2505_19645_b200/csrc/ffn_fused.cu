@@ -97,7 +97,7 @@ struct FfnArgs {
     int max_pairs;               // capacity of the table
     int32_t *claim_counter;      // grid-wide: next unclaimed routed position / item of this pass
     int32_t *done[2];            // per segment of each group kind: 16-column units of h finished
-                                 // by the gate/up pass, summed over its four epilogue warps
+                                 // by the gate/up pass, summed over its eight epilogue warps
     int first_fixed;             // round-robin mode: every worker's first item is fixed
     int round_robin;             // routed work dealt as (pair, tile) items instead of ranges
     int32_t *status;
@@ -370,8 +370,11 @@ struct ItemWalk {
             }
             if (!__all_sync(0xffffffffu, published))
                 return false;
-        } else if (!mbar_wait<PAIR>(ring.full0 + 8u * slot, par, ring.abort_flag, ring.status)) {
-            return false;
+        } else {
+            // (the lanes of a warp wait one by one: when a wait gives up, all leave together)
+            const bool got = mbar_wait<PAIR>(ring.full0 + 8u * slot, par, ring.abort_flag, ring.status);
+            if (!__all_sync(0xffffffffu, got))
+                return false;
         }
         ++n_claims;
         lo = e[0];
@@ -1472,7 +1475,7 @@ static double routed_down_items(const moe_config_t &c, int T)
 // (segment, tile) items per CTA -- few tokens, or few experts with long reductions -- some SMs
 // have no weight stream to pull and one SM cannot pull a tile faster than a fraction of what
 // HBM delivers, so the reduction is cut; each chunk writes its own plane of y and the combine
-// adds the planes.  (Fewer than three items per CTA also means the pass deals single items.)
+// adds the planes.
 int routed_down_parts(const moe_config_t &c, int T)
 {
     if (!use_round_robin())

@@ -209,6 +209,20 @@ def test_row_permutation_equivariance():
     assert torch.equal(out_p, out[p])
 
 
+@pytest.mark.parametrize("E,k,T", [
+    (8, 1, 33),      # the smallest: a chunk of one CTA, fewer assignments than a warp pair
+    (24, 16, 512),   # 8192 assignments: the last size that groups and gathers in one launch
+    (24, 16, 513),   # one token more: two launches
+    (512, 8, 300),   # the expert limit
+    (60, 3, 1365),   # chunks that end inside a warp
+])
+def test_grouping_and_gather_of_medium_batches(E, k, T):
+    shape = wl.small_shape("grouped", 160, E, k, 64, 32, 0, 1, 1)
+    w = wl.make_weights(shape, 700 + E, "cuda", zipf_s=1.0 if E > 100 else None)
+    x = wl.make_tokens(shape, T, 800 + T, "cuda")
+    check_layer_against_oracle(shape, w, x, T, 0)
+
+
 PAIR_CASES = [
     ("pair-tile-edges", 288, 5, 2, 352, 1408, 150, 1),   # last tiles of 32 and 96 features, 2 shared segments
     ("pair-few-rows", 160, 6, 3, 224, 96, 1, 5),         # groups of 1..6 rows: the second CTA's rows are all padding

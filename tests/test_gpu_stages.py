@@ -41,6 +41,27 @@ def test_route_topk_bit_exact(E, k, score_fn, renorm):
     assert np.abs(w.cpu().numpy().astype(np.float64) - w_ref).max() <= GATE_W_ATOL * shape.routed_scale
 
 
+@pytest.mark.parametrize("E,k", [(8, 3), (60, 4), (512, 16)])
+def test_route_topk_orders_zeros_and_extremes_like_floats(E, k):
+    """-0 and +0 are equal (ties go to the lower index), and the largest, smallest and denormal
+    finite values keep their float order."""
+    api = _api()
+    rng = np.random.default_rng(E)
+    big, tiny = np.float32(3e38), np.float32(1e-45)
+    pool = np.array([0.0, -0.0, tiny, -tiny, 1.0, -1.0, big, -big], dtype=np.float32)
+    z = rng.choice(pool, size=(64, E)).astype(np.float32)
+    z[0, :] = rng.choice(pool[:2], size=E)
+    z[1, :] = -big
+    shape = wl.small_shape("ex", 64, E, k, 64, 0, 1, 0, 0)
+    idx = torch.empty((64, k), dtype=torch.int32, device="cuda")
+    w = torch.empty((64, k), dtype=torch.float32, device="cuda")
+    api.moe_route_topk(api.make_config(shape), torch.from_numpy(z).cuda(), idx, w)
+    torch.cuda.synchronize()
+    idx_ref, w_ref = oracle.route_topk(z, k, 1, 0, 1.0)
+    np.testing.assert_array_equal(idx.cpu().numpy(), idx_ref)
+    assert np.abs(w.cpu().numpy().astype(np.float64) - w_ref).max() <= GATE_W_ATOL
+
+
 @pytest.mark.parametrize("E,k", [(8, 2), (60, 4), (256, 8)])
 def test_route_topk_stays_in_bounds_on_non_finite_logits(E, k):
     """Logits are finite by contract; NaN / Inf rows may come out in any order, but the
