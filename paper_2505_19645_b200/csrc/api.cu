@@ -203,7 +203,7 @@ moe_status_t run_ffn(const moe_config_t &c, const moe_weights_t &w, const __nv_b
                      const int32_t *offsets, const int32_t *perm, __nv_bfloat16 *y,
                      __nv_bfloat16 *shared_y, char *ws, const Workspace &L, cudaStream_t s,
                      int &launches, bool plan_ready, int shared_parts, int routed_parts,
-                     bool gathered)
+                     bool gathered, bool f32_out)
 {
     const bool with_shared = shared_y != nullptr && c.shared_inter > 0;
     const PlanView plan = plan_view(ws, L, ffn_segment_rows(c, T));
@@ -219,7 +219,7 @@ moe_status_t run_ffn(const moe_config_t &c, const moe_weights_t &w, const __nv_b
               launch_ffn_gateup(c, w, x, xs, T, plan, with_shared, h, hs, status, s));
     MOE_STAGE(MOE_STAGE_DOWN,
               launch_ffn_down(c, w, T, plan, with_shared, h, hs, y, shared_y, shared_parts,
-                              routed_parts, status, s));
+                              routed_parts, f32_out, status, s));
     return MOE_OK;
 }
 
@@ -484,12 +484,12 @@ moe_status_t moe_verify_layer(const moe_config_t *cfg, const moe_weights_t *w, c
     const int shared_parts = has_shared ? shared_down_parts(*cfg) : 1;
     const int routed_parts = routed_down_parts(*cfg, T);
     st = run_ffn(*cfg, *w, xb, T, offsets, perm, y, ys, base, L, s, launches, true, shared_parts,
-                 routed_parts, small || grouped);
+                 routed_parts, small || grouped, f32_outputs(T));
     if (st != MOE_OK)
         return st;
     MOE_STAGE(MOE_STAGE_COMBINE,
               launch_combine(*cfg, y, routed_parts, inv_perm, topk_w, ys, shared_parts, gated ? shared_scale : nullptr, T,
-                             static_cast<__nv_bfloat16 *>(out), s));
+                             static_cast<__nv_bfloat16 *>(out), s, f32_outputs(T)));
     g_last_launches = launches;
 
     return copy_debug_out(*cfg, T, dbg, base, L, s);

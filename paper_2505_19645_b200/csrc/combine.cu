@@ -21,13 +21,47 @@ __device__ __forceinline__ void accumulate8(float (&acc)[8], float w, const uint
     acc[7] = fmaf(w, bf16_hi(v.w), acc[7]);
 }
 
+// Eight consecutive values of a row as they are stored: bf16, or floats for calls of a few tokens.
+template <bool F32>
+struct Row8;
+template <>
+struct Row8<false> {
+    uint4 v;
+    __device__ __forceinline__ void load(const void *base, size_t at)
+    {
+        v = *reinterpret_cast<const uint4 *>(static_cast<const __nv_bfloat16 *>(base) + at);
+    }
+    __device__ __forceinline__ void add(float (&acc)[8], float w) const { accumulate8(acc, w, v); }
+};
+template <>
+struct Row8<true> {
+    float4 lo, hi;
+    __device__ __forceinline__ void load(const void *base, size_t at)
+    {
+        const float4 *p = reinterpret_cast<const float4 *>(static_cast<const float *>(base) + at);
+        lo = p[0];
+        hi = p[1];
+    }
+    __device__ __forceinline__ void add(float (&acc)[8], float w) const
+    {
+        acc[0] = fmaf(w, lo.x, acc[0]);
+        acc[1] = fmaf(w, lo.y, acc[1]);
+        acc[2] = fmaf(w, lo.z, acc[2]);
+        acc[3] = fmaf(w, lo.w, acc[3]);
+        acc[4] = fmaf(w, hi.x, acc[4]);
+        acc[5] = fmaf(w, hi.y, acc[5]);
+        acc[6] = fmaf(w, hi.z, acc[6]);
+        acc[7] = fmaf(w, hi.w, acc[7]);
+    }
+};
+
 // KP: top_k rounded up to 2, 4, 8 or 16 -- the arrays of row pieces in flight are sized by it,
 // so that a top-2 or top-4 layer keeps its registers (and its occupancy).
-template <int KP>
-__global__ void __launch_bounds__(CB_THREADS, KP <= 2 ? 4 : (KP <= 4 ? 3 : (KP <= 8 ? 2 : 1)))
-combine_kernel(const __nv_bfloat16 *__restrict__ y, int routed_parts,
+template <int KP, bool F32>
+__global__ void __launch_bounds__(CB_THREADS, F32 ? 1 : (KP <= 2 ? 4 : (KP <= 4 ? 3 : (KP <= 8 ? 2 : 1))))
+combine_kernel(const void *__restrict__ y, int routed_parts,
                const int32_t *__restrict__ inv_perm, const float *__restrict__ topk_w,
-               const __nv_bfloat16 *__restrict__ shared_y, int shared_parts,
+               const void *__restrict__ shared_y, int shared_parts,
                const float *__restrict__ shared_scale, int T, int H, int k,
                __nv_bfloat16 *__restrict__ out)
 {
@@ -51,42 +85,40 @@ combine_kernel(const __nv_bfloat16 *__restrict__ y, int routed_parts,
         }
         const float s = shared_y && shared_scale ? shared_scale[t] : 1.0f;
         // the shared expert's planes, four at a time, requested before the routed rows are used
-        uint4 sv[4];
+        Row8<F32> sv[4];
         const int sp0 = shared_y ? (shared_parts < 4 ? shared_parts : 4) : 0;
 #pragma unroll
         for (int p = 0; p < 4; ++p)
             if (p < sp0)
-                sv[p] = *reinterpret_cast<const uint4 *>(shared_y + ((size_t)p * T + t) * H + h);
+                sv[p].load(shared_y, ((size_t)p * T + t) * H + h);
         float acc[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q)
             acc[q] = 0.f;
         for (int part = 0; part < routed_parts; ++part) {
-            const __nv_bfloat16 *yp = y + (size_t)part * plane;
-            uint4 v[KP];
+            Row8<F32> v[KP];
 #pragma unroll
             for (int j = 0; j < KP; ++j)
                 if (j < k)
-                    v[j] = *reinterpret_cast<const uint4 *>(yp + (size_t)rows[j] * H + h);
+                    v[j].load(y, (size_t)part * plane + (size_t)rows[j] * H + h);
 #pragma unroll
             for (int j = 0; j < KP; ++j)
                 if (j < k)
-                    accumulate8(acc, wts[j], v[j]);
+                    v[j].add(acc, wts[j]);
         }
 #pragma unroll
         for (int p = 0; p < 4; ++p)
             if (p < sp0)
-                accumulate8(acc, s, sv[p]);
+                sv[p].add(acc, s);
         if (shared_y && shared_parts > 4) {
 #pragma unroll
             for (int p = 0; p < 4; ++p)
                 if (4 + p < shared_parts)
-                    sv[p] = *reinterpret_cast<const uint4 *>(
-                        shared_y + ((size_t)(4 + p) * T + t) * H + h);
+                    sv[p].load(shared_y, ((size_t)(4 + p) * T + t) * H + h);
 #pragma unroll
             for (int p = 0; p < 4; ++p)
                 if (4 + p < shared_parts)
-                    accumulate8(acc, s, sv[p]);
+                    sv[p].add(acc, s);
         }
         uint4 o;
         __nv_bfloat162 p;
@@ -105,7 +137,7 @@ combine_kernel(const __nv_bfloat16 *__restrict__ y, int routed_parts,
 cudaError_t launch_combine(const moe_config_t &c, const __nv_bfloat16 *y, int routed_parts,
                            const int32_t *inv_perm, const float *topk_w,
                            const __nv_bfloat16 *shared_y, int shared_parts,
-                           const float *shared_scale, int T, __nv_bfloat16 *out, cudaStream_t s)
+                           const float *shared_scale, int T, __nv_bfloat16 *out, cudaStream_t s, bool f32)
 {
     if (shared_parts > MOE_MAX_SHARED_PARTS)
         return cudaErrorInvalidValue;
@@ -115,9 +147,12 @@ cudaError_t launch_combine(const moe_config_t &c, const __nv_bfloat16 *y, int ro
     if (blocks > cap)
         blocks = cap;
 #define MOE_CB_LAUNCH(KP)                                                                        \
-    return launch_pdl(combine_kernel<KP>, dim3((unsigned)blocks), dim3(CB_THREADS), 0, s, y,     \
-                      routed_parts, inv_perm, topk_w, shared_y, shared_parts, shared_scale, T,   \
-                      c.hidden, c.top_k, out)
+    return f32 ? launch_pdl(combine_kernel<KP, true>, dim3((unsigned)blocks), dim3(CB_THREADS), 0, s, y, \
+                            routed_parts, inv_perm, topk_w, shared_y, shared_parts, shared_scale, T, \
+                            c.hidden, c.top_k, out)                                                  \
+               : launch_pdl(combine_kernel<KP, false>, dim3((unsigned)blocks), dim3(CB_THREADS), 0, s, y, \
+                            routed_parts, inv_perm, topk_w, shared_y, shared_parts, shared_scale, T, \
+                            c.hidden, c.top_k, out)
     if (c.top_k <= 2)
         MOE_CB_LAUNCH(2);
     if (c.top_k <= 4)

@@ -140,6 +140,12 @@ bool layer_small_applies(const moe_config_t &c, int T);
 size_t layer_small_logit_part_bytes(const moe_config_t &c);
 size_t layer_small_h_bytes(const moe_config_t &c, int T);
 
+// Calls of a few tokens keep the expert outputs in fp32 between the down projection and the
+// combine step (y and y_shared then hold floats): a few rows, whose rounding the one-launch layer
+// does not have either.
+constexpr int F32_OUTPUT_TOKENS = 4;
+inline bool f32_outputs(int T) { return T <= F32_OUTPUT_TOKENS; }
+
 inline Workspace workspace_layout(const moe_config_t &c, int T)
 {
     Workspace w{};
@@ -166,9 +172,15 @@ inline Workspace workspace_layout(const moe_config_t &c, int T)
     w.h_shared = cut.take((size_t)T * c.shared_inter * 2);
     // y: [A,H], or while the down pass is short of work items partial planes of it
     const size_t A_split = ROUTED_SPLIT_MAX_PARTS * routed_split_max_rows(c, T);
-    const size_t y_rows = A > A_split ? A : A_split;
+    size_t y_rows = A > A_split ? A : A_split;
+    // floats while there are a few tokens (also inside a workspace made for more)
+    const size_t few = T < F32_OUTPUT_TOKENS ? T : F32_OUTPUT_TOKENS;
+    const size_t few_split = ROUTED_SPLIT_MAX_PARTS * routed_split_max_rows(c, (int)few);
+    const size_t few_rows = 2 * (few * c.top_k > few_split ? few * c.top_k : few_split);
+    y_rows = y_rows > few_rows ? y_rows : few_rows;
     w.y = cut.take(y_rows * H * 2);
-    w.y_shared = cut.take((size_t)T * H * 2 * shared_down_parts(c));
+    const size_t ys_rows = (size_t)T > 2 * few ? (size_t)T : 2 * few;
+    w.y_shared = cut.take(ys_rows * H * 2 * shared_down_parts(c));
     w.rl_planes = cut.take(router_tc_plane_bytes(c, T));
     w.rl_partial = cut.take(router_tc_partial_bytes(c, T));
     w.small_logit_part = cut.take(layer_small_logit_part_bytes(c));
@@ -219,7 +231,7 @@ cudaError_t launch_ffn_gateup(const moe_config_t &c, const moe_weights_t &w, con
 cudaError_t launch_ffn_down(const moe_config_t &c, const moe_weights_t &w, int T, PlanView plan,
                             bool with_shared, const __nv_bfloat16 *h, const __nv_bfloat16 *h_shared,
                             __nv_bfloat16 *y, __nv_bfloat16 *y_shared, int shared_parts,
-                            int routed_parts,
+                            int routed_parts, bool f32_out,
                             int32_t *status, cudaStream_t s);
 // top-k, grouping, plan and gather of a small batch in one launch (replaces
 // launch_route_topk + launch_permute + launch_gather_rows where it applies)
@@ -247,11 +259,12 @@ cudaError_t launch_tagged_wait_selftest(int32_t *status, int limit_us, cudaStrea
 cudaError_t launch_gather_rows(const moe_config_t &c, const __nv_bfloat16 *x, const int32_t *perm,
                                int T, __nv_bfloat16 *x_sorted, cudaStream_t s);
 // y and shared_y may hold `routed_parts` / `shared_parts` partial planes ([A,H] / [T,H]: k
-// chunks of the down pass), summed here
+// chunks of the down pass), summed here; f32: they hold floats
 cudaError_t launch_combine(const moe_config_t &c, const __nv_bfloat16 *y, int routed_parts,
                            const int32_t *inv_perm, const float *topk_w,
                            const __nv_bfloat16 *shared_y, int shared_parts,
-                           const float *shared_scale, int T, __nv_bfloat16 *out, cudaStream_t s);
+                           const float *shared_scale, int T, __nv_bfloat16 *out, cudaStream_t s,
+                           bool f32 = false);
 
 // Router logits, top-k, grouping, expert FFNs, shared expert and combine of at most four tokens
 // in one cooperative launch; uses the regions status, logits .. inv_perm, small_logit_part and
@@ -289,7 +302,7 @@ moe_status_t run_ffn(const moe_config_t &c, const moe_weights_t &w, const __nv_b
                      const int32_t *offsets, const int32_t *perm, __nv_bfloat16 *y,
                      __nv_bfloat16 *shared_y, char *ws, const Workspace &L, cudaStream_t s,
                      int &launches, bool plan_ready = false, int shared_parts = 1,
-                     int routed_parts = 1, bool gathered = false);
+                     int routed_parts = 1, bool gathered = false, bool f32_out = false);
 
 // ---------------------------------------------------------------------------------------
 // Device helpers.

@@ -91,6 +91,7 @@ struct FfnArgs {
     int K[2];      // reduction length per group kind
     __nv_bfloat16 *out[2];
     int out_ld[2];
+    int f32_out;   // down pass: out[] are float planes (same element offsets), see f32_outputs
     const int32_t *plan_header;  // [0] = [1] = number of segments
     const Segment *seg;
     const PairEntry *pairs;      // one entry per segment, with its group
@@ -979,6 +980,19 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                                 if (GATED)
                                     tmem_ld16(t0 + acc_block + cc + 32, u[half ^ 1]);
                             }
+                            if (!GATED && args.f32_out) {
+                                // a lane's values as they are: 128 contiguous bytes per token
+                                float *of = reinterpret_cast<float *>(args.out[it.grp]) + it.out_off +
+                                            (size_t)(it.row0 + cc) * ld + it.f0 + rank * hc + 128 * m +
+                                            quarter * 32 + lane;
+                                if (quarter * 32 + lane < rows_blk) {
+#pragma unroll
+                                    for (int i = 0; i < 16; ++i)
+                                        if (cc + i < it.n)
+                                            of[(size_t)i * ld] = __uint_as_float(g[half][i]);
+                                }
+                                continue;
+                            }
                             uint32_t w[16];
 #pragma unroll
                             for (int i = 0; i < 16; ++i) {
@@ -1524,7 +1538,7 @@ int shared_down_parts(const moe_config_t &c)
 cudaError_t launch_ffn_down(const moe_config_t &c, const moe_weights_t &w, int T, PlanView plan,
                             bool with_shared, const __nv_bfloat16 *h, const __nv_bfloat16 *h_shared,
                             __nv_bfloat16 *y, __nv_bfloat16 *y_shared, int shared_parts,
-                            int routed_parts, int32_t *status, cudaStream_t s)
+                            int routed_parts, bool f32_out, int32_t *status, cudaStream_t s)
 {
     const uint64_t A = (uint64_t)T * c.top_k, H = c.hidden, E = c.n_experts;
     FfnArgs a{};
@@ -1562,6 +1576,7 @@ cudaError_t launch_ffn_down(const moe_config_t &c, const moe_weights_t &w, int T
     a.seg = plan.seg;
     a.pairs = plan.pairs;
     a.max_pairs = max_segments(c.n_experts, T * c.top_k);
+    a.f32_out = f32_out ? 1 : 0;
     a.claim_counter = plan.header + 3;
     a.done[0] = plan.done_routed;
     a.done[1] = plan.done_shared;
