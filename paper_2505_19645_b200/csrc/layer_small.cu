@@ -44,8 +44,7 @@ constexpr int LS_ROUTE_WARPS = 4;     // warps of every CTA that wait for the lo
 constexpr int LS_DOWN_CHUNK_MAX = 4096;  // most columns of a down-projection work item ...
 constexpr int LS_DOWN_CHUNK_MIN = 2048;  // ... and the least the host goes down to for more items
 constexpr int LS_DOWN_ITEMS_WANTED = 48; // down-projection items per CTA (three per warp) it aims at
-constexpr size_t LS_SHARED_MAX_ONE = 40u << 20;  // I_s * H up to which the kernel is used for one token
-constexpr size_t LS_WORK_MAX_FEW = 48u << 20;    // T * H * (top_k * I + I_s) up to which for two to four
+constexpr size_t LS_SHARED_WORK_MAX = 80u << 20;  // T * I_s * H up to which the kernel is used for T > 1
 constexpr int LS_DOWN_ROWS = 4;       // output features per down-projection work item
 constexpr int LS_SLOT_FLOATS = LS_DOWN_ROWS * LS_MAX_TOKENS;  // partial sums of one such item
 constexpr size_t LS_MAX_SLOT_BYTES = 160u << 10;
@@ -852,16 +851,17 @@ static bool small_shape(const moe_config_t &c, int T)
 {
     if (T > LS_MAX_TOKENS || T * c.top_k > LS_MAX_ASSIGN || slot_bytes(c, T) > LS_MAX_SLOT_BYTES)
         return false;
-    // Against the kernel chain (tensor cores, deeper streams, five launches), us per call, one launch /
-    // chain.  One token: Qwen1.5 shape 36.9 / 38.4, Mixtral 120 / 123, DeepSeek-V3 135.8 / 134.9, tiny
-    // 14.8 / 21.0, but Qwen2 146.5 / 138.2, whose shared expert (I_s * H = 73 M) alone keeps the
-    // twelve warps beside the routing ones busy.  Two tokens: tiny (0.5 M multiplications) 18.3 / 20.4,
-    // Qwen1.5 (46 M) 48.8 / 49.3, Mixtral (235 M) 197 / 190, DeepSeek-V3 237.7 / 225; three: Qwen1.5
-    // (69 M) 62.3 / 55.1; four: Qwen1.5 74.6 / 64.1, Mixtral 343 / 324, DeepSeek-V3 437 / 400: every
-    // token row adds its products on the CUDA cores.
-    if (T == 1)
-        return (size_t)c.shared_inter * c.hidden <= LS_SHARED_MAX_ONE;
-    return (size_t)T * c.hidden * ((size_t)c.top_k * c.inter + c.shared_inter) <= LS_WORK_MAX_FEW;
+    // This kernel's sums are fp32 fused multiply-adds, and more exact than the tensor cores' of the
+    // kernel chain: against 64 bits the layer is off by 2.3320e-3 here and 2.3326e-3 there
+    // (DeepSeek-V3 shape, T = 4; Qwen1.5 T = 3 2.3476e-3 and 2.3498e-3, Mixtral T = 2 2.3411e-3 and
+    // 2.3421e-3), and 3-4 % of the outputs are not the rounding of the exact sum over the rounded
+    // SwiGLU intermediate, against 7-11 %.  So it also keeps calls that the chain would serve
+    // sooner: us per call, one launch / chain, two tokens Qwen1.5 50.7 / 48.8, Mixtral 191 / 185,
+    // DeepSeek-V3 247 / 232; four tokens 75.6 / 62.8, 312 / 291, 450 / 412, tiny 23.3 / 21.3; one token
+    // 37.1 / 39.2, 118 / 124, 134 / 136, tiny 15 / 21.7.  It ends where the shared expert, whose every
+    // weight is multiplied with all T rows, alone outlasts the weight stream: the Qwen2 shape
+    // (I_s * H = 73 M; one token 144 / 138 us, with a cold L2 154 / 156) is left to the chain from two.
+    return T == 1 || (size_t)T * c.shared_inter * c.hidden <= LS_SHARED_WORK_MAX;
 }
 
 // the largest T' <= T the one-launch kernel takes (0: none)

@@ -137,6 +137,59 @@ def test_few_tokens_take_one_launch():
     assert api.moe_last_launch_count() > 1
 
 
+def _share_not_the_rounding_of_the_exact_sum(shape, w, x, idx, out):
+    """Share of the outputs that are not the bf16 rounding of the layer in 64 bits over the
+    SwiGLU intermediate rounded to bf16 (plain torch)."""
+    d = torch.float64
+    X = x.to(d)
+    z = X @ w["w_router"].to(d).T
+    score = torch.sigmoid(z) if shape.score_fn == wl.SCORE_SIGMOID else torch.softmax(z, 1)
+    gate = score.gather(1, idx)
+    if shape.renormalize:
+        gate = gate / gate.sum(1, keepdim=True)
+
+    def ffn(v, g, u, down):
+        a = g.to(d) @ v
+        return down.to(d) @ (a / (1 + torch.exp(-a)) * (u.to(d) @ v)).float().bfloat16().to(d)
+
+    ref = torch.zeros(x.shape, dtype=d, device=x.device)
+    for t in range(x.shape[0]):
+        for j in range(shape.top_k):
+            e = int(idx[t, j])
+            ref[t] += gate[t, j] * shape.routed_scale * ffn(X[t], w["w_gate"][e], w["w_up"][e], w["w_down"][e])
+        if shape.shared_inter:
+            s = torch.sigmoid(w["w_shared_gate"].to(d) @ X[t]) if shape.shared_gate else 1.0
+            ref[t] += s * ffn(X[t], w["ws_gate"], w["ws_up"], w["ws_down"])
+    return float((ref.float().bfloat16() != out).double().mean())
+
+
+# A sum with relative error eps moves a SwiGLU value across a rounding boundary with probability
+# about 2^8 eps, and that value is then off by 2^-8 of itself; the output, a sum over thousands of
+# them, is off by about sqrt(2^8 eps) 2^-8 of itself, and its own rounding turns over with
+# probability about sqrt(2^8 eps): the share follows the square root of the sums' error.  Measured
+# over 12 seeds and T = 1 to 4 of these shapes: fp32 fused multiply-adds 2.6-4.3 %, tensor-core
+# sums 7.1-11.3 %; the bound is the geometric mean of 4.3 and 7.1.
+FP32_SUMS_SHARE = 0.055
+
+
+@pytest.mark.parametrize("name,T", [("qwen1.5-moe-a2.7b", 3), ("mixtral-8x7b", 2), ("mixtral-8x7b", 4),
+                                    ("deepseek-v3", 4)])
+def test_few_tokens_keep_fp32_sums(name, T):
+    """Two to four tokens of the shapes without a very large shared expert: one launch, whose
+    projections are fp32 sums, not the tensor cores' accumulation."""
+    from paper_2505_19645_b200 import api
+
+    shape = wl.CONFIGS[name]
+    w = wl.make_weights(shape, 7, "cuda")
+    x = wl.make_tokens(shape, T, 500, "cuda")
+    out, dbg = run_gpu_layer(shape, w, x, T, 0)
+    launches = api.moe_last_launch_count()
+    idx = torch.from_numpy(dbg["topk_idx"]).cuda().long().view(T, shape.top_k)
+    share = _share_not_the_rounding_of_the_exact_sum(shape, w, x, idx, out)
+    assert share <= FP32_SUMS_SHARE, share
+    assert launches == 1
+
+
 def test_one_workspace_serves_calls_of_every_size_in_turn():
     """The one-launch kernel's barrier word and counters live in the workspace and are never
     cleared: each call tags them with its own epoch.  Calls of one to five tokens (the last on
