@@ -6,19 +6,12 @@
 
 #include "device_once.h"
 #include "moe_verify.h"
+#include "plan.h"
 
 namespace moe {
 
-// ---------------------------------------------------------------------------------------
-// Segment plan.  The token rows of an activated expert (a "group") are cut into segments of
-// at most SEG_TOKENS (or, for calls whose groups run to hundreds of rows, 2 * SEG_TOKENS)
-// consecutive sorted rows, the N extent of one tensor-core instruction.
-// The plan lists one entry per segment; every entry carries its whole group, so that any
-// segment index leads to the group, its first segment and its number of segments.  The plan
-// is derived from the grouping offsets on the device: the host never needs the
-// data-dependent counts and no launch waits for a copy.
-// ---------------------------------------------------------------------------------------
-constexpr int SEG_TOKENS = 128;
+// plan header (ints): [0] number of segments over all activated experts, [1] the same,
+//                     [2], [3] routed work claimed so far by the gate/up and the down pass
 constexpr int PLAN_HEADER_INTS = 16;
 
 // Status region (first of the workspace): word [0] is the device status word, raised by a
@@ -26,23 +19,6 @@ constexpr int PLAN_HEADER_INTS = 16;
 // it; word [1] holds STATUS_MAGIC once the region has been initialised (a fresh workspace holds
 // garbage: the first kernel of every call clears word [0] unless the magic is already there).
 constexpr int32_t STATUS_MAGIC = 0x4d6f4553;
-
-struct Segment {
-    int32_t expert;     // routed expert id of the group
-    int32_t row0;       // first sorted row of the group
-    int32_t n;          // rows of the group (all its segments together)
-    int32_t first_seg;  // plan index of the group's first segment
-};
-
-// plan header (ints): [0] number of segments over all activated experts, [1] the same,
-//                     [2], [3] routed work claimed so far by the gate/up and the down pass
-// A segment with its group: everything a CTA needs to start on a (segment, tile) item in one
-// 32-byte load.
-struct __align__(16) PairEntry {
-    int32_t expert, row0, n, first_seg;  // the group (as in Segment)
-    int32_t seg;                         // plan index of the segment
-    int32_t pad[3];
-};
 
 struct PlanView {
     int seg_rows;         // token rows per segment: SEG_TOKENS or twice that (set by the host)

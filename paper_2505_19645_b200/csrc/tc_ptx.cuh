@@ -105,6 +105,9 @@ __device__ __forceinline__ bool elect_one()
     return p != 0;
 }
 
+// A word that other CTAs advance, as it is at the moment.
+__device__ __forceinline__ int peek(const int32_t *p) { return *reinterpret_cast<const volatile int32_t *>(p); }
+
 // A value that is the same in all lanes of a converged warp, in a form the compiler knows to be.
 __device__ __forceinline__ int warp_uniform(int v) { return __reduce_max_sync(0xffffffffu, v); }
 
