@@ -295,6 +295,9 @@ struct ItemWalk {
             }
             if (!__all_sync(0xffffffffu, published))
                 return false;
+            // the first lane wrote the entry and no barrier stands between it and the others here
+            // (a vote orders no memory); also: all lanes have read an entry before it is reused
+            __syncwarp();
         } else {
             // (the lanes of a warp wait one by one: when a wait gives up, all leave together)
             const bool got = mbar_wait<PAIR>(ring.full0 + 8u * slot, par, ring.abort_flag, ring.status);
