@@ -3,15 +3,19 @@
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
                     [--config NAME] [--B B] [--gamma G] [--zipf S] [--sweeps all|config|none]
+                    [--record FILE]
 
-Prints ONE JSON line.  Headline workload (value, roofline, e2e, cpu_baseline): the
+Prints ONE JSON line, short enough (LINE_MAX) to survive in a log that keeps a run's last few
+thousand characters.  Headline workload (value, roofline, e2e, cpu_baseline): the
 DeepSeek-V3-shaped layer -- the largest of the five benchmark shapes that fits one GPU -- at
-B=32 sequences x (gamma=3)+1 tokens.  With no --config the same line carries, under "sweeps",
+B=32 sequences x (gamma=3)+1 tokens.  With no --config the same run sweeps
 the (B, gamma) grids of all five shapes, the Zipf(1.2) variant of the Qwen2-57B-A14B shape, the
 Zipf(1.0) variant of the DeepSeek-V3 shape and the extra token counts 2048 and 4096 on those two
 shapes: per point the layer time, tokens/s, roofline fraction, the cost ratio T(B,gamma)/T(B,0)
 and the activation statistics of Sec. 3.2 / 3.3 (activated experts against Eq. N(t), tokens per
-activated expert against Eq. T_exp, whether T is beyond the threshold of Eq. T_thres).
+activated expert against Eq. T_exp, whether T is beyond the threshold of Eq. T_thres).  The
+full record, the line's keys with every sweep row under "sweeps", is one JSON line on standard
+error, or in --record FILE; the line itself counts the rows.
 Inputs are seeded and synthetic.  N > 1 runs N independent replicas (weak scaling).
 """
 from __future__ import annotations
@@ -35,6 +39,7 @@ sys.path.insert(0, ROOT)
 
 from paper_2505_19645_b200 import replicas, workloads as wl  # noqa: E402
 
+LINE_MAX = 2900               # characters of the printed line, at most
 L2_FLUSH_BYTES = 512 << 20
 NOMINAL_HBM_GBS = 7700.0      # HBM3e, HGX B200 data sheet
 NOMINAL_BF16_TFLOPS = 2250.0  # dense bf16, data sheet
@@ -52,7 +57,8 @@ EXTRA_POINTS = {"qwen2-57b-a14b": [(512, 3), (1024, 3)], "deepseek-v3": [(512, 3
 # DRAM bytes of one gate/up launch as counted by ncu, with the hash of the kernel source they
 # were taken on (written by --record-traffic from an ncu CSV; see the file for the command)
 TRAFFIC_RECORD = os.path.join(ROOT, "profiles", "gate_up_dram_traffic.txt")
-KERNEL_SOURCES = ["paper_2505_19645_b200/csrc/ffn_fused.cu", "paper_2505_19645_b200/csrc/common.cuh"]
+KERNEL_SOURCES = ["paper_2505_19645_b200/csrc/" + f
+                  for f in ("ffn_fused.cu", "ffn_walk.cuh", "plan.h", "tc_ptx.cuh", "common.cuh")]
 
 
 def load_peaks():
@@ -486,6 +492,30 @@ def record_traffic(csv_path, workload, command):
     print("wrote", TRAFFIC_RECORD)
 
 
+def rounded(v):
+    """Floats to seven significant digits, through dicts and lists."""
+    if isinstance(v, float):
+        return float("%.7g" % v)
+    if isinstance(v, dict):
+        return {k: rounded(x) for k, x in v.items()}
+    if isinstance(v, list):
+        return [rounded(x) for x in v]
+    return v
+
+
+def result_line(record):
+    """The printed line of a full record: the sweeps as [points, points at or above 0.70 of the
+    roofline] per sweep, no explanatory texts."""
+    line = rounded(record)
+    line["sweeps"] = {key: [len(sw["rows"]), sum(r["roof_frac"] >= 0.70 for r in sw["rows"])]
+                      for key, sw in record["sweeps"].items()}
+    line["small_batch"].pop("host_us_per_call_how", None)
+    for key in ("small_batch", "sweeps", "layer_roofline"):  # what a longer line would lose first
+        if len(json.dumps(line)) > LINE_MAX:
+            line[key] = None
+    return json.dumps(line)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -511,6 +541,8 @@ def main():
                     help="only the headline loop and the kernel's event pair (for profiler runs): "
                          "no end-to-end, small-batch, sweep or CPU legs")
     ap.add_argument("--sweep-steps", type=int, default=30, help="samples per sweep point")
+    ap.add_argument("--record", default=None, metavar="FILE",
+                    help="write the full record there instead of to standard error")
     ap.add_argument("--record-traffic", default=None, metavar="NCU_CSV",
                     help="write the DRAM-traffic record of the gate/up kernel from an ncu CSV log")
     ap.add_argument("--ncu-command", default="(not given)")
@@ -699,7 +731,7 @@ def main():
                          % (n, T, reps, dt)}
 
     if rank == 0:
-        line = {
+        record = {
             "metric": "moe_verify_layer_tokens_per_s", "value": value, "unit": "tokens/s",
             "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_step,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "bf16",
@@ -711,7 +743,12 @@ def main():
             "gpu_launches": launches_per_step * args.steps, "clocks": clocks,
             "layer_us": ms_step * 1e3, "small_batch": small, "sweeps": sweeps,
         }
-        print(json.dumps(line))
+        if args.record:
+            with open(args.record, "w") as f:
+                f.write(json.dumps(record) + "\n")
+        else:
+            print(json.dumps(record), file=sys.stderr)
+        print(result_line(record))
     replicas.shutdown()
     return 0
 

@@ -15,7 +15,7 @@ a single FFN layer and are left out.
 
 The optimiser is a projected Levenberg-Marquardt iteration written out here (forward
 difference Jacobian, damping adapted per step, iterates clipped to the box), started from
-several points; it uses numpy only.  Measurements are the "sweep" rows that bench.py prints.
+several points; it uses numpy only.  Measurements are the "sweeps" rows of bench.py records.
 
     python -m paper_2505_19645_b200.model_fit RESULT.json [RESULT.json ...]
 """
@@ -151,14 +151,14 @@ def mse(params, data, ridge: float) -> float:
 
 
 def load_sweeps(paths):
-    """Rows (t, K, E, us) of the sweeps in bench.py result files, sorted as the paper sorts
+    """Rows (t, K, E, us) of the sweeps in bench.py records, sorted as the paper sorts
     its measurements: by K, then gamma, then batch size."""
     rows = []
     shape = None
     for p in paths:
         line = open(p).read().strip().splitlines()[-1]
         d = json.loads(line)
-        # every sweep of the line (bench.py --config X --sweeps config carries one)
+        # every sweep of the record (bench.py --config X --sweeps config carries one)
         for sw in d["sweeps"].values():
             shape = sw["shape"]
             K, E = shape["top_k"], shape["n_experts"]

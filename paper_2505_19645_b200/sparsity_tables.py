@@ -1,10 +1,10 @@
 """Tables of the sparsity sweep (Sec. 4.3) and of the analytical-model fit (Sec. 3.4) from
-bench.py result lines.
+bench.py records.
 
     python -m paper_2505_19645_b200.sparsity_tables OUT.md RESULT.json [RESULT.json ...]
 
-Each RESULT.json holds the line of one run
-    python bench.py --config qwen2-57b-a14b --top-k K --grid sparsity --no-cpu-baseline
+Each RESULT.json is the record of one run
+    python bench.py --config qwen2-57b-a14b --top-k K --grid sparsity --no-cpu-baseline --record RESULT.json
 (or --dense-contrast instead of --top-k).  Writes OUT.md: target efficiency T(B,0)/T(B,gamma)
 per variant and batch size, roofline fractions, and the fit of
 time(t) = bias + k1 G(t) + k2 N(t) + k3 G(T_exp(t)) to the K variants' layer times with the
@@ -40,7 +40,7 @@ def main(argv):
     peaks = variants[0][3]["layer_roofline"]["peaks"]
     out = ["# Sparsity sweep and dense contrast on the Qwen2-57B-A14B shape; fit of the analytical model",
            "",
-           "Generated by `python -m paper_2505_19645_b200.sparsity_tables` from the lines printed by",
+           "Generated by `python -m paper_2505_19645_b200.sparsity_tables` from the records of",
            "`python bench.py --config qwen2-57b-a14b --top-k K --grid sparsity --no-cpu-baseline` for",
            "K = %s and `--dense-contrast` (B200, %s peaks %.1f GB/s / %.1f TFLOP/s; cold L2, CUDA events,"
            % (", ".join(str(v[0]["top_k"]) for v in variants if v[0]["n_experts"] > 1),

@@ -1,8 +1,8 @@
-"""Turns the "sweeps" of a bench.py result line into one table per shape / variant.
+"""Turns the "sweeps" of a bench.py record into one table per shape / variant.
 
     python -m paper_2505_19645_b200.sweep_tables RESULT.json [OUT_DIR]
 
-RESULT.json holds the JSON line bench.py printed (its last line is read).  Writes
+RESULT.json is the file `bench.py --record` wrote (its last line is read).  Writes
 OUT_DIR/sweep_<key>.md (default OUT_DIR: profiles/ beside the package) with, per (B, gamma)
 point, the layer time, tokens/s, the roofline fraction, the verify-cost ratio
 T(B,gamma)/T(B,0) of Sec. 3.1 and the activation statistics of Sec. 3.2 / 3.3.
@@ -21,7 +21,7 @@ def table(key: str, sw: dict, meta: dict) -> str:
     out = ["# Sweep of the %s layer%s" % (key, "" if not sw.get("zipf") else
                                            " (Zipf-like expert popularity, s = %g)" % sw["zipf"]),
            "",
-           "Generated by `python -m paper_2505_19645_b200.sweep_tables` from the line printed by",
+           "Generated by `python -m paper_2505_19645_b200.sweep_tables` from the record of",
            "`%s` (B200, %s peaks: %.1f GB/s, %.1f TFLOP/s bf16; clocks during the run: median %s MHz,"
            % (meta["command"], meta["peak_source"], meta["hbm_gbs"], meta["bf16_tflops"],
               meta["clocks"].get("sm_mhz")),
