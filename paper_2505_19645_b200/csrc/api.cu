@@ -53,15 +53,6 @@ bool pdl_enabled()
     return on;
 }
 
-int schedule_override()
-{
-    static const int v = [] {
-        const char *e = getenv("MOE_FF_RR");
-        return !e ? -1 : (e[0] == '1' ? 1 : (e[0] == '0' ? 0 : -1));
-    }();
-    return v;
-}
-
 int geometry_override()
 {
     static const int v = [] {
@@ -194,7 +185,6 @@ PlanView plan_view(char *ws, const Workspace &L, int seg_rows)
 {
     return PlanView{seg_rows, reinterpret_cast<int32_t *>(ws + L.plan_header),
                     reinterpret_cast<Segment *>(ws + L.plan_seg),
-                    reinterpret_cast<PairEntry *>(ws + L.plan_pairs),
                     reinterpret_cast<int32_t *>(ws + L.plan_done),
                     reinterpret_cast<int32_t *>(ws + L.plan_done) + L.plan_done_shared_at};
 }

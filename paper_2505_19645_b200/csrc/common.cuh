@@ -10,9 +10,12 @@
 
 namespace moe {
 
-// plan header (ints): [0] number of segments over all activated experts, [1] the same,
-//                     [2], [3] routed work claimed so far by the gate/up and the down pass
+// plan header (ints): [0] number of segments over all activated experts,
+//                     [2], [3] routed items claimed so far by the gate/up and the down pass
 constexpr int PLAN_HEADER_INTS = 16;
+// Kept free per segment in front of the plan's entries: the stated limit of the static-scratch
+// entry point, and the workspace sizes callers have taken, count these bytes.
+constexpr int PLAN_RESERVED_BYTES = 16;
 
 // Status region (first of the workspace): word [0] is the device status word, raised by a
 // bounded wait that gave up and left alone by everything else until moe_check reads and clears
@@ -24,7 +27,6 @@ struct PlanView {
     int seg_rows;         // token rows per segment: SEG_TOKENS or twice that (set by the host)
     int32_t *header;      // written by the plan; [2], [3] advanced by the FFN kernels
     Segment *seg;         // capacity max_segments()
-    PairEntry *pairs;     // one entry per segment (with its group), capacity max_segments()
     // Progress of the gate/up pass, read by the down pass: 16-row units of h written so far
     // (counted once per epilogue warp) for every routed segment [max_segments()] and for
     // every 128-row segment of the shared expert [max_shared_segments()].
@@ -57,7 +59,6 @@ struct Workspace {
     size_t inv_perm;      // i32 [A]
     size_t plan_header;   // i32 [PLAN_HEADER_INTS]
     size_t plan_seg;      // Segment[max_segments]
-    size_t plan_pairs;    // PairEntry [max_segments]
     size_t plan_done;     // i32 [max_segments + max_shared_segments]
     size_t plan_done_shared_at;  // index of the shared expert's counters inside plan_done
     size_t x_sorted;      // bf16 [A, H]      token rows in sorted order
@@ -139,8 +140,8 @@ inline Workspace workspace_layout(const moe_config_t &c, int T)
     w.perm = cut.take(A * 4);
     w.inv_perm = cut.take(A * 4);
     w.plan_header = cut.take(PLAN_HEADER_INTS * 4);
+    cut.take(PLAN_RESERVED_BYTES * (size_t)max_segments((int)E, (int)A));
     w.plan_seg = cut.take(sizeof(Segment) * (size_t)max_segments((int)E, (int)A));
-    w.plan_pairs = cut.take(sizeof(PairEntry) * (size_t)max_segments((int)E, (int)A));
     w.plan_done = cut.take(4 * ((size_t)max_segments((int)E, (int)A) + max_shared_segments(T)));
     w.plan_done_shared_at = (size_t)max_segments((int)E, (int)A);
     w.x_sorted = cut.take(A * H * 2);
@@ -251,10 +252,8 @@ cudaError_t launch_layer_small(const moe_config_t &c, const moe_weights_t &w, co
 
 int sm_count();
 bool pdl_enabled();  // programmatic dependent launch between the layer's kernels
-// Test hook, read once per process from MOE_FF_RR: 0 / 1 forces the FFN kernels to deal the
-// routed work as ranges / as single items, -1 (unset) leaves the choice to the host heuristic.
-int schedule_override();
-// The same for the ring geometry, from MOE_FF_WIDE: 0 / 1 forces segments of 128 / 256 rows.
+// Test hook, read once per process from MOE_FF_WIDE: 0 / 1 forces the ring geometry with segments
+// of 128 / 256 rows, -1 (unset) leaves the choice to the host's rule.
 int geometry_override();
 // From MOE_SMALL_FUSED: 0 keeps calls of a few tokens on the chain of kernels every other call
 // uses, -1 (unset) lets them take the one-launch kernel.

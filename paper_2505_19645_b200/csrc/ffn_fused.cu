@@ -17,10 +17,7 @@
 //
 // Work partition.  Output features are independent, so the routed work is cut into (segment,
 // tile, k chunk) items which the workers of the persistent grid claim at run time from a
-// grid-wide counter: one that starts late or runs slowly takes less.  (The kernels can also deal
-// ranges: the weight rows of all routed groups laid end to end, one position = 16 rows of one
-// group for one of its segments, chunk ends on tile boundaries, sizes shrinking as the work runs
-// out; see use_round_robin.)
+// grid-wide counter: one that starts late or runs slowly takes less.
 // The shared expert's rows are cut into (tile, k chunk, segment) units that are dealt
 // round-robin to the CTAs; they depend on nothing the layer computes, so they run before the
 // routing result exists.  Tiles have at most 128 features (gate/up: two blocks, gate and up)
@@ -919,19 +916,6 @@ static void ffn_geometry(const moe_config_t &c, int T, FfnArgs &a)
     a.shared_seg = shared_segment_rows(c, T);
 }
 
-// The routed work is dealt as single (segment, tile, k chunk) items.  Ranges of consecutive tiles,
-// the other way the kernels know (a test hook chooses it), keep a worker on "its" groups' token
-// rows, but their ends are uneven and their chunks coarse; since a copy and an instruction cost
-// little to issue, items are the faster way throughout: layer, ranges -> items, Qwen1.5 shape T = 77
-// 180.2 -> 177.6 us, T = 128 189 -> 186, T = 192 199.4 -> 195.1; Qwen2 shape T = 64 589.6 -> 586.9;
-// Mixtral and DeepSeek-V3 shapes equal.  (Items of half the tile height for the last round of every
-// worker: 1-6 % slower.)
-static bool use_round_robin()
-{
-    const int force = schedule_override();
-    return force >= 0 ? force == 1 : true;
-}
-
 template <bool GATED, bool PAIR>
 static cudaError_t launch_ffn(FfnArgs &a, const FfnMaps &maps, cudaStream_t s)
 {
@@ -997,13 +981,11 @@ cudaError_t launch_ffn_gateup(const moe_config_t &c, const moe_weights_t &w, con
     a.out_ld[1] = c.shared_inter;
     a.plan_header = plan.header;
     a.seg = plan.seg;
-    a.pairs = plan.pairs;
-    a.max_pairs = max_segments(c.n_experts, T * c.top_k);
+    a.max_seg = max_segments(c.n_experts, T * c.top_k);
     a.first_fixed = 1;
     a.claim_counter = plan.header + 2;
     a.done[0] = plan.done_routed;
     a.done[1] = plan.done_shared;
-    a.round_robin = use_round_robin() ? 1 : 0;
     a.routed_ksplit = 1;
     a.routed_kchunk = c.hidden;
     a.status = status;
@@ -1033,8 +1015,6 @@ static double routed_down_items(const moe_config_t &c, int T)
 // adds the planes.
 int routed_down_parts(const moe_config_t &c, int T)
 {
-    if (!use_round_robin())
-        return 1;
     int parts = (int)ceil(3.0 * ffn_grid() / routed_down_items(c, T));
     const int cap = c.inter / 1024;  // chunks below half a megabyte cost more than they level
     if (parts > cap)
@@ -1115,15 +1095,11 @@ cudaError_t launch_ffn_down(const moe_config_t &c, const moe_weights_t &w, int T
     a.out_ld[0] = a.out_ld[1] = c.hidden;
     a.plan_header = plan.header;
     a.seg = plan.seg;
-    a.pairs = plan.pairs;
-    a.max_pairs = max_segments(c.n_experts, T * c.top_k);
+    a.max_seg = max_segments(c.n_experts, T * c.top_k);
     a.f32_out = f32_out ? 1 : 0;
     a.claim_counter = plan.header + 3;
     a.done[0] = plan.done_routed;
     a.done[1] = plan.done_shared;
-    a.round_robin = use_round_robin() ? 1 : 0;
-    if (routed_parts > 1 && !a.round_robin)
-        return cudaErrorInvalidValue;  // planes exist only where single items are dealt
     a.routed_ksplit = routed_parts;
     a.routed_kchunk = split_chunk(c.inter, routed_parts);
     if ((long long)(routed_parts - 1) * a.routed_kchunk >= c.inter ||

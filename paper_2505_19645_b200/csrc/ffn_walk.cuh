@@ -24,15 +24,13 @@ struct FfnArgs {
     __nv_bfloat16 *out[2];
     int out_ld[2];
     int f32_out;   // down pass: out[] are float planes (same element offsets), see f32_outputs
-    const int32_t *plan_header;  // [0] = [1] = number of segments
-    const Segment *seg;
-    const PairEntry *pairs;      // one entry per segment, with its group
-    int max_pairs;               // capacity of the table
-    int32_t *claim_counter;      // grid-wide: next unclaimed routed position / item of this pass
+    const int32_t *plan_header;  // [0] = number of segments
+    const Segment *seg;          // one entry per segment, with its group
+    int max_seg;                 // capacity of the table
+    int32_t *claim_counter;      // grid-wide: routed items of this pass claimed so far
     int32_t *done[2];            // per segment of each group kind: 16-column units of h finished
                                  // by the gate/up pass, summed over its eight epilogue warps
-    int first_fixed;             // round-robin mode: every worker's first item is fixed
-    int round_robin;             // routed work dealt as (pair, tile) items instead of ranges
+    int first_fixed;             // every worker's first routed item is fixed
     int32_t *status;
     int T;             // token rows (the shared expert's group)
     int with_shared;   // shared expert present in this launch
@@ -41,7 +39,7 @@ struct FfnArgs {
                          // to out[1] + s * shared_part_stride
     int shared_kchunk;   // multiple of 128
     long long shared_part_stride;  // elements
-    int routed_ksplit;   // the same for the routed groups (round-robin mode of the down pass only)
+    int routed_ksplit;   // the same for the routed groups
     int routed_kchunk;
     long long routed_part_stride;
     int shared_tiles;  // tiles of the shared expert's rows; (tile, k chunk, segment) units are dealt
@@ -74,15 +72,17 @@ struct Item {
     long long out_off;  // element offset of this item's output plane (k chunk) in out[grp]
 };
 
-// Hand-over of the routed work a CTA claims at run time.  One thread of the CTA (the weight
-// producer) claims chunks from a grid-wide counter and publishes them in a small ring; the
-// other roles read the same sequence, so all roles walk identical items.
+// Hand-over of the routed work a worker claims at run time.  One thread (of the weight producer)
+// claims items from a grid-wide counter and publishes them in a small ring; the other roles read
+// the same sequence, so all roles walk identical items.
 constexpr int FF_CLAIMS = 4;      // ring entries
 // token producer, MMA issuer, epilogue warps; in the second CTA of a pair the weight producer
 // reads as well and nothing is issued
 constexpr int FF_CLAIM_READERS = 2 + FF_EPI_WARPS;
 
-constexpr int FF_CLAIM_WORDS = 8;  // lo, hi, and (round-robin mode) the item's group, decoded
+// An entry: the item's number (-1: none left), the plan index of its segment, and the segment's
+// group (expert, row0, n, first_seg), so that the other roles need not look it up.
+constexpr int FF_CLAIM_WORDS = 8;
 struct ClaimRing {
     int *data;                 // shared memory [FF_CLAIMS][FF_CLAIM_WORDS]
     uint32_t full0, empty0;    // shared addresses of the barrier arrays [FF_CLAIMS]
@@ -93,18 +93,19 @@ struct ClaimRing {
     uint32_t peer_data, peer_full0, leader_empty0;
 };
 
-// Walks the items of one CTA, in every lane of the role's warp: its units of the shared expert first (dealt round-robin: they
-// depend on nothing the layer computes), then chunks of the routed groups' work, claimed from
-// a grid-wide counter so that a CTA that is late or slow simply takes less.  The routed part
-// needs the segment plan, which the preceding kernels write: next() calls
+// Walks the items of one worker, in every lane of the role's warp: its units of the shared expert
+// first (dealt round-robin: they depend on nothing the layer computes), then the routed items it
+// claims from a grid-wide counter, so that a worker that is late or slow simply takes less.  The
+// routed part needs the segment plan, which the preceding kernels write: next() calls
 // griddepcontrol.wait once before it touches the plan (or before reporting the end).
 //
-// Routed work, range mode: positions (16 rows of one group for one of its segments, groups
-// laid end to end); a chunk is a run of positions whose ends are moved to tile boundaries, its
-// length shrinks as the work runs out (a third of the remaining per-CTA share, at least one
-// tile).  Round-robin mode: a chunk is one (segment, tile, k chunk) item; consecutive items are
-// the tiles of one segment, which then run on many CTAs at once and share the segment's token
-// rows in L2.
+// A routed item is one (segment, tile, k chunk); consecutive items are the tiles of one segment,
+// which then run on many SMs at once and share the segment's token rows in L2.  Ranges of
+// consecutive tiles per worker instead, each "its" groups' rows, have uneven ends and coarse chunks:
+// layer, ranges -> items, Qwen1.5 shape T = 77 180.2 -> 177.6 us, T = 128 189 -> 186, T = 192
+// 199.4 -> 195.1, Qwen2 shape T = 64 589.6 -> 586.9, Mixtral and DeepSeek-V3 shapes equal.  (Items of
+// half the tile height for the last round of every worker: 1-6 % slower.)
+
 // Rows per segment of a group of n rows cut into nseg segments: equal shares rounded up to the
 // 16-row unit of the token boxes (never more than the segment limit, since nseg = ceil(n /
 // limit)).  Equal shares instead of "full segments and a remainder": the instruction time
@@ -126,63 +127,34 @@ struct ItemWalk {
     const bool lead;       // first lane: claims, or arrives on the ring's barriers for its role
     const int max_units;
     const int worker, workers;
-    int n_claims;
-    // shared expert: units (tile, k chunk, segment) sj, sj + grid, ...
-    int sj, Us, s_base, s_rem, nseg_s, s_units;
-    // routed groups: current chunk from (fs, u) to (fs_hi, u_hi); fs = plan index of a
-    // group's first segment
-    int R0, nseg_total, fs, u, fs_hi, u_hi;
-    long long P;
-    int ntiles;
-    bool synced, group_loaded, have_chunk, finished, end_published;
-    int n_pub;  // claimer: chunks published so far
-    int4 pair_group;  // claimer: the plan entry looked up last
-    int pair_seg;
-    // current group and tile
-    Segment sg;
-    int g_nseg, g_u_end;
-    bool have_tile;
-    int t_grp, t_expert, t_u0, t_h, t_row0, t_n, t_s, t_s_end, t_seg0, t_seg_rows;
-    bool t_once;  // the tile's weights are read by this pass over it only
-    int t_k0, t_k1;
-    long long t_out_off;
+    int n_claims;  // items taken from the ring so far
+    int n_pub;     // claimer: items published so far
+    // shared expert: units (tile, k chunk, segment) sj, sj + workers, ...
+    int sj, s_base, s_rem, nseg_s, s_units;
+    // routed groups
+    int R0, ntiles, n_items;  // row units of a group, tiles of a group, items of the pass
+    bool synced, finished, end_published;
+    Segment entry;  // claimer: the plan entry looked up last
 
     __device__ ItemWalk(const FfnArgs &args, const ClaimRing &r, bool is_claimer, bool already_synced)
         : a(args), ring(r), claimer(is_claimer), lead((threadIdx.x & 31) == 0),
           max_units(args.max_tile >> 4),  // a pair's tile is twice as high, as is its unit
           worker(PAIR ? blockIdx.x >> 1 : blockIdx.x), workers(PAIR ? gridDim.x >> 1 : gridDim.x),
-          n_claims(0), synced(false), group_loaded(false), have_chunk(false), finished(false),
-          end_published(false), n_pub(0),
-          have_tile(false)
+          n_claims(0), n_pub(0), n_items(0), synced(false), finished(false), end_published(false)
     {
-        Us = a.with_shared ? a.rows[1] >> USH : 0;
+        const int Us = a.with_shared ? a.rows[1] >> USH : 0;
         s_base = a.shared_tiles ? Us / a.shared_tiles : 0;
         s_rem = a.shared_tiles ? Us % a.shared_tiles : 0;
         sj = worker;
         nseg_s = (a.T + a.shared_seg - 1) / a.shared_seg;
         s_units = a.shared_tiles * a.shared_ksplit * nseg_s;
         R0 = a.rows[0] >> USH;
-        nseg_total = fs = u = fs_hi = u_hi = 0;
         ntiles = (R0 + max_units - 1) / max_units;
-        P = 0;
         if (already_synced)
             sync(false);
     }
     // segments of a group of n rows (seg_rows is 128 or 256)
     __device__ int n_segments(int n) const { return (n + a.seg_rows - 1) >> (a.seg_rows == SEG_TOKENS ? 7 : 8); }
-    // position p -> (group, row unit rounded down to a tile boundary of the group)
-    __device__ void boundary(long long p, int &fs_out, int &u_out) const
-    {
-        if (p >= P) {
-            fs_out = nseg_total;
-            u_out = 0;
-            return;
-        }
-        const Segment s = a.seg[(int)(p / R0)];
-        const int ns = n_segments(s.n);
-        fs_out = s.first_seg;
-        u_out = (int)((p - (long long)s.first_seg * R0) / ns) / max_units * max_units;
-    }
     __device__ void sync(bool wait)
     {
         if (wait)
@@ -190,91 +162,71 @@ struct ItemWalk {
         // (the entry of a fixed first item is requested with the header, not after it)
         const int4 hdr = *reinterpret_cast<const int4 *>(a.plan_header);
         if (claimer && lead && a.first_fixed)
-            load_pair(min((workers - 1 - worker) / (ntiles * a.routed_ksplit), a.max_pairs - 1));
-        nseg_total = hdr.x;
-        P = a.round_robin ? (long long)hdr.y * ntiles * a.routed_ksplit : (long long)nseg_total * R0;
+            load_entry(min((workers - 1 - worker) / (ntiles * a.routed_ksplit), a.max_seg - 1));
+        n_items = hdr.x * ntiles * a.routed_ksplit;
         synced = true;
     }
     // The plan's entry of a segment, with its group: one load level between a claim and its tile.
-    __device__ void load_pair(int i)
+    __device__ void load_entry(int i)
     {
-        const int4 *pe = reinterpret_cast<const int4 *>(a.pairs + i);
-        pair_group = pe[0];
-        pair_seg = pe[1].x;
+        const int4 *p = reinterpret_cast<const int4 *>(a.seg + i);
+        const int4 group = p[0];
+        entry.seg = p[1].x;
+        entry.expert = group.x;
+        entry.row0 = group.y;
+        entry.n = group.z;
+        entry.first_seg = group.w;
     }
-    // Claims the next chunk from the grid-wide counter (claimer only).  In round-robin mode
-    // of the gate/up pass, whose workers all start together,
-    // the first item of every worker is fixed -- item workers - 1 - worker, so that the workers
-    // without a shared-expert tile (the high ones) take the first routed items -- and costs no
-    // round trip to the counter; the counter hands out the items from `workers` on.  The workers
+    // Claims the next item (claimer only; -1: none left).  In the gate/up pass, whose workers all
+    // start together, the first item of every worker is fixed -- item workers - 1 - worker, so
+    // that the workers without a shared-expert tile (the high ones) take the first routed items --
+    // and costs no round trip to the counter, which hands out the items from `workers` on.  The workers
     // of the down pass start as the gate/up pass leaves their SMs, so all its items are handed
     // out in that order: with few items (8 at T = 16 on the tiny shape) a fixed share went to
     // the SMs that were busy longest (26.0 -> 22.4 us with the shorter path from the plan to the
     // first tile; Qwen1.5 shape T = 5 69.6 -> 68.5).
-    __device__ void claim(int &lo, int &hi)
+    __device__ int claim()
     {
-        if (a.round_robin) {
-            lo = !a.first_fixed  ? atomicAdd(a.claim_counter, 1)
-                 : n_pub == 0 ? workers - 1 - worker
-                              : workers + atomicAdd(a.claim_counter, 1);
-            hi = lo + 1;
-        } else {
-            const long long left = P - peek(a.claim_counter);
-            const long long guided = left / (3 * (long long)workers);
-            const int size = (int)(guided > max_units ? guided : max_units);
-            lo = atomicAdd(a.claim_counter, size);
-            hi = (int)(lo + (long long)size < P ? lo + size : P);
-        }
-        if (lo >= P)
-            lo = hi = -1;
+        const int i = !a.first_fixed ? atomicAdd(a.claim_counter, 1)
+                      : n_pub == 0   ? workers - 1 - worker
+                                     : workers + atomicAdd(a.claim_counter, 1);
+        return i < n_items ? i : -1;
     }
-    // Claimer: claims one more chunk and publishes it in the ring (with its group looked up
-    // in round-robin mode, so that the other roles need not go to global memory for it).
+    // Claimer: claims one more item and publishes it in the ring.
     __device__ bool publish_one()
     {
         const int slot = n_pub % FF_CLAIMS;
         const uint32_t par = (uint32_t)(n_pub / FF_CLAIMS) & 1u;
-        int lo, hi, sidx = 0;
-        Segment grp = sg;
-        claim(lo, hi);
-        if (lo >= 0 && a.round_robin) {
-            if (n_pub > 0 || !a.first_fixed)
-                load_pair(lo / (ntiles * a.routed_ksplit));
-            sidx = pair_seg;
-            grp.expert = pair_group.x;
-            grp.row0 = pair_group.y;
-            grp.n = pair_group.z;
-            grp.first_seg = pair_group.w;
-        }
+        const int item = claim();
+        if (item >= 0 && (n_pub > 0 || !a.first_fixed))
+            load_entry(item / (ntiles * a.routed_ksplit));
         if (!mbar_wait<PAIR>(ring.empty0 + 8u * slot, par ^ 1u, ring.abort_flag, ring.status))
             return false;
         if (PAIR) {
             const uint32_t pe = ring.peer_data + slot * FF_CLAIM_WORDS * 4;
-            st_cluster_v4(pe, lo, hi, sidx, grp.expert);
-            st_cluster_v4(pe + 16, grp.row0, grp.n, grp.first_seg, 0);
+            st_cluster_v4(pe, item, entry.seg, entry.expert, entry.row0);
+            st_cluster_v4(pe + 16, entry.n, entry.first_seg, 0, 0);
             mbar_arrive_cluster(ring.peer_full0 + 8u * slot);
         }
         int *e = ring.data + slot * FF_CLAIM_WORDS;
-        e[0] = lo;
-        e[1] = hi;
-        e[2] = sidx;
-        e[3] = grp.expert;
-        e[4] = grp.row0;
-        e[5] = grp.n;
-        e[6] = grp.first_seg;
+        e[0] = item;
+        e[1] = entry.seg;
+        e[2] = entry.expert;
+        e[3] = entry.row0;
+        e[4] = entry.n;
+        e[5] = entry.first_seg;
         __threadfence_block();
         mbar_arrive(ring.full0 + 8u * slot);
         ++n_pub;
-        if (lo < 0)
+        if (item < 0)
             end_published = true;
         return true;
     }
-    // Next chunk [lo, hi) of the routed work; false when none is left (or on abort).  In
-    // round-robin mode the chunk is one item and `grp` receives its group.  While plenty of
-    // work is left the claimer publishes one chunk beyond the one it is about to work on, so
-    // that every role knows its next item before it finishes the current one (near the end a
-    // chunk held in reserve would starve another CTA).
-    __device__ bool acquire(int &lo, int &hi, Segment &grp, int &sidx)
+    // Next routed item and its segment; -1 when none is left (or on abort).  While plenty of work
+    // is left the claimer publishes one item beyond the one it is about to work on, so that every
+    // role knows its next item before it finishes the current one (near the end an item held in
+    // reserve would starve another worker).
+    __device__ int acquire(Segment &sg)
     {
         const int slot = n_claims % FF_CLAIMS;
         const uint32_t par = (uint32_t)(n_claims / FF_CLAIMS) & 1u;
@@ -283,9 +235,8 @@ struct ItemWalk {
             bool published = true;
             while (lead) {
                 // (the counter is only read where the answer can be yes)
-                const long long ample = 4 * (long long)workers * (a.round_robin ? 1 : max_units);
-                const bool plenty =
-                    P > ample && P - peek(a.claim_counter) > ample;
+                const int ample = 4 * workers;
+                const bool plenty = n_items > ample && n_items - peek(a.claim_counter) > ample;
                 if (end_published || n_pub >= n_claims + (plenty ? 2 : 1))
                     break;
                 if (!publish_one()) {
@@ -294,7 +245,7 @@ struct ItemWalk {
                 }
             }
             if (!__all_sync(0xffffffffu, published))
-                return false;
+                return -1;
             // the first lane wrote the entry and no barrier stands between it and the others here
             // (a vote orders no memory); also: all lanes have read an entry before it is reused
             __syncwarp();
@@ -302,16 +253,15 @@ struct ItemWalk {
             // (the lanes of a warp wait one by one: when a wait gives up, all leave together)
             const bool got = mbar_wait<PAIR>(ring.full0 + 8u * slot, par, ring.abort_flag, ring.status);
             if (!__all_sync(0xffffffffu, got))
-                return false;
+                return -1;
         }
         ++n_claims;
-        lo = e[0];
-        hi = e[1];
-        sidx = e[2];
-        grp.expert = e[3];
-        grp.row0 = e[4];
-        grp.n = e[5];
-        grp.first_seg = e[6];
+        const int item = e[0];
+        sg.seg = e[1];
+        sg.expert = e[2];
+        sg.row0 = e[3];
+        sg.n = e[4];
+        sg.first_seg = e[5];
         if (!claimer) {
             __syncwarp();  // every lane has read the entry before it is released
             if (lead) {
@@ -321,122 +271,55 @@ struct ItemWalk {
                     mbar_arrive(ring.empty0 + 8u * slot);
             }
         }
-        return lo >= 0;
+        return item;
     }
-    // false when this CTA has no further item
+    // false when this worker has no further item
     __device__ bool next(Item &it)
     {
-        for (;;) {
-            if (have_tile) {
-                if (t_s < t_s_end) {
-                    it.grp = t_grp;
-                    it.expert = t_expert;
-                    it.f0 = t_u0 << USH;
-                    it.h = t_h << USH;
-                    it.row0 = t_row0 + t_s * t_seg_rows;
-                    it.n = min(t_seg_rows, t_n - t_s * t_seg_rows);
-                    it.seg = t_seg0 + t_s;
-                    it.w_once = t_once;
-                    it.k0 = t_k0;
-                    it.k1 = t_k1;
-                    it.out_off = t_out_off;
-                    ++t_s;
-                    return true;
-                }
-                have_tile = false;
-            }
-            if (sj < s_units) {  // next unit of the shared expert: (tile, k chunk, segment)
-                const int tc = sj / nseg_s, q = sj - tc * nseg_s;
-                const int tile = tc / a.shared_ksplit, chunk = tc - tile * a.shared_ksplit;
-                t_k0 = chunk * a.shared_kchunk;
-                t_k1 = min(a.K[1], t_k0 + a.shared_kchunk);
-                t_out_off = chunk * a.shared_part_stride;
-                t_u0 = tile * s_base + min(tile, s_rem);
-                t_h = s_base + (tile < s_rem ? 1 : 0);
-                t_grp = 1;
-                t_expert = 0;
-                t_row0 = 0;
-                t_seg0 = 0;
-                t_n = a.T;
-                t_seg_rows = balanced_segment_rows(a.T, nseg_s);
-                t_s = q;
-                t_s_end = q + 1;
-                t_once = nseg_s <= 1;
-                sj += workers;
-                have_tile = true;
-                continue;
-            }
-            if (!synced)
-                sync(true);
-            if (finished)
-                return false;
-            if (!have_chunk) {
-                int lo, hi, sidx;
-                if (!acquire(lo, hi, sg, sidx)) {
-                    finished = true;
-                    return false;
-                }
-                if (a.round_robin) {
-                    // one (segment, tile, k chunk) item
-                    const int st = a.routed_ksplit == 1 ? lo : lo / a.routed_ksplit;
-                    const int chunk = lo - st * a.routed_ksplit;
-                    const int tile = st % ntiles;
-                    g_nseg = n_segments(sg.n);
-                    t_u0 = tile * max_units;
-                    t_h = min(max_units, R0 - t_u0);
-                    t_grp = 0;
-                    t_expert = sg.expert;
-                    t_row0 = sg.row0;
-                    t_seg0 = sg.first_seg;
-                    t_n = sg.n;
-                    t_seg_rows = balanced_segment_rows(sg.n, g_nseg);
-                    t_s = sidx - sg.first_seg;
-                    t_s_end = t_s + 1;
-                    t_once = g_nseg <= 1;
-                    t_k0 = chunk * a.routed_kchunk;
-                    t_k1 = min(a.K[0], t_k0 + a.routed_kchunk);
-                    t_out_off = chunk * a.routed_part_stride;
-                    have_tile = true;
-                    continue;
-                }
-                boundary(lo, fs, u);
-                boundary(hi, fs_hi, u_hi);
-                group_loaded = false;
-                have_chunk = true;
-            }
-            if (fs >= nseg_total || fs > fs_hi || (fs == fs_hi && u >= u_hi)) {
-                have_chunk = false;  // chunk exhausted (or empty after rounding)
-                continue;
-            }
-            if (!group_loaded) {
-                sg = a.seg[fs];
-                g_nseg = n_segments(sg.n);
-                g_u_end = fs == fs_hi ? u_hi : R0;
-                group_loaded = true;
-            }
-            if (u < g_u_end) {  // next tile of this group, all its segments
-                t_h = min(max_units, g_u_end - u);
-                t_grp = 0;
-                t_expert = sg.expert;
-                t_u0 = u;
-                t_row0 = sg.row0;
-                t_seg0 = sg.first_seg;
-                t_n = sg.n;
-                t_seg_rows = balanced_segment_rows(sg.n, g_nseg);
-                t_s = 0;
-                t_s_end = g_nseg;
-                t_once = g_nseg <= 1;
-                t_k0 = 0;
-                t_k1 = a.K[0];
-                t_out_off = 0;
-                u += t_h;
-                have_tile = true;
-                continue;
-            }
-            fs += g_nseg;  // group done: on to the next one
-            u = 0;
-            group_loaded = false;
+        if (sj < s_units) {  // next unit of the shared expert: (tile, k chunk, segment)
+            const int tc = sj / nseg_s, q = sj - tc * nseg_s;
+            const int tile = tc / a.shared_ksplit, chunk = tc - tile * a.shared_ksplit;
+            const int rows = balanced_segment_rows(a.T, nseg_s);
+            it.grp = 1;
+            it.expert = 0;
+            it.f0 = (tile * s_base + min(tile, s_rem)) << USH;
+            it.h = (s_base + (tile < s_rem ? 1 : 0)) << USH;
+            it.row0 = q * rows;
+            it.n = min(rows, a.T - q * rows);
+            it.seg = q;
+            it.w_once = nseg_s <= 1;
+            it.k0 = chunk * a.shared_kchunk;
+            it.k1 = min(a.K[1], it.k0 + a.shared_kchunk);
+            it.out_off = chunk * a.shared_part_stride;
+            sj += workers;
+            return true;
         }
+        if (!synced)
+            sync(true);
+        if (finished)
+            return false;
+        Segment sg;
+        const int item = acquire(sg);
+        if (item < 0) {
+            finished = true;
+            return false;
+        }
+        const int st = a.routed_ksplit == 1 ? item : item / a.routed_ksplit;
+        const int chunk = item - st * a.routed_ksplit, tile = st % ntiles;
+        const int u0 = tile * max_units, nseg = n_segments(sg.n), q = sg.seg - sg.first_seg;
+        const int rows = balanced_segment_rows(sg.n, nseg);
+        it.grp = 0;
+        it.expert = sg.expert;
+        it.f0 = u0 << USH;
+        it.h = min(max_units, R0 - u0) << USH;
+        it.row0 = sg.row0 + q * rows;
+        it.n = min(rows, sg.n - q * rows);
+        it.seg = sg.seg;
+        it.w_once = nseg <= 1;
+        it.k0 = chunk * a.routed_kchunk;
+        it.k1 = min(a.K[0], it.k0 + a.routed_kchunk);
+        it.out_off = chunk * a.routed_part_stride;
+        return true;
     }
 };
 

@@ -47,8 +47,8 @@ static Workspace static_scratch_layout(const moe_config_t &c, int T)
     WorkspaceCarver cut(w);
     w.status = cut.take(64 * 4);
     w.plan_header = cut.take(PLAN_HEADER_INTS * 4);
+    cut.take(PLAN_RESERVED_BYTES * (size_t)max_segments(c.n_experts, (int)A));
     w.plan_seg = cut.take(sizeof(Segment) * (size_t)max_segments(c.n_experts, (int)A));
-    w.plan_pairs = cut.take(sizeof(PairEntry) * (size_t)max_segments(c.n_experts, (int)A));
     w.plan_done = cut.take(4 * ((size_t)max_segments(c.n_experts, (int)A) + max_shared_segments(T)));
     w.plan_done_shared_at = (size_t)max_segments(c.n_experts, (int)A);
     w.x_sorted = cut.take(A * (size_t)c.hidden * 2);

@@ -64,35 +64,15 @@ __device__ void build_plan(const int *cnt_sh, const int *off_sh, int *scan, int 
         scan[tid] = nseg;
     __syncthreads();
     block_exclusive_scan(scan, tmp, E, total);
-    if (nseg > 0) {
-        const int first = scan[tid];
-        Segment sg;
-        sg.expert = tid;
-        sg.row0 = row0;
-        sg.n = cnt;
-        sg.first_seg = first;
-        for (int i = 0; i < nseg; ++i) {
-            plan.seg[first + i] = sg;
-            plan.done_routed[first + i] = 0;
-        }
-    }
-    if (tid == 0)
-        plan.header[0] = *total;
-    // the item list: one entry per segment, carrying its group
+    // one entry per segment, carrying its group
     const int first = nseg > 0 ? scan[tid] : 0;
-    for (int q = 0; q < nseg; ++q) {
-        PairEntry pe;
-        pe.expert = tid;
-        pe.row0 = row0;
-        pe.n = cnt;
-        pe.first_seg = first;
-        pe.seg = first + q;
-        pe.pad[0] = pe.pad[1] = pe.pad[2] = 0;
-        plan.pairs[first + q] = pe;
+    for (int i = 0; i < nseg; ++i) {
+        plan.seg[first + i] = Segment{tid, row0, cnt, first, first + i, {0, 0, 0}};
+        plan.done_routed[first + i] = 0;
     }
     if (tid == 0) {
-        plan.header[1] = *total;
-        plan.header[2] = 0;  // work claimed so far by the gate/up pass ...
+        plan.header[0] = *total;
+        plan.header[2] = 0;  // items claimed so far by the gate/up pass ...
         plan.header[3] = 0;  // ... and by the down pass
     }
 }
@@ -446,22 +426,9 @@ route_group_small_kernel(const float *__restrict__ logits, const __nv_bfloat16 *
                 total = __popc(firsts);
             if (blockIdx.x == 1 && first) {
                 active[arank] = e;
-                if (plan.header != nullptr) {  // one segment and one pair per activated expert
-                    Segment sg;
-                    sg.expert = e;
-                    sg.row0 = less;
-                    sg.n = __popc(peers);
-                    sg.first_seg = arank;
-                    plan.seg[arank] = sg;
+                if (plan.header != nullptr) {  // one segment per activated expert
+                    plan.seg[arank] = Segment{e, less, __popc(peers), arank, arank, {0, 0, 0}};
                     plan.done_routed[arank] = 0;
-                    PairEntry pe;
-                    pe.expert = e;
-                    pe.row0 = less;
-                    pe.n = sg.n;
-                    pe.first_seg = arank;
-                    pe.seg = arank;
-                    pe.pad[0] = pe.pad[1] = pe.pad[2] = 0;
-                    plan.pairs[arank] = pe;
                 }
             }
         }
@@ -485,8 +452,7 @@ route_group_small_kernel(const float *__restrict__ logits, const __nv_bfloat16 *
                 offsets[E] = A;
                 n_active[0] = n_act;
                 if (plan.header != nullptr) {
-                    plan.header[0] = n_act;  // segments
-                    plan.header[1] = n_act;  // pairs
+                    plan.header[0] = n_act;
                     plan.header[2] = 0;
                     plan.header[3] = 0;
                 }

@@ -15,18 +15,14 @@ namespace moe {
 // ---------------------------------------------------------------------------------------
 constexpr int SEG_TOKENS = 128;
 
-struct Segment {
+// A segment with its group: everything a CTA needs to start on a (segment, tile) item in one
+// 32-byte load.
+struct alignas(16) Segment {
     int32_t expert;     // routed expert id of the group
     int32_t row0;       // first sorted row of the group
     int32_t n;          // rows of the group (all its segments together)
     int32_t first_seg;  // plan index of the group's first segment
-};
-
-// A segment with its group: everything a CTA needs to start on a (segment, tile) item in one
-// 32-byte load.
-struct alignas(16) PairEntry {
-    int32_t expert, row0, n, first_seg;  // the group (as in Segment)
-    int32_t seg;                         // plan index of the segment
+    int32_t seg;        // plan index of this segment
     int32_t pad[3];
 };
 

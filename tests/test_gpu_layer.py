@@ -61,7 +61,7 @@ SCHEDULING_CASES = [
 
 @pytest.mark.parametrize("name,H,E,k,I,Is,B,gamma", SCHEDULING_CASES)
 def test_scheduling_mode_case(name, H, E, k, I, Is, B, gamma):
-    """One case of the scheduling-mode test below (in this process: the host's own choice)."""
+    """Shapes that exercise the dealing of the work (shared units, segments, ragged tiles)."""
     shape = wl.small_shape(name, H, E, k, I, Is, 0, 0, 1)
     w = wl.make_weights(shape, 300 + E, "cuda")
     T = B * (gamma + 1)
@@ -82,14 +82,6 @@ def _run_child(env_extra, k_expr):
         env=env, cwd=root, capture_output=True, text=True, timeout=900)
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-2000:]
     assert "passed" in r.stdout
-
-
-@pytest.mark.parametrize("mode", ["0", "1"])
-def test_layer_parity_in_both_scheduling_modes(mode):
-    """The FFN kernels hand out the routed work either as chunks of consecutive tiles or as
-    single (segment pair, tile) items; MOE_FF_RR (a test hook the library reads once per
-    process) forces one of the two, so the cases run in a child process per mode."""
-    _run_child({"MOE_FF_RR": mode}, "scheduling_mode_case")
 
 
 # One to four tokens with at most 32 assignments take the one-launch kernel (logits, routing,

@@ -163,23 +163,19 @@ static void trial(Rng &rng)
     for (int i = rng.in(1, 7); i > 0; --i)
         groups.push_back(rng.pick({1, 5, 16, 100, 128, 129, 200, 256, 257, 400}));
     std::vector<Segment> seg;
-    std::vector<PairEntry> pairs;
     int row = 0;
     for (size_t e = 0; e < groups.size(); ++e) {
         const int n = groups[e], ns = (n + a.seg_rows - 1) / a.seg_rows, first = (int)seg.size();
         for (int q = 0; q < ns; ++q) {
-            seg.push_back(Segment{(int)(3 * e + 1), row, n, first});
-            pairs.push_back(PairEntry{(int)(3 * e + 1), row, n, first, first + q, {0, 0, 0}});
+            seg.push_back(Segment{(int)(3 * e + 1), row, n, first, first + q, {0, 0, 0}});
         }
         row += n;
     }
-    alignas(16) int32_t header[16] = {(int)seg.size(), (int)seg.size(), 0, 0};
+    alignas(16) int32_t header[16] = {(int)seg.size(), 0, 0, 0};
     a.plan_header = header;
     a.seg = seg.data();
-    a.max_pairs = (int)pairs.size();
-    a.pairs = pairs.data();
+    a.max_seg = (int)seg.size();
     a.claim_counter = header + (down ? 3 : 2);
-    a.round_robin = 1;
 
     // roles: the weight producer's warp and R readers in every CTA
     const int R = 2, workers = rng.in(1, 3), ctas = workers * CTAS;
