@@ -53,24 +53,6 @@ bool pdl_enabled()
     return on;
 }
 
-int geometry_override()
-{
-    static const int v = [] {
-        const char *e = getenv("MOE_FF_WIDE");
-        return !e ? -1 : (e[0] == '1' ? 1 : (e[0] == '0' ? 0 : -1));
-    }();
-    return v;
-}
-
-int pair_override()
-{
-    static const int v = [] {
-        const char *e = getenv("MOE_FF_PAIR");
-        return !e ? -1 : (e[0] == '1' ? 1 : (e[0] == '0' ? 0 : -1));
-    }();
-    return v;
-}
-
 static thread_local int g_last_launches = 0;
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

@@ -252,14 +252,9 @@ cudaError_t launch_layer_small(const moe_config_t &c, const moe_weights_t &w, co
 
 int sm_count();
 bool pdl_enabled();  // programmatic dependent launch between the layer's kernels
-// Test hook, read once per process from MOE_FF_WIDE: 0 / 1 forces the ring geometry with segments
-// of 128 / 256 rows, -1 (unset) leaves the choice to the host's rule.
-int geometry_override();
-// From MOE_SMALL_FUSED: 0 keeps calls of a few tokens on the chain of kernels every other call
+// Test hook, read once per process from MOE_SMALL_FUSED: 0 keeps calls of a few tokens on the chain of kernels every other call
 // uses, -1 (unset) lets them take the one-launch kernel.
 int small_layer_override();
-// From MOE_FF_PAIR: 0 / 1 forces the FFN kernels to run on single CTAs / on CTA pairs.
-int pair_override();
 // Token rows per segment of the routed groups for a call with T tokens: 128 or 256 (the plan and
 // the FFN kernels of one call must agree on it).
 int ffn_segment_rows(const moe_config_t &c, int T);

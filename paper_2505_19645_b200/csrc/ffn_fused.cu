@@ -64,12 +64,14 @@
 // overlaps the routing kernels; everything produced inside the layer is touched after it,
 // except h, which the down pass takes segment by segment as described above.
 #include <math.h>
+#include <stdlib.h>
 #include <string.h>
 
 #include <mutex>
 
 #include "tc_ptx.cuh"
 
+#include "ffn_geometry.h"
 #include "ffn_walk.cuh"
 
 namespace moe {
@@ -303,12 +305,10 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
         // down pass: h is written by the preceding kernel, which may still be running; a
         // segment's rows are fetched once its progress counter says they are complete
         ItemWalk<PAIR> walk(args, claims, false, !GATED);
-        XRingWalk ring(args.x_units);
+        TokenRing ring(args.x_units);
+        int starts[FF_STEPS];
         int seen = -1;  // (group kind, segment) key last found complete
         const uint64_t pol_keep = l2_policy_evict_last();
-        int released = 0;          // entries known to have been consumed
-        int v_cur = 0, v_rel = 0;  // virtual unit positions: issued up to / free up to
-        int v_start_of[FF_STEPS];  // where each entry's rows begin (after its padding)
         bool ok = true;
         Item it;
         while (ok && walk.next(it)) {
@@ -335,22 +335,15 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
             for (int k0 = k_begin; k0 < k_end; k0 += 64 * kb) {
                 const int nbox = min(kb, (k_end - k0 + 63) >> 6);
                 const int j = ring.count;
-                int pad;
-                const int at = ring.place(m, pad);
-                const int v_start = v_cur + pad, v_end = v_start + m;
-                // the entry's units (and its barrier pair) must have been released:
-                // everything before the oldest entry still in use is free, the
-                // padding in front of it included
-                while (ok && released < j && (j - released >= FF_STEPS || v_end - v_rel > args.x_units)) {
-                    const bool free = mbar_wait(empty(released), parity(released), abortp, args.status);
+                const int at = ring.place(m);
+                while (ok && ring.must_release()) {
+                    const bool free = mbar_wait(empty(ring.released), parity(ring.released), abortp, args.status);
                     ok = __all_sync(0xffffffffu, free);
-                    ++released;
-                    v_rel = released < j ? v_start_of[released % FF_STEPS] : v_start;
+                    ring.release(starts);
                 }
                 if (!ok)
                     break;
-                v_start_of[j % FF_STEPS] = v_start;
-                v_cur = v_end;
+                ring.issued(starts);
                 const uint32_t base = ring_x + (uint32_t)at * FF_X_UNIT;
                 const uint32_t bar = leader_bar(full(j));
                 if (elect_one()) {
@@ -377,8 +370,9 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
             }
         }
         if (PAIR)  // the leader's last releases have arrived before this CTA may exit
-            for (; ok && released < ring.count; ++released)
-                ok = __all_sync(0xffffffffu, mbar_wait(empty(released), parity(released), abortp, args.status));
+            for (; ok && ring.released < ring.count; ++ring.released)
+                ok = __all_sync(0xffffffffu, mbar_wait(empty(ring.released), parity(ring.released), abortp,
+                                                       args.status));
         if (!walk.synced)
             walk.sync(true);
         if (!GATED)
@@ -422,8 +416,7 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
                 for (int box = 0; box < n_box; box += kb) {
                     const int nbox = min(kb, n_box - box);
                     const int j = ring.count;
-                    int pad;
-                    const int at = ring.place(pieces * kb, pad);
+                    const int at = ring.place(pieces * kb);
                     const uint32_t xbase = ring_x + (uint32_t)at * FF_X_UNIT;
                     bool ready = mbar_wait(full(j), parity(j), abortp, args.status);
                     if (box == 0)
@@ -783,31 +776,27 @@ static MapKey map_key(bool gated, const void *p0, const void *p1, const void *p2
     return k;
 }
 
-// Expected number of activated experts for T tokens (Eq. N(t): E(1 - (1 - K/E)^T)); the host
-// never sees the routing result, so it sizes rings and shared tiles from the expectation.
-static double expected_active_experts(int E, int k, int T)
+int geometry_override()
 {
-    return E * (1.0 - pow(1.0 - (double)k / E, (double)T));
+    static const int v = [] {
+        const char *e = getenv("MOE_FF_WIDE");
+        return !e ? -1 : (e[0] == '1' ? 1 : (e[0] == '0' ? 0 : -1));
+    }();
+    return v;
 }
+
+int pair_override()
+{
+    static const int v = [] {
+        const char *e = getenv("MOE_FF_PAIR");
+        return !e ? -1 : (e[0] == '1' ? 1 : (e[0] == '0' ? 0 : -1));
+    }();
+    return v;
+}
+
+int ffn_segment_rows(const moe_config_t &c, int T) { return segment_rows(c, T); }
 
 static int ffn_grid() { return sm_count(); }
-
-// Whether the FFN kernels of a call run on CTA pairs: always in the contraction geometry (see the
-// top of the file), in the streaming one beyond 128 tokens.  There a pair's token entries are half
-// as large, so that three weight slots fit where a single CTA has two (96 KB of token ring for
-// segments of 128 rows).  Layer on single CTAs -> pairs: DeepSeek-V3 shape T = 256 3367 -> 3287 us,
-// T = 1024 3647 -> 3560, T = 2048 4075 -> 3944, T = 3072 4428 -> 4374; Mixtral shape T = 192
-// 488 -> 474, T = 384 537 -> 527; Qwen1.5 shape T = 192 to 640 within 1 %.  Up to 128 tokens the
-// token rows are a small part of what an SM loads, single CTAs have three slots too, and a pair
-// waits for the slower of its two streams (DeepSeek-V3 shape T = 128 3172 on single CTAs, 3248 on
-// pairs; Mixtral shape T = 80 443 and 450).
-static bool ffn_pairs(const moe_config_t &c, int T)
-{
-    if (ffn_segment_rows(c, T) > FF_SEG)
-        return true;
-    const int force = pair_override();
-    return force >= 0 ? force == 1 : T > FF_SEG;
-}
 
 // What pulls work items: a CTA, or a pair of CTAs whose tiles are twice as high.
 struct FfnWorkers {
@@ -819,52 +808,6 @@ static FfnWorkers ffn_workers(const moe_config_t &c, int T)
     return FfnWorkers{ctas, ffn_grid() / ctas};
 }
 
-// Segment size of a call (the N limit of its tensor-core instructions).  Groups in the hundreds
-// of rows want the contraction geometry: segments of 256 rows, so that a weight tile is fetched
-// once per 256 tokens and the instruction runs at its full rate.  Small groups want the
-// streaming geometry (segments of 128 rows, 64 KB weight slots, double-buffered accumulators).
-// The host never sees the routing result, so it decides on the expected rows per group -- and on
-// the shared expert, whose group is all T tokens: where its weights are a large part of the
-// layer's, every extra segment is another pass over them through L2.
-int ffn_segment_rows(const moe_config_t &c, int T)
-{
-    const int force = geometry_override();
-    if (force >= 0)
-        return force == 1 ? FF_SEG_WIDE : FF_SEG;
-    if (T <= FF_SEG)
-        return FF_SEG;
-    // measured cross-over: about 112 expected rows per group (most groups then exceed one
-    // 128-row segment), or a shared expert several times an expert's size
-    const double rows_per_group = (double)T * c.top_k / expected_active_experts(c.n_experts, c.top_k, T);
-    if (rows_per_group > 0.875 * FF_SEG)
-        return FF_SEG_WIDE;
-    return c.shared_inter >= 6 * c.inter ? FF_SEG_WIDE : FF_SEG;
-}
-
-// Up to 128 tokens no group of the layer has more than one 128-row segment and the token ring
-// can be 32 KB, which leaves room for a third weight slot (worth 3-4 % of the layer) --
-// provided the entries stay within half of the ring, i.e. 64 rows: always so up to 64 tokens;
-// between 65 and 128 tokens only while the routed groups are expected to be small (a larger
-// group still works, its rows are then not fetched ahead), and the shared expert's rows are
-// then cut into two 64-row segments.
-static bool small_token_ring(const moe_config_t &c, int T)
-{
-    if (T <= FF_SEG / 2)
-        return true;
-    if (T > FF_SEG)
-        return false;
-    // (a mean of up to a quarter of a segment: the largest group then stays within a half)
-    return (double)T * c.top_k / expected_active_experts(c.n_experts, c.top_k, T) <= FF_SEG / 4 + 0.5;
-}
-
-// Token rows per segment of the shared expert (see small_token_ring).
-static int shared_segment_rows(const moe_config_t &c, int T)
-{
-    if (T > FF_SEG / 2 && small_token_ring(c, T))
-        return FF_SEG / 2;
-    return ffn_segment_rows(c, T);
-}
-
 // Number of tiles the shared expert's rows are cut into.  The shared expert's work units are
 // (tile, k chunk, segment); a unit should cost about the expected per-CTA share of the whole
 // pass (or less), with the tile height within [min_tile, max_tile] rows (a weight block
@@ -874,7 +817,7 @@ static int shared_tile_count(const moe_config_t &c, int T, int rows_routed, int 
 {
     const FfnWorkers wk = ffn_workers(c, T);
     const int unit = 16 * wk.ctas;  // (a pair's tiles: twice the height, units of 32 rows)
-    const int seg_s = shared_segment_rows(c, T), seg_r = ffn_segment_rows(c, T);
+    const int seg_s = shared_segment_rows(c, T), seg_r = segment_rows(c, T);
     const int nseg_s = (T + seg_s - 1) / seg_s;
     const int units = rows_shared / unit;
     const double k_ratio = (double)K_shared / K_routed;  // cost of a shared row unit per segment
@@ -887,33 +830,6 @@ static int shared_tile_count(const moe_config_t &c, int T, int rows_routed, int 
     if (tu > (max_tile >> 4))
         tu = max_tile >> 4;
     return (units + tu - 1) / tu;
-}
-
-// Ring geometry.  Streaming: two k boxes per weight slot (64 KB for a full tile: every row is
-// fetched in 256 contiguous bytes, which both HBM and L2 serve markedly faster than 128); the
-// token ring holds two entries of the largest possible segment on CTA pairs and while no group
-// can exceed 64 rows (32 KB, three weight slots), three 128-row entries otherwise (96 KB, two
-// slots).  (One k box per slot, five slots, measured 3-4 % slower on pairs as well.)
-// Contraction: pairs, one k box per slot and per entry, four entries of half a 256-row segment
-// (64 KB), five slots.
-static void ffn_geometry(const moe_config_t &c, int T, FfnArgs &a)
-{
-    a.seg_rows = ffn_segment_rows(c, T);
-    const bool wide = a.seg_rows > FF_SEG;
-    a.kboxes = wide ? 1 : 2;
-    a.acc_sets = wide ? 1 : 2;
-    a.w_slot_bytes = 256 * 128 * a.kboxes;  // a full tile: 256 rows per k box
-    // (a CTA of a pair holds half of a segment's rows: entries of at most 16 KB in both geometries)
-    const int x_ring_bytes = wide ? 64 * 1024
-                             : ffn_pairs(c, T) || small_token_ring(c, T) ? 32 * 1024 : 96 * 1024;
-    a.x_units = x_ring_bytes / FF_X_UNIT;
-    const int avail = FF_SMEM_LIMIT - 1024 - 512;  // alignment slack, static shared memory
-    int ns = (avail - x_ring_bytes) / a.w_slot_bytes;
-    if (ns > FF_STEPS)
-        ns = FF_STEPS;
-    a.n_w_slots = ns;
-    a.wait_us = (int)(FF_WAIT_NS / 1000ull);
-    a.shared_seg = shared_segment_rows(c, T);
 }
 
 template <bool GATED, bool PAIR>
@@ -957,6 +873,7 @@ cudaError_t launch_ffn_gateup(const moe_config_t &c, const moe_weights_t &w, con
                                                      1, 64, 128)
                                  : 0;
     ffn_geometry(c, T, a);
+    a.wait_us = (int)(FF_WAIT_NS / 1000ull);
     FfnMaps maps;
     const MapKey key = map_key(true, w.w_gate, w.w_up, x_sorted, with_shared ? w.ws_gate : nullptr,
                                with_shared ? w.ws_up : nullptr, with_shared ? x : nullptr, nullptr, E,
@@ -1074,6 +991,7 @@ cudaError_t launch_ffn_down(const moe_config_t &c, const moe_weights_t &w, int T
                                                      a.shared_ksplit, 128, 256)
                                  : 0;
     ffn_geometry(c, T, a);
+    a.wait_us = (int)(FF_WAIT_NS / 1000ull);
     FfnMaps maps;
     const MapKey key = map_key(false, w.w_down, h, with_shared ? w.ws_down : nullptr,
                                with_shared ? h_shared : nullptr, nullptr, nullptr, nullptr, E,

@@ -327,10 +327,10 @@ struct ItemWalk {
 // when it does not fit before the end of the ring it starts at unit 0.  Producer and MMA
 // issuer replay the same sequence of sizes, so they agree on every position.
 struct XRingWalk {
-    int units, cur, count;
-    __device__ XRingWalk(int n_units) : units(n_units), cur(0), count(0) {}
+    int units, cur, count, pad;
+    __device__ XRingWalk(int n_units) : units(n_units), cur(0), count(0), pad(0) {}
     // returns the first unit of the next entry; `pad` = units skipped at the end of the ring
-    __device__ int place(int m, int &pad)
+    __device__ int place(int m)
     {
         pad = 0;
         if (cur + m > units) {
@@ -341,6 +341,41 @@ struct XRingWalk {
         cur += m;
         ++count;
         return at;
+    }
+};
+
+// The producer's side: which entries must have been consumed before the next one may be issued.
+// place() an entry, wait for entry `released` and release() it while must_release(), then issue.
+// `starts`: where each entry's rows begin, after its padding (an array of the caller's, so that the
+// rest stays in registers).
+struct TokenRing : XRingWalk {
+    int released;            // entries known to have been consumed
+    int v_cur, v_rel;        // virtual unit positions: issued up to / free up to
+    int v_start, v_end;      // of the entry placed last
+    __device__ TokenRing(int n_units) : XRingWalk(n_units), released(0), v_cur(0), v_rel(0), v_start(0), v_end(0) {}
+    __device__ int place(int m)
+    {
+        const int at = XRingWalk::place(m);
+        v_start = v_cur + pad;
+        v_end = v_start + m;
+        return at;
+    }
+    // the entry's units and its barrier pair must be free: everything before the oldest entry still
+    // in use is, the padding in front of it included
+    __device__ bool must_release() const
+    {
+        const int j = count - 1;
+        return released < j && (j - released >= FF_STEPS || v_end - v_rel > units);
+    }
+    __device__ void release(const int (&starts)[FF_STEPS])
+    {
+        ++released;
+        v_rel = released < count - 1 ? starts[released % FF_STEPS] : v_start;
+    }
+    __device__ void issued(int (&starts)[FF_STEPS])
+    {
+        starts[(count - 1) % FF_STEPS] = v_start;
+        v_cur = v_end;
     }
 };
 
