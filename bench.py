@@ -58,7 +58,7 @@ EXTRA_POINTS = {"qwen2-57b-a14b": [(512, 3), (1024, 3)], "deepseek-v3": [(512, 3
 # were taken on (written by --record-traffic from an ncu CSV; see the file for the command)
 TRAFFIC_RECORD = os.path.join(ROOT, "profiles", "gate_up_dram_traffic.txt")
 KERNEL_SOURCES = ["paper_2505_19645_b200/csrc/" + f
-                  for f in ("ffn_fused.cu", "ffn_walk.cuh", "plan.h", "tc_ptx.cuh", "common.cuh")]
+                  for f in ("ffn_fused.cu", "ffn_walk.cuh", "ffn_geometry.h", "plan.h", "tc_ptx.cuh", "common.cuh")]
 
 
 def load_peaks():

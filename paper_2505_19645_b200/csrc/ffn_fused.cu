@@ -45,8 +45,9 @@
 // bytes: each SM is filled at no more than about 44 bytes per clock, a 256 x 256 tile of a single
 // CTA wants 64 at the full instruction rate and 256 x 160 wants 81; a pair's CTA wants 47 and 66.
 // The leader (even CTA) claims the work for both, its barriers count the bytes of both and its
-// commits release the slots of both.  Layer, single CTAs -> pairs: Qwen2 shape T = 1280
-// 1298 -> 1208 us, Mixtral shape T = 1280 1082 -> 1004.
+// commits release the slots of both.  Layer at the power cap, single CTAs -> pairs when this was
+// taken up, medians of three runs of either in turn: Qwen2 shape T = 1280 1300 -> 1266 us, Mixtral
+// shape T = 1280 1163 -> 1123.
 //
 // CTA = 11 warps.  warp 0: weight producer, warp 1: MMA issuer (idle in a pair's second CTA) and
 // owner of the TMEM allocation, warp 2: token-operand producer (in all three the warp runs in
@@ -151,10 +152,11 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
     __shared__ __align__(16) int claim_data[FF_CLAIMS * FF_CLAIM_WORDS];
 
     const int NS = args.n_w_slots;
-    const int kb = args.kboxes;
+    // (only pairs run the contraction geometry)
+    const int kb = PAIR ? args.kboxes : 2;
     // TMEM: a set of accumulators is two blocks (gate and up, or two blocks of 128 down rows) of
     // acc_block columns each; two sets of 2 x 128 columns, or one set of 2 x 256
-    const int acc_sets = args.acc_sets;
+    const int acc_sets = PAIR ? args.acc_sets : 2;
     const uint32_t acc_block = acc_sets == 2 ? 128u : 256u;
     // token ring first (an MMA reads exactly the rows of its entry, rounded up to 16; a weight
     // block is read as 128 rows, which for a shorter tile ends inside the slot's capacity)
@@ -785,11 +787,11 @@ int geometry_override()
     return v;
 }
 
-int pair_override()
+bool pairs_forced()
 {
-    static const int v = [] {
+    static const bool v = [] {
         const char *e = getenv("MOE_FF_PAIR");
-        return !e ? -1 : (e[0] == '1' ? 1 : (e[0] == '0' ? 0 : -1));
+        return e && e[0] == '1';
     }();
     return v;
 }
@@ -849,7 +851,7 @@ static cudaError_t launch_ffn(FfnArgs &a, const FfnMaps &maps, cudaStream_t s)
         configured.mark(dev);
     }
     const size_t smem = (size_t)a.x_units * FF_X_UNIT + (size_t)a.n_w_slots * a.w_slot_bytes + 1024;
-    if (a.n_w_slots < 2 || smem > FF_SMEM_LIMIT - 512)
+    if (a.n_w_slots < 2 || smem > FF_SMEM_LIMIT - 512 || (!PAIR && a.seg_rows != FF_SEG))
         return cudaErrorInvalidConfiguration;
     const int grid = PAIR ? ffn_grid() & ~1 : ffn_grid();
     return launch_pdl<PAIR ? 2 : 1>(ffn_fused_kernel<GATED, PAIR>, dim3(grid), dim3(FF_THREADS), smem, s, a,

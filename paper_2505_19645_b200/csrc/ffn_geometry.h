@@ -11,8 +11,8 @@ namespace moe {
 // Test hooks, read once per process.  MOE_FF_WIDE: 0 / 1 forces the ring geometry with segments of
 // 128 / 256 rows, -1 (unset) leaves the choice to segment_rows().
 int geometry_override();
-// From MOE_FF_PAIR: 0 / 1 forces the FFN kernels to run on single CTAs / on CTA pairs.
-int pair_override();
+// MOE_FF_PAIR: 1 runs the FFN kernels on CTA pairs in every call.
+bool pairs_forced();
 
 // Expected number of activated experts for T tokens (Eq. N(t): E(1 - (1 - K/E)^T)); the host
 // never sees the routing result, so it sizes rings and shared tiles from the expectation.
@@ -70,7 +70,8 @@ inline int shared_segment_rows(const moe_config_t &c, int T)
 // Whether the FFN kernels of a call run on CTA pairs: always in the contraction geometry (see the
 // top of the file), in the streaming one beyond 128 tokens.  There a pair's token entries are half
 // as large, so that three weight slots fit where a single CTA has two (96 KB of token ring for
-// segments of 128 rows).  Layer on single CTAs -> pairs: DeepSeek-V3 shape T = 256 3367 -> 3287 us,
+// segments of 128 rows; the kernels' single-CTA instances are built for the streaming geometry
+// alone).  Layer on single CTAs -> pairs, when both could be chosen: DeepSeek-V3 shape T = 256 3367 -> 3287 us,
 // T = 1024 3647 -> 3560, T = 2048 4075 -> 3944, T = 3072 4428 -> 4374; Mixtral shape T = 192
 // 488 -> 474, T = 384 537 -> 527; Qwen1.5 shape T = 192 to 640 within 1 %.  Up to 128 tokens the
 // token rows are a small part of what an SM loads, single CTAs have three slots too, and a pair
@@ -78,10 +79,7 @@ inline int shared_segment_rows(const moe_config_t &c, int T)
 // pairs; Mixtral shape T = 80 443 and 450).
 inline bool ffn_pairs(const moe_config_t &c, int T)
 {
-    if (segment_rows(c, T) > FF_SEG)
-        return true;
-    const int force = pair_override();
-    return force >= 0 ? force == 1 : T > FF_SEG;
+    return segment_rows(c, T) > FF_SEG || T > FF_SEG || pairs_forced();
 }
 
 // Ring geometry.  Streaming: two k boxes per weight slot (64 KB for a full tile: every row is

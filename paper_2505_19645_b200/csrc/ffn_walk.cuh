@@ -153,8 +153,12 @@ struct ItemWalk {
         if (already_synced)
             sync(false);
     }
-    // segments of a group of n rows (seg_rows is 128 or 256)
-    __device__ int n_segments(int n) const { return (n + a.seg_rows - 1) >> (a.seg_rows == SEG_TOKENS ? 7 : 8); }
+    // segments of a group of n rows (seg_rows is 128, or for pairs 256)
+    __device__ int n_segments(int n) const
+    {
+        const int wide = PAIR && a.seg_rows != SEG_TOKENS;
+        return (n + (SEG_TOKENS << wide) - 1) >> (7 + wide);
+    }
     __device__ void sync(bool wait)
     {
         if (wait)

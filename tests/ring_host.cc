@@ -42,9 +42,9 @@ bool mbar_wait(uint32_t, uint32_t, volatile int *, int32_t *);
 
 using namespace moe;
 
-static int g_wide = -1, g_pair = -1;
+static int g_wide = -1, g_pair = 0;
 int moe::geometry_override() { return g_wide; }
-int moe::pair_override() { return g_pair; }
+bool moe::pairs_forced() { return g_pair; }
 
 #define CHECK(cond)                                                                               \
     do {                                                                                          \
@@ -140,9 +140,11 @@ int main(int argc, char **argv)
                 moe_config_t c{};
                 c.n_experts = s[0], c.top_k = s[1], c.hidden = s[2], c.inter = s[3], c.shared_inter = s[4];
                 g_wide = trial % 4 < 2 ? -1 : trial % 4 - 2;
-                g_pair = trial % 3 == 2 ? 1 : -1;
+                g_pair = trial % 3 == 2;
                 FfnArgs a{};
                 ffn_geometry(c, T, a);
+                if (!ffn_pairs(c, T) && (a.seg_rows != FF_SEG || a.kboxes != 2 || a.acc_sets != 2))
+                    return printf("T=%d: not the geometry the single-CTA kernels are built for\n", T), 1;
                 ++rings[a.x_units];
                 if (ffn_pairs(c, T))
                     ++pairs, replay<true>(c, T, a, g);

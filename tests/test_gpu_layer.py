@@ -269,10 +269,16 @@ def test_grouping_and_gather_of_medium_batches(E, k, T):
 
 
 PAIR_CASES = [
-    ("pair-tile-edges", 288, 5, 2, 352, 1408, 150, 1),   # last tiles of 32 and 96 features, 2 shared segments
-    ("pair-few-rows", 160, 6, 3, 224, 96, 1, 5),         # groups of 1..6 rows: the second CTA's rows are all padding
-    ("pair-segments", 256, 2, 1, 544, 0, 259, 1),        # groups of about 259 rows: two segments, ragged tile ends
-    ("pair-half-box", 544, 4, 4, 96, 32, 33, 0),         # reductions that end in half a k box; 33 rows: 17 per CTA
+    # gate/up tiles of 256 and 96 features, a down tile of 288 (144 per CTA: blocks of 128 and 16), 300 shared rows
+    ("pair-tile-edges", 288, 5, 2, 352, 1408, 150, 1),
+    # groups of 1..6 rows: the second CTA's rows are all padding; tiles of 224 and 160 features
+    ("pair-few-rows", 160, 6, 3, 224, 96, 1, 5),
+    # groups of about 259 rows in two or three segments; gate/up tiles of 256, 256 and 32 features (16 per CTA)
+    ("pair-segments", 256, 2, 1, 544, 0, 259, 1),
+    # reductions that end in half a k box; groups of 33 rows: 32 in the first CTA, one in the second; down tiles 512 and 32
+    ("pair-half-box", 544, 4, 4, 96, 32, 33, 0),
+    # groups of 41 rows: the next group begins inside the second CTA's first 16-row piece; tiles of 256 and 32
+    ("pair-mid-piece", 96, 3, 3, 288, 0, 41, 0),
 ]
 
 
@@ -284,19 +290,19 @@ def test_cta_pair_case(name, H, E, k, I, Is, B, gamma):
 
 @pytest.mark.parametrize("wide", ["0", "1"])
 def test_layer_parity_on_cta_pairs(wide):
-    """The FFN kernels on CTA pairs (MOE_FF_PAIR, a test hook read once per process) in either
-    ring geometry, at the edges of their tiles and of the token halves."""
+    """The FFN kernels on CTA pairs in either ring geometry (MOE_FF_PAIR and MOE_FF_WIDE, test hooks
+    read once per process; 256-row segments always run on pairs), at the edges of their tiles and
+    of the token halves."""
     _run_child({"MOE_FF_PAIR": "1", "MOE_FF_WIDE": wide, "MOE_SMALL_FUSED": "0"},
                "cta_pair_case or scheduling_mode_case or test_layer_parity_small_shapes")
 
 
-@pytest.mark.parametrize("wide", ["0", "1"])
-def test_layer_parity_in_both_ring_geometries(wide):
+def test_layer_parity_with_short_segments_at_every_size():
     """The FFN kernels run with segments of up to 128 token rows (two k boxes per weight slot,
-    two sets of accumulators) or of up to 256 (one k box, one set); MOE_FF_WIDE (a test hook
-    read once per process) forces one of the two on every call, also where the host would
-    choose the other: the scheduling cases and a few small shapes in a child process each."""
-    _run_child({"MOE_FF_WIDE": wide},
+    two sets of accumulators) or of up to 256 (one k box, one set, on CTA pairs: the test above);
+    MOE_FF_WIDE=0 (a test hook read once per process) forces the former also where the host would
+    choose the other, up to 128 tokens on single CTAs: the scheduling cases and a few small shapes."""
+    _run_child({"MOE_FF_WIDE": "0"},
                "scheduling_mode_case or (small_shapes and (qwen-like or dense-contrast or "
                "ksplit-routed or ragged or e24-33tok or dsv3-like-zipf))")
 
