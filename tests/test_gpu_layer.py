@@ -164,11 +164,13 @@ def _share_not_the_rounding_of_the_exact_sum(shape, w, x, idx, out):
 FP32_SUMS_SHARE = 0.055
 
 
-@pytest.mark.parametrize("name,T", [("qwen1.5-moe-a2.7b", 3), ("mixtral-8x7b", 2), ("mixtral-8x7b", 4),
-                                    ("deepseek-v3", 4)])
-def test_few_tokens_keep_fp32_sums(name, T):
-    """Two to four tokens of the shapes without a very large shared expert: one launch, whose
-    projections are fp32 sums, not the tensor cores' accumulation."""
+# Expert outputs rounded to bf16 before the gate-weighted sum add an error of the size of the
+# output's own rounding: 41 % of the outputs then differ (measured on the chain, Qwen2 shape,
+# T = 2 to 4).  The bound is the geometric mean of that and of the 11.3 % above.
+FP32_OUTPUTS_SHARE = 0.215
+
+
+def _few_token_share(name, T):
     from paper_2505_19645_b200 import api
 
     shape = wl.CONFIGS[name]
@@ -177,9 +179,31 @@ def test_few_tokens_keep_fp32_sums(name, T):
     out, dbg = run_gpu_layer(shape, w, x, T, 0)
     launches = api.moe_last_launch_count()
     idx = torch.from_numpy(dbg["topk_idx"]).cuda().long().view(T, shape.top_k)
-    share = _share_not_the_rounding_of_the_exact_sum(shape, w, x, idx, out)
+    return _share_not_the_rounding_of_the_exact_sum(shape, w, x, idx, out), launches
+
+
+@pytest.mark.parametrize("name,T", [("qwen1.5-moe-a2.7b", 3), ("mixtral-8x7b", 2), ("mixtral-8x7b", 4),
+                                    ("deepseek-v3", 4)])
+def test_few_tokens_keep_fp32_sums(name, T):
+    """Two to four tokens of the shapes without a very large shared expert: one launch, whose
+    projections are fp32 sums, not the tensor cores' accumulation."""
+    share, launches = _few_token_share(name, T)
     assert share <= FP32_SUMS_SHARE, share
     assert launches == 1
+
+
+@pytest.mark.parametrize("name,T", [("qwen2-57b-a14b", 2), ("qwen2-57b-a14b", 4), ("mixtral-8x7b", 3),
+                                    ("deepseek-v3", 2)])
+def test_few_token_outputs_stay_fp32(name, T):
+    """Up to four tokens keep the expert outputs in fp32 up to the combine, on the kernel chain too
+    (the Qwen2 shape here, all of them in the child process below), where the routed and the
+    shared reduction are cut into planes of floats."""
+    share, _ = _few_token_share(name, T)
+    assert share <= FP32_OUTPUTS_SHARE, share
+
+
+def test_few_token_outputs_stay_fp32_on_the_kernel_chain():
+    _run_child({"MOE_SMALL_FUSED": "0"}, "test_few_token_outputs_stay_fp32 and not chain")
 
 
 def test_one_workspace_serves_calls_of_every_size_in_turn():
