@@ -460,8 +460,9 @@ moe_status_t moe_verify_layer(const moe_config_t *cfg, const moe_weights_t *w, c
     if (st != MOE_OK)
         return st;
     MOE_STAGE(MOE_STAGE_COMBINE,
-              launch_combine(*cfg, y, routed_parts, inv_perm, topk_w, ys, shared_parts, gated ? shared_scale : nullptr, T,
-                             static_cast<__nv_bfloat16 *>(out), s, f32_outputs(T)));
+              launch_combine(*cfg, y, routed_parts, inv_perm, topk_w, ys, shared_parts,
+                             gated ? shared_scale : nullptr, T, static_cast<__nv_bfloat16 *>(out), s,
+                             f32_outputs(T)));
     g_last_launches = launches;
 
     return copy_debug_out(*cfg, T, dbg, base, L, s);

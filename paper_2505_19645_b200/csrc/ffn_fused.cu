@@ -41,23 +41,23 @@
 // CTA pairs.  In the contraction geometry, and in the streaming one beyond 128 tokens
 // (ffn_pairs), a cluster of two CTAs works on a tile of twice the features with tcgen05
 // cta_group::2: each CTA loads its half of the weight rows and half of the token rows, the
-// tensor cores of both read both halves of the tokens, and each CTA's TMEM and epilogue get its half of the features for all tokens.  What bounds the contraction is
-// bytes: each SM is filled at no more than about 44 bytes per clock, a 256 x 256 tile of a single
-// CTA wants 64 at the full instruction rate and 256 x 160 wants 81; a pair's CTA wants 47 and 66.
-// The leader (even CTA) claims the work for both, its barriers count the bytes of both and its
-// commits release the slots of both.  Layer at the power cap, single CTAs -> pairs when this was
-// taken up, medians of three runs of either in turn: Qwen2 shape T = 1280 1300 -> 1266 us, Mixtral
-// shape T = 1280 1163 -> 1123.
+// tensor cores of both read both halves of the tokens, and each CTA's TMEM and epilogue get its
+// half of the features for all tokens.  What bounds the contraction is bytes: each SM is filled at
+// no more than about 44 bytes per clock, a 256 x 256 tile of a single CTA wants 64 at the full
+// instruction rate and 256 x 160 wants 81; a pair's CTA wants 47 and 66.  The leader (even CTA)
+// claims the work for both, its barriers count the bytes of both and its commits release the slots
+// of both.  Layer at the power cap, single CTAs -> pairs when this was taken up, medians of three
+// runs of either in turn: Qwen2 shape T = 1280 1300 -> 1266 us, Mixtral shape T = 1280 1163 -> 1123.
 //
 // CTA = 11 warps.  warp 0: weight producer, warp 1: MMA issuer (idle in a pair's second CTA) and
 // owner of the TMEM allocation, warp 2: token-operand producer (in all three the warp runs in
-// step and one elected lane issues), warps 3..10:
-// epilogue, two warps per TMEM lane quarter that take alternate 16-token chunks (tcgen05.ld,
-// SwiGLU, transposition, 16-byte bf16 stores): where no second set of accumulators exists the
-// epilogue is not hidden behind the next tile, and two warps per scheduler hide its latencies.  Rings and the
-// accumulator sets are handed over through mbarriers.  Every wait is bounded: when one
-// gives up it raises the CTA's abort flag and the device status word, all roles leave their
-// loops (the other CTA of a pair by its own limits), TMEM is freed and the kernel returns.
+// step and one elected lane issues), warps 3..10: epilogue, two warps per TMEM lane quarter that
+// take alternate 16-token chunks (tcgen05.ld, SwiGLU, transposition, 16-byte bf16 stores): where no
+// second set of accumulators exists the epilogue is not hidden behind the next tile, and two warps
+// per scheduler hide its latencies.  Rings and the accumulator sets are handed over through
+// mbarriers.  Every wait is bounded: when one gives up it raises the CTA's abort flag and the device
+// status word, all roles leave their loops (the other CTA of a pair by its own limits), TMEM is
+// freed and the kernel returns.
 //
 // Programmatic dependent launch: the kernels may start while their predecessor in the stream
 // is still running.  Work that depends only on the caller's inputs (shared-expert tiles in the
@@ -579,7 +579,7 @@ ffn_fused_kernel(const FfnArgs args, const __grid_constant__ FfnMaps maps)
     if (PAIR)
         cluster_barrier();  // nothing of the other CTA refers to this one's memory any more
     if (warp == 1) {
-        __syncwarp();  // lane 0 arrived from the issue loop: reconverge for the aligned dealloc
+        __syncwarp();  // the deallocation is warp-collective
         tc_fence_after();
         if (PAIR)
             asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),

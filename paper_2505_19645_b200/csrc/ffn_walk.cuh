@@ -93,6 +93,16 @@ struct ClaimRing {
     uint32_t peer_data, peer_full0, leader_empty0;
 };
 
+// Rows per segment of a group of n rows cut into nseg segments: equal shares rounded up to the
+// 16-row unit of the token boxes (never more than the segment limit, since nseg = ceil(n /
+// limit)).  Equal shares instead of "full segments and a remainder": the instruction time
+// follows the rows of a segment with a floor of about 64 rows, so 320 rows cost less as
+// 160 + 160 than as 256 + 64.
+__device__ __forceinline__ int balanced_segment_rows(int n, int nseg)
+{
+    return nseg == 1 ? (n + 15) & ~15 : (((n + nseg - 1) / nseg) + 15) & ~15;
+}
+
 // Walks the items of one worker, in every lane of the role's warp: its units of the shared expert
 // first (dealt round-robin: they depend on nothing the layer computes), then the routed items it
 // claims from a grid-wide counter, so that a worker that is late or slow simply takes less.  The
@@ -105,17 +115,7 @@ struct ClaimRing {
 // layer, ranges -> items, Qwen1.5 shape T = 77 180.2 -> 177.6 us, T = 128 189 -> 186, T = 192
 // 199.4 -> 195.1, Qwen2 shape T = 64 589.6 -> 586.9, Mixtral and DeepSeek-V3 shapes equal.  (Items of
 // half the tile height for the last round of every worker: 1-6 % slower.)
-
-// Rows per segment of a group of n rows cut into nseg segments: equal shares rounded up to the
-// 16-row unit of the token boxes (never more than the segment limit, since nseg = ceil(n /
-// limit)).  Equal shares instead of "full segments and a remainder": the instruction time
-// follows the rows of a segment with a floor of about 64 rows, so 320 rows cost less as
-// 160 + 160 than as 256 + 64.
-__device__ __forceinline__ int balanced_segment_rows(int n, int nseg)
-{
-    return nseg == 1 ? (n + 15) & ~15 : (((n + nseg - 1) / nseg) + 15) & ~15;
-}
-
+//
 // PAIR: the worker is a CTA pair that walks the items together, each CTA computing half of a
 // tile's features; row units are then 32 weight rows, so that the halves are whole 16-row units.
 template <bool PAIR>

@@ -209,7 +209,8 @@ cudaError_t launch_permute(const moe_config_t &c, const int32_t *idx, int T, int
 // smaller chunks, so that as many CTAs as the copy wants share it, each then copying its own
 // tokens' rows to their sorted places (a token's row is read once and written top_k times).  Two
 // launches had a boundary between two short kernels, and the gather read every row top_k times.
-// Bound by latencies (A / 4096 rounds of counting, the scans, one pass over the rows).  CTA b owns `tokens` tokens (at most PERM_THREADS assignments); the last CTA writes the tables.
+// Bound by latencies (A / 4096 rounds of counting, the scans, one pass over the rows).  CTA b owns
+// `tokens` tokens (at most PERM_THREADS assignments); the last CTA writes the tables.
 __global__ void __launch_bounds__(PERM_THREADS)
 group_gather_kernel(const int32_t *__restrict__ topk_idx, const __nv_bfloat16 *__restrict__ x, int T, int H,
                     int E, int k, int tokens, int32_t *__restrict__ counts, int32_t *__restrict__ offsets,
