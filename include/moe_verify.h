@@ -215,7 +215,8 @@ moe_status_t moe_combine(const moe_config_t *cfg, const void *y, const int32_t *
  * then the expert projections on the CUDA cores with the weights streamed once.  The SwiGLU
  * intermediate is rounded to bf16 there as everywhere.  Calls that use the same workspace must
  * not overlap on the GPU (as for every entry point); the device needs cooperative-launch
- * support, else the call takes the kernel sequence of the larger sizes. */
+ * support, else the call takes the kernel sequence of the larger sizes.
+ * A call of any size may be captured into a CUDA graph and replayed. */
 moe_status_t moe_verify_layer(const moe_config_t *cfg, const moe_weights_t *w, const void *x,
                               int32_t B, int32_t gamma, void *out, const moe_debug_out_t *dbg,
                               void *ws, size_t ws_bytes, void *stream);

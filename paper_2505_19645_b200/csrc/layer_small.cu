@@ -51,6 +51,7 @@ constexpr size_t LS_MAX_SLOT_BYTES = 160u << 10;
 constexpr uint64_t LS_WAIT_NS = 1000ull * 1000ull * 1000ull;
 constexpr int LS_SELFTEST_WORD = 4;  // int32 index there of the word the wait self-test waits on
 constexpr int LS_BARRIER_WORD = 8;  // int32 index of the grid barrier's word inside the status region
+constexpr int LS_SEQ_WORD = 10;     // ... and of the number of one-launch calls on the workspace
 constexpr size_t LS_UNIT_WORD_BYTES = 512;  // the units' counters lead the partial-logit region
 
 struct SmallArgs {
@@ -69,7 +70,8 @@ struct SmallArgs {
     __nv_bfloat16 *h_shared;  // [T, Is_pad]
     int I_pad, Is_pad;        // row pitches: whole 128-byte lines, so no line belongs to two units
     unsigned long long *barrier;    // (epoch << 32) | CTAs arrived
-    unsigned long long *unit_done;  // [LS_MAX_UNITS]: (epoch << 32) | CTAs done with the unit's gate/up
+    unsigned long long *unit_done;  // [LS_MAX_UNITS]: (tag << 32) | CTAs done with the unit's gate/up
+    uint32_t *seq;                  // one-launch calls on this workspace so far (starts anywhere)
     int32_t *status;
     uint32_t epoch;
     int wait_us;
@@ -228,21 +230,28 @@ __device__ __forceinline__ void down_item(const __nv_bfloat16 *wd, int ld, int f
 
 // ---- counters across the grid --------------------------------------------------------------------
 //
-// A 64-bit word: the call's epoch in the high half, a count in the low half.  The workspace need
+// A 64-bit word: a tag of the call in the high half, a count in the low half.  The workspace need
 // not be initialised and may hold the word of an earlier call (complete or abandoned): whoever
-// finds another epoch there replaces the word by (epoch, own count); counts that went to the stale
+// finds another tag there replaces the word by (tag, own count); counts that went to the stale
 // word meanwhile are repeated by their owners.
-__device__ __forceinline__ void tagged_add(unsigned long long *word, uint32_t epoch)
+//
+// A call captured into a graph is launched with the same arguments, the host's epoch among them, at
+// every replay.  The barrier's tag is the epoch: every launch counts `limit` arrivals in all, so a
+// word that has them belongs to an earlier launch of the same call.  The units' tag joins the epoch
+// with the workspace's sequence number, which the first CTA advances before it arrives at the
+// barrier and every CTA reads behind it (a unit's word may be left over from any earlier replay).
+__device__ __forceinline__ void tagged_add(unsigned long long *word, uint32_t tag, uint32_t limit = 0xffffffffu)
 {
-    // count first: all but the call's first few arrivals find the epoch in place
-    if ((uint32_t)(atomicAdd(word, 1ull) >> 32) == epoch)
+    auto current = [&](unsigned long long w) { return (uint32_t)(w >> 32) == tag && (uint32_t)w < limit; };
+    // count first: all but the call's first few arrivals find the tag in place
+    if (current(atomicAdd(word, 1ull)))
         return;
-    // the add went to a stale word: install (epoch, 1), or count again if somebody else has
-    // installed the epoch meanwhile (adds to the stale word are dropped with it)
-    const unsigned long long base = (unsigned long long)epoch << 32;
+    // the add went to a stale word: install (tag, 1), or count again if somebody else has
+    // installed the tag meanwhile (adds to the stale word are dropped with it)
+    const unsigned long long base = (unsigned long long)tag << 32;
     unsigned long long seen = *reinterpret_cast<volatile unsigned long long *>(word);
     for (;;) {
-        if ((uint32_t)(seen >> 32) == epoch) {
+        if (current(seen)) {
             atomicAdd(word, 1ull);
             return;
         }
@@ -253,12 +262,16 @@ __device__ __forceinline__ void tagged_add(unsigned long long *word, uint32_t ep
     }
 }
 
-// Bounded wait (one thread) until the word reads (epoch, target); acquire.  On giving up raises
+// (an odd factor: no two launches of one epoch share a tag, and the tags of calls of different
+// epochs meet only billions of calls apart)
+__device__ __forceinline__ uint32_t unit_tag(uint32_t epoch, uint32_t seq) { return seq * 0x9e3779b1u + epoch; }
+
+// Bounded wait (one thread) until the word reads (tag, target); acquire.  On giving up raises
 // the status word and returns false.
-__device__ __forceinline__ bool tagged_wait(const unsigned long long *word, uint32_t epoch,
+__device__ __forceinline__ bool tagged_wait(const unsigned long long *word, uint32_t tag,
                                             uint32_t target, int32_t *status, int wait_us)
 {
-    const unsigned long long want = ((unsigned long long)epoch << 32) + target;
+    const unsigned long long want = ((unsigned long long)tag << 32) + target;
     auto reached = [&]() {
         unsigned long long v;
         asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
@@ -325,6 +338,8 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
     __shared__ int s_unit_ready[LS_MAX_UNITS];  // a warp of the CTA has seen the unit's gate/up complete
     __shared__ int s_q_shared, s_q_routed, s_q_down;  // work queues
     __shared__ int s_n_groups;
+    __shared__ uint32_t s_tag;  // of the unit counters, known behind the grid barrier
+    __shared__ int s_tag_set;
     __shared__ int s_ok;     // the grid barrier was passed
     __shared__ int s_abort;  // a wait gave up: leave
 
@@ -340,12 +355,15 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
         s_q_shared = s_q_routed = s_q_down = 0;
         s_abort = 0;
         s_ok = 0;
+        s_tag_set = 0;
         s_unit_left[0] = owned_below(n_shared_items, b, G);
         for (int u = 0; u < LS_MAX_UNITS; ++u)
             s_unit_ready[u] = 0;
         if (b == 0)
             status_region_init(a.status);
     }
+    // (in flight through the logits)
+    const uint32_t seq0 = b == 0 && tid == 0 ? *reinterpret_cast<volatile uint32_t *>(a.seq) : 0u;
     __syncthreads();
 
     // Gate/up items of the shared expert, handed out to whichever warp asks.
@@ -377,7 +395,13 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
                 __threadfence();  // h before the count
                 if (atomicSub(&s_unit_left[0], 1) == 1) {
                     __threadfence();  // the other warps' h, seen through their counts
-                    tagged_add(a.unit_done + 0, a.epoch);
+                    // (the CTA's routing warps set the tag when they have passed or given up the
+                    // barrier, as a rule before the shared rows are done; the barrier's wait ends
+                    // within a second, this one by itself a little later)
+                    for (int i = 0; i < (1 << 24) && *reinterpret_cast<volatile int *>(&s_tag_set) == 0; ++i)
+                        __nanosleep(100);
+                    __threadfence_block();
+                    tagged_add(a.unit_done + 0, s_tag);
                 }
             }
         }
@@ -458,10 +482,18 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
     } else {
         constexpr int RT = LS_ROUTE_WARPS * 32;
         named_sync(1, LS_THREADS);  // every warp of the CTA has written its partial logits
+        uint32_t seq = 0;
         if (tid == 0) {
+            if (b == 0)
+                *reinterpret_cast<volatile uint32_t *>(a.seq) = seq0 + 1u;
             __threadfence();
-            tagged_add(a.barrier, a.epoch);
-            s_ok = tagged_wait(a.barrier, a.epoch, G, a.status, a.wait_us) ? 1 : 0;
+            tagged_add(a.barrier, a.epoch, G);
+            const bool ok = tagged_wait(a.barrier, a.epoch, G, a.status, a.wait_us);
+            s_ok = ok ? 1 : 0;
+            if (ok)
+                seq = *reinterpret_cast<volatile uint32_t *>(a.seq);
+            else
+                *reinterpret_cast<volatile int *>(&s_tag_set) = 1;
         }
         named_sync(2, RT);
         if (s_ok) {
@@ -502,6 +534,11 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
                             a.logits[idx] = v;
                     }
                 }
+            }
+            if (tid == 0) {  // (not before the logits: nothing waits for the sequence number yet)
+                s_tag = unit_tag(a.epoch, seq);
+                __threadfence_block();
+                *reinterpret_cast<volatile int *>(&s_tag_set) = 1;
             }
             if (a.gated && tid < T) {
                 const float *p = a.logit_part + (size_t)E * a.logit_chunks * LS_MAX_TOKENS + tid;
@@ -633,7 +670,7 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
                 __threadfence();
                 if (atomicSub(&s_unit_left[1 + g], 1) == 1) {
                     __threadfence();
-                    tagged_add(a.unit_done + 1 + g, a.epoch);
+                    tagged_add(a.unit_done + 1 + g, s_tag);
                 }
             }
         }
@@ -671,7 +708,7 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
                 int ok = 1;
                 if (lane == 0) {
                     if (*reinterpret_cast<volatile int *>(&s_unit_ready[unit]) == 0) {
-                        ok = tagged_wait(a.unit_done + unit, a.epoch, n_done, a.status, a.wait_us) ? 1 : 0;
+                        ok = tagged_wait(a.unit_done + unit, s_tag, n_done, a.status, a.wait_us) ? 1 : 0;
                         __threadfence_block();
                         if (ok)
                             *reinterpret_cast<volatile int *>(&s_unit_ready[unit]) = 1;
@@ -993,6 +1030,7 @@ cudaError_t launch_layer_small(const moe_config_t &c, const moe_weights_t &w, co
     a.h_shared = a.h + (size_t)T * c.top_k * a.I_pad;
     a.status = reinterpret_cast<int32_t *>(ws + L.status);
     a.barrier = reinterpret_cast<unsigned long long *>(a.status + LS_BARRIER_WORD);
+    a.seq = reinterpret_cast<uint32_t *>(a.status + LS_SEQ_WORD);
     a.epoch = epoch;
     a.wait_us = (int)(LS_WAIT_NS / 1000ull);
     a.logit_chunks = (c.hidden + LS_LOGIT_CHUNK - 1) / LS_LOGIT_CHUNK;

@@ -227,6 +227,40 @@ def test_one_workspace_serves_calls_of_every_size_in_turn():
     api.moe_check(ws)
 
 
+@pytest.mark.parametrize("T", [1, 2, 3, 4, 5, 40, 200, 700])
+def test_a_captured_call_is_replayed_like_a_new_one(T):
+    """A layer call captured into a CUDA graph: every replay, on new tokens in the same buffer and
+    between other calls on the same workspace, gives what a call on a fresh workspace gives.  (One
+    to four tokens: the one-launch kernel, whose counters carry the captured call's epoch each time.)"""
+    from paper_2505_19645_b200 import api
+
+    shape = wl.small_shape("graph", 512, 60, 4, 352, 1408, 0, 0, 1)
+    w = wl.make_weights(shape, 41, "cuda")
+    cfg, cw = api.make_config(shape), api.make_weights(w)
+    xs = [wl.make_tokens(shape, T, 50 + i, "cuda") for i in range(4)]
+    want = [run_gpu_layer(shape, w, x, T, 0)[0] for x in xs]
+    x, out, ws = xs[0].clone(), torch.empty_like(xs[0]), api.alloc_workspace(cfg, T)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        api.moe_verify_layer(cfg, cw, x, T, 0, out, ws)
+    s.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        api.moe_verify_layer(cfg, cw, x, T, 0, out, ws)
+    for i in (1, 2, 2, 3, 0):
+        x.copy_(xs[i])
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want[i]), i
+        if i == 3:  # a call of its own in between
+            other = torch.empty_like(out)
+            api.moe_verify_layer(cfg, cw, xs[1], T, 0, other, ws)
+            assert torch.equal(other, want[1])
+    api.moe_check(ws)
+
+
 def test_kernel_chain_on_the_same_few_tokens():
     """The same cases with the one-launch kernel switched off (a test hook read once per
     process, hence the child process)."""
