@@ -34,6 +34,8 @@ def test_no_hand_over_relies_on_less_than_it_waits_for(tmp_path):
     exe = _build(tmp_path / "walk_tsan", "walk_host.cc", "-fsanitize=thread")
     r = subprocess.run([exe, "2", "40"], capture_output=True, text=True, timeout=300,
                        env=dict(os.environ, TSAN_OPTIONS="halt_on_error=1"))
+    if "unexpected memory mapping" in r.stderr:
+        pytest.skip("the sanitizer run-time does not fit this kernel's address space")
     assert "data race" not in r.stderr, r.stderr[:3000]
     assert r.returncode == 0 and "walks agree" in r.stdout, r.stdout + r.stderr[-2000:]
 
