@@ -68,21 +68,29 @@ combine_kernel(const void *__restrict__ y, int routed_parts,
     griddep_launch();
     griddep_wait();  // y and shared_y come from the preceding kernel
     const int vec_per_row = H >> 3;
-    const size_t total = (size_t)T * vec_per_row;
     const size_t plane = (size_t)T * k * H;
-    for (size_t i = blockIdx.x * (size_t)CB_THREADS + threadIdx.x; i < total;
-         i += (size_t)gridDim.x * CB_THREADS) {
-        const int t = (int)(i / vec_per_row);
-        const int h = (int)(i - (size_t)t * vec_per_row) << 3;
-        // the k rows of this token: positions and weights first, then the row pieces of a
-        // plane, so that the loads of one level are in flight together
-        int rows[KP];
-        float wts[KP];
+    // A thread's pieces lie gridDim x CB_THREADS apart; their (token, column) advance by additions (no
+    // 64-bit division per piece), and the positions and weights of the next piece are requested while
+    // the rows of the current one are in flight.  Bound by loads in flight: 2 CTAs of 256 threads per SM with eight
+    // 16-byte row pieces each.  Alone, inputs larger than L2, us: DeepSeek-V3 shape T = 3072 96.3 -> 90.5
+    // (4.9 TB/s), T = 1024 36.5 -> 32.6, Qwen2 T = 1280 24.1 -> 22.0, Mixtral T = 1280 9.05 -> 7.77, Qwen1.5
+    // T = 640 4.18 -> 3.93, DeepSeek-V3 T = 128 equal; three CTAs per SM spill (128 us).
+    const unsigned step = gridDim.x * CB_THREADS, step_t = step / vec_per_row, step_v = step - step_t * vec_per_row;
+    const unsigned first = blockIdx.x * CB_THREADS + threadIdx.x;
+    int t = (int)(first / vec_per_row), v8 = (int)(first - (unsigned)t * vec_per_row);
+    int rows[KP];
+    float wts[KP];
+    auto fetch = [&](int tok) {
 #pragma unroll
         for (int j = 0; j < KP; ++j) {
-            rows[j] = j < k ? inv_perm[(size_t)t * k + j] : 0;
-            wts[j] = j < k ? topk_w[(size_t)t * k + j] : 0.f;
+            rows[j] = j < k ? inv_perm[(size_t)tok * k + j] : 0;
+            wts[j] = j < k ? topk_w[(size_t)tok * k + j] : 0.f;
         }
+    };
+    if (t < T)
+        fetch(t);
+    while (t < T) {
+        const int h = v8 << 3;
         const float s = shared_y && shared_scale ? shared_scale[t] : 1.0f;
         // the shared expert's planes, four at a time, requested before the routed rows are used
         Row8<F32> sv[4];
@@ -91,20 +99,32 @@ combine_kernel(const void *__restrict__ y, int routed_parts,
         for (int p = 0; p < 4; ++p)
             if (p < sp0)
                 sv[p].load(shared_y, ((size_t)p * T + t) * H + h);
-        float acc[8];
+        float acc[8], cur_w[KP];
+        const int cur_t = t;
 #pragma unroll
         for (int q = 0; q < 8; ++q)
             acc[q] = 0.f;
+#pragma unroll
+        for (int j = 0; j < KP; ++j)
+            cur_w[j] = wts[j];
+        t += (int)step_t;
+        v8 += (int)step_v;
+        if (v8 >= vec_per_row) {
+            v8 -= vec_per_row;
+            ++t;
+        }
         for (int part = 0; part < routed_parts; ++part) {
             Row8<F32> v[KP];
 #pragma unroll
             for (int j = 0; j < KP; ++j)
                 if (j < k)
                     v[j].load(y, (size_t)part * plane + (size_t)rows[j] * H + h);
+            if (part == routed_parts - 1 && t < T && t != cur_t)
+                fetch(t);
 #pragma unroll
             for (int j = 0; j < KP; ++j)
                 if (j < k)
-                    v[j].add(acc, wts[j]);
+                    v[j].add(acc, cur_w[j]);
         }
 #pragma unroll
         for (int p = 0; p < 4; ++p)
@@ -114,7 +134,7 @@ combine_kernel(const void *__restrict__ y, int routed_parts,
 #pragma unroll
             for (int p = 0; p < 4; ++p)
                 if (4 + p < shared_parts)
-                    sv[p].load(shared_y, ((size_t)(4 + p) * T + t) * H + h);
+                    sv[p].load(shared_y, ((size_t)(4 + p) * T + cur_t) * H + h);
 #pragma unroll
             for (int p = 0; p < 4; ++p)
                 if (4 + p < shared_parts)
@@ -130,7 +150,7 @@ combine_kernel(const void *__restrict__ y, int routed_parts,
         o.z = *reinterpret_cast<uint32_t *>(&p);
         p = __floats2bfloat162_rn(acc[6], acc[7]);
         o.w = *reinterpret_cast<uint32_t *>(&p);
-        *reinterpret_cast<uint4 *>(out + (size_t)t * H + h) = o;
+        *reinterpret_cast<uint4 *>(out + (size_t)cur_t * H + h) = o;
     }
 }
 
@@ -143,7 +163,9 @@ cudaError_t launch_combine(const moe_config_t &c, const __nv_bfloat16 *y, int ro
         return cudaErrorInvalidValue;
     const size_t total = (size_t)T * (c.hidden >> 3);
     size_t blocks = (total + CB_THREADS - 1) / CB_THREADS;
-    const size_t cap = (size_t)sm_count() * 8;
+    // as many CTAs as are resident at once (see the launch bounds): every thread has the same number of
+    // pieces or one less
+    const size_t cap = (size_t)sm_count() * (f32 ? 1 : c.top_k <= 2 ? 4 : c.top_k <= 4 ? 3 : c.top_k <= 8 ? 2 : 1);
     if (blocks > cap)
         blocks = cap;
 #define MOE_CB_LAUNCH(KP)                                                                        \
