@@ -322,7 +322,8 @@ __device__ __forceinline__ int pull(int *counter, int lane)
 
 // ---- the kernel -------------------------------------------------------------------------------
 
-template <int VPL>
+// VPL: logits per lane of the top-k
+template <int VPL, bool EVEN>
 __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallArgs a)
 {
     extern __shared__ __align__(16) float s_slot[];        // partial sums of the CTA's down items
@@ -678,13 +679,12 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
     }
 
     // ---- 4: down projection of the CTA's output features, unit by unit ------------------------
-    // Consecutive features, the same number for every CTA or one less.  Whole blocks of LS_DOWN_ROWS dealt in
-    // turn gave some CTAs a block more than others (Qwen1.5 shape: 4 or 3, 2048 / 148 = 13.8 features): one token
-    // 36.8 us, now 35.4; the other shapes within 0.3 %.  Where there is at most a block per CTA the blocks
-    // stay whole (tiny shape, four tokens: 22.5 us, 24.0 in pieces).
-    const bool few = H <= G * LS_DOWN_ROWS;
-    const int feat0 = few ? min(b * LS_DOWN_ROWS, H) : (int)((long long)b * H / G);
-    const int n_feat = (few ? min((b + 1) * LS_DOWN_ROWS, H) : (int)((long long)(b + 1) * H / G)) - feat0;
+    // Blocks of LS_DOWN_ROWS features are dealt to the CTAs in turn.  EVEN: every CTA owns consecutive features
+    // instead, the same number or one less, its last block a short one (see even_features()).
+    const int feat0 = EVEN ? (int)((long long)b * H / G) : 0;
+    const int n_feat = EVEN ? (int)((long long)(b + 1) * H / G) - feat0
+                            : owned_below(H / LS_DOWN_ROWS, b, G) * LS_DOWN_ROWS;
+    auto block_feature = [&](int k) { return EVEN ? feat0 + k * LS_DOWN_ROWS : (b + k * G) * LS_DOWN_ROWS; };
     const int my_blocks = (n_feat + LS_DOWN_ROWS - 1) / LS_DOWN_ROWS;
     const int n_uc = a.chunks_s + s_n_groups * a.chunks_r;  // (unit, column chunk) pairs
     {
@@ -697,7 +697,8 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
             if (item >= n_items)
                 break;
             const int uc = item / my_blocks, k = item - uc * my_blocks;
-            const int f0 = feat0 + k * LS_DOWN_ROWS, rows = min(LS_DOWN_ROWS, n_feat - k * LS_DOWN_ROWS);
+            const int f0 = block_feature(k);
+            const int rows = EVEN ? min(LS_DOWN_ROWS, n_feat - k * LS_DOWN_ROWS) : LS_DOWN_ROWS;
             int unit, c, n_done;
             if (uc < a.chunks_s) {
                 unit = 0;
@@ -776,28 +777,81 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
         return;
 
     // ---- 5: combine the CTA's features -----------------------------------------------------------
-    for (int idx = tid; idx < n_feat * T; idx += LS_THREADS) {
-        const int t = idx / n_feat, f = idx - t * n_feat;
-        const int k = f / LS_DOWN_ROWS, j = f - k * LS_DOWN_ROWS;
-        // the sum of a (unit, chunk) for this feature and the unit's row r
-        auto part = [&](int uc, int r) {
-            return s_slot[((size_t)uc * my_blocks + k) * LS_SLOT_FLOATS + j * LS_MAX_TOKENS + r];
-        };
-        float o = 0.f;
-        for (int slot_j = 0; slot_j < K; ++slot_j) {
-            const int asg = t * K + slot_j;
-            float y = 0.f;
-            for (int c = 0; c < a.chunks_r; ++c)
-                y += part(a.chunks_s + s_group_of[asg] * a.chunks_r + c, s_row_of[asg]);
-            o = fmaf(s_gate_w[asg], y, o);
+    if constexpr (EVEN) {
+        for (int idx = tid; idx < n_feat * T; idx += LS_THREADS) {
+            const int t = idx / n_feat, f = idx - t * n_feat;
+            const int k = f / LS_DOWN_ROWS, j = f - k * LS_DOWN_ROWS;
+            // the sum of a (unit, chunk) for this feature and the unit's row r
+            auto part = [&](int uc, int r) {
+                return s_slot[((size_t)uc * my_blocks + k) * LS_SLOT_FLOATS + j * LS_MAX_TOKENS + r];
+            };
+            float o = 0.f;
+            for (int slot_j = 0; slot_j < K; ++slot_j) {
+                const int asg = t * K + slot_j;
+                float y = 0.f;
+                for (int c = 0; c < a.chunks_r; ++c)
+                    y += part(a.chunks_s + s_group_of[asg] * a.chunks_r + c, s_row_of[asg]);
+                o = fmaf(s_gate_w[asg], y, o);
+            }
+            if (a.Is > 0) {
+                float y = 0.f;
+                for (int c = 0; c < a.chunks_s; ++c)
+                    y += part(c, t);
+                o = fmaf(a.gated ? s_shared_scale[t] : 1.0f, y, o);
+            }
+            a.out[(size_t)t * H + block_feature(k) + j] = __float2bfloat16_rn(o);
         }
-        if (a.Is > 0) {
-            float y = 0.f;
-            for (int c = 0; c < a.chunks_s; ++c)
-                y += part(c, t);
-            o = fmaf(a.gated ? s_shared_scale[t] : 1.0f, y, o);
+    } else {
+        for (int idx = tid; idx < my_blocks * T; idx += LS_THREADS) {
+            const int k = idx / T, t = idx - k * T;
+            const int f0 = (b + k * G) * LS_DOWN_ROWS;
+            float o[LS_DOWN_ROWS];
+#pragma unroll
+            for (int j = 0; j < LS_DOWN_ROWS; ++j)
+                o[j] = 0.f;
+            for (int slot_j = 0; slot_j < K; ++slot_j) {
+                const int asg = t * K + slot_j;
+                const int uc0 = a.chunks_s + s_group_of[asg] * a.chunks_r;
+                const int r = s_row_of[asg];
+                float y[LS_DOWN_ROWS];
+#pragma unroll
+                for (int j = 0; j < LS_DOWN_ROWS; ++j)
+                    y[j] = 0.f;
+                for (int c = 0; c < a.chunks_r; ++c) {
+                    const float *slot = s_slot + ((size_t)(uc0 + c) * my_blocks + k) * LS_SLOT_FLOATS;
+#pragma unroll
+                    for (int j = 0; j < LS_DOWN_ROWS; ++j)
+                        y[j] += slot[j * LS_MAX_TOKENS + r];
+                }
+                const float gw = s_gate_w[asg];
+#pragma unroll
+                for (int j = 0; j < LS_DOWN_ROWS; ++j)
+                    o[j] = fmaf(gw, y[j], o[j]);
+            }
+            if (a.Is > 0) {
+                float y[LS_DOWN_ROWS];
+#pragma unroll
+                for (int j = 0; j < LS_DOWN_ROWS; ++j)
+                    y[j] = 0.f;
+                for (int c = 0; c < a.chunks_s; ++c) {
+                    const float *slot = s_slot + ((size_t)c * my_blocks + k) * LS_SLOT_FLOATS;
+#pragma unroll
+                    for (int j = 0; j < LS_DOWN_ROWS; ++j)
+                        y[j] += slot[j * LS_MAX_TOKENS + t];
+                }
+                const float sc = a.gated ? s_shared_scale[t] : 1.0f;
+#pragma unroll
+                for (int j = 0; j < LS_DOWN_ROWS; ++j)
+                    o[j] = fmaf(sc, y[j], o[j]);
+            }
+            static_assert(LS_DOWN_ROWS == 4, "the store below writes two bf16 pairs");
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(o[0], o[1]);
+            const __nv_bfloat162 hi = __floats2bfloat162_rn(o[2], o[3]);
+            uint2 packed;
+            packed.x = *reinterpret_cast<const uint32_t *>(&lo);
+            packed.y = *reinterpret_cast<const uint32_t *>(&hi);
+            *reinterpret_cast<uint2 *>(a.out + (size_t)t * H + f0) = packed;
         }
-        a.out[(size_t)t * H + feat0 + f] = __float2bfloat16_rn(o);
     }
 }
 
@@ -933,7 +987,7 @@ bool layer_small_applies(const moe_config_t &c, int T)
     return small_shape(c, T) && small_layer_override() != 0 && cooperative_ok();
 }
 
-template <int VPL>
+template <int VPL, bool EVEN>
 static cudaError_t launch_variant(const SmallArgs &a, size_t smem, cudaStream_t s)
 {
     static DeviceOnce configured;
@@ -942,7 +996,7 @@ static cudaError_t launch_variant(const SmallArgs &a, size_t smem, cudaStream_t 
     if (err != cudaSuccess)
         return err;
     if (!configured.done(dev)) {
-        err = cudaFuncSetAttribute(layer_small_kernel<VPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        err = cudaFuncSetAttribute(layer_small_kernel<VPL, EVEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)LS_MAX_SLOT_BYTES);
         if (err != cudaSuccess)
             return err;
@@ -958,7 +1012,33 @@ static cudaError_t launch_variant(const SmallArgs &a, size_t smem, cudaStream_t 
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, layer_small_kernel<VPL>, a);
+    return cudaLaunchKernelEx(&cfg, layer_small_kernel<VPL, EVEN>, a);
+}
+
+// Whether the CTAs share the output features evenly instead of in whole blocks.  With a handful of blocks
+// per CTA those with one more are the last to finish (Qwen1.5 shape: 4 or 3 for 2048 / 148 = 13.8 features); one
+// token 36.8 -> 35.4 us per call.  More tokens make the short blocks' idle rows cost what they level (two tokens
+// equal, four 75.0 -> 75.8); from six blocks on there is less to level (Qwen2 shape, 6.05 blocks: equal; DeepSeek-V3
+// shape, 12.1, four tokens: 447 -> 451), and up to one block per CTA nothing.
+constexpr int LS_EVEN_BLOCKS = 6;
+static bool even_features(const moe_config_t &c, int T)
+{
+    const int blocks = c.hidden / LS_DOWN_ROWS;
+    return T == 1 && blocks > sm_count() && blocks < LS_EVEN_BLOCKS * sm_count();
+}
+
+template <bool EVEN>
+static cudaError_t launch_even(const SmallArgs &a, int E, size_t smem, cudaStream_t s)
+{
+    if (E <= 32)
+        return launch_variant<1, EVEN>(a, smem, s);
+    if (E <= 64)
+        return launch_variant<2, EVEN>(a, smem, s);
+    if (E <= 128)
+        return launch_variant<4, EVEN>(a, smem, s);
+    if (E <= 256)
+        return launch_variant<8, EVEN>(a, smem, s);
+    return launch_variant<16, EVEN>(a, smem, s);
 }
 
 cudaError_t launch_layer_small(const moe_config_t &c, const moe_weights_t &w, const __nv_bfloat16 *x,
@@ -1021,15 +1101,7 @@ cudaError_t launch_layer_small(const moe_config_t &c, const moe_weights_t &w, co
     a.chunk_s = down_chunk_cols(c, c.shared_inter);
     const size_t smem = slot_bytes(c, T);
     const int E = c.n_experts;
-    if (E <= 32)
-        return launch_variant<1>(a, smem, s);
-    if (E <= 64)
-        return launch_variant<2>(a, smem, s);
-    if (E <= 128)
-        return launch_variant<4>(a, smem, s);
-    if (E <= 256)
-        return launch_variant<8>(a, smem, s);
-    return launch_variant<16>(a, smem, s);
+    return even_features(c, T) ? launch_even<true>(a, E, smem, s) : launch_even<false>(a, E, smem, s);
 }
 
 }  // namespace moe
