@@ -175,7 +175,7 @@ moe_status_t run_ffn(const moe_config_t &c, const moe_weights_t &w, const __nv_b
                      const int32_t *offsets, const int32_t *perm, __nv_bfloat16 *y,
                      __nv_bfloat16 *shared_y, char *ws, const Workspace &L, cudaStream_t s,
                      int &launches, bool plan_ready, int shared_parts, int routed_parts,
-                     bool gathered, bool f32_out)
+                     bool gathered, bool f32_out, const int32_t *inv_perm)
 {
     const bool with_shared = shared_y != nullptr && c.shared_inter > 0;
     const PlanView plan = plan_view(ws, L, ffn_segment_rows(c, T));
@@ -185,7 +185,9 @@ moe_status_t run_ffn(const moe_config_t &c, const moe_weights_t &w, const __nv_b
     __nv_bfloat16 *xs = reinterpret_cast<__nv_bfloat16 *>(ws + L.x_sorted);
     if (!plan_ready)
         MOE_STAGE(MOE_STAGE_PLAN, launch_plan(c, T, offsets, status, plan, s));
-    if (!gathered)
+    if (!gathered && inv_perm != nullptr)
+        MOE_STAGE(MOE_STAGE_GATHER, launch_gather_tokens(c, x, inv_perm, T, xs, s));
+    else if (!gathered)
         MOE_STAGE(MOE_STAGE_GATHER, launch_gather_rows(c, x, perm, T, xs, s));
     MOE_STAGE(MOE_STAGE_GATE_UP,
               launch_ffn_gateup(c, w, x, xs, T, plan, with_shared, h, hs, status, s));
@@ -456,7 +458,7 @@ moe_status_t moe_verify_layer(const moe_config_t *cfg, const moe_weights_t *w, c
     const int shared_parts = has_shared ? shared_down_parts(*cfg) : 1;
     const int routed_parts = routed_down_parts(*cfg, T);
     st = run_ffn(*cfg, *w, xb, T, offsets, perm, y, ys, base, L, s, launches, true, shared_parts,
-                 routed_parts, small || grouped, f32_outputs(T));
+                 routed_parts, small || grouped, f32_outputs(T), inv_perm);
     if (st != MOE_OK)
         return st;
     MOE_STAGE(MOE_STAGE_COMBINE,

@@ -235,6 +235,9 @@ cudaError_t launch_tagged_wait_selftest(int32_t *status, int limit_us, cudaStrea
 // token rows in sorted order (the token operand of the routed gate/up tiles)
 cudaError_t launch_gather_rows(const moe_config_t &c, const __nv_bfloat16 *x, const int32_t *perm,
                                int T, __nv_bfloat16 *x_sorted, cudaStream_t s);
+// the same with the inverse permutation (a layer call's)
+cudaError_t launch_gather_tokens(const moe_config_t &c, const __nv_bfloat16 *x, const int32_t *inv_perm, int T,
+                                 __nv_bfloat16 *x_sorted, cudaStream_t s);
 // y and shared_y may hold `routed_parts` / `shared_parts` partial planes ([A,H] / [T,H]: k
 // chunks of the down pass), summed here; f32: they hold floats
 cudaError_t launch_combine(const moe_config_t &c, const __nv_bfloat16 *y, int routed_parts,
@@ -272,7 +275,8 @@ moe_status_t run_ffn(const moe_config_t &c, const moe_weights_t &w, const __nv_b
                      const int32_t *offsets, const int32_t *perm, __nv_bfloat16 *y,
                      __nv_bfloat16 *shared_y, char *ws, const Workspace &L, cudaStream_t s,
                      int &launches, bool plan_ready = false, int shared_parts = 1,
-                     int routed_parts = 1, bool gathered = false, bool f32_out = false);
+                     int routed_parts = 1, bool gathered = false, bool f32_out = false,
+                     const int32_t *inv_perm = nullptr);
 
 // ---------------------------------------------------------------------------------------
 // Device helpers.
