@@ -138,7 +138,8 @@ static void trial(Rng &rng)
     const bool down = rng.in(0, 1);
     FfnArgs a{};
     a.seg_rows = PAIR && rng.in(0, 1) ? 256 : 128;
-    a.max_tile = down ? 256 : 128;
+    const int full = down ? 256 : 128;  // rows of a full tile; the routed ones may be lower
+    a.max_tile = down ? rng.pick({64, 128, 256}) : rng.pick({64, 128});
     a.rows[0] = rng.pick({32, 96, 224, 288, 544, 1088});
     a.rows[1] = down ? a.rows[0] : rng.pick({32, 96, 704, 1408});
     a.K[0] = rng.pick({32, 96, 512, 1056});
@@ -155,9 +156,9 @@ static void trial(Rng &rng)
     a.routed_part_stride = 1000000;
     a.shared_part_stride = 10000000;
     a.shared_seg = a.T > 64 && a.T <= 128 && rng.in(0, 1) ? 64 : a.seg_rows;
-    const int most = a.max_tile >> 4;  // units per tile at most
+    const int most[2] = {a.max_tile >> 4, full >> 4};  // units per routed and per shared tile at most
     const int s_units = a.rows[1] / UNIT;
-    a.shared_tiles = a.with_shared ? rng.in((s_units + most - 1) / most, s_units) : 0;
+    a.shared_tiles = a.with_shared ? rng.in((s_units + most[1] - 1) / most[1], s_units) : 0;
 
     std::vector<int> groups;
     for (int i = rng.in(1, 7); i > 0; --i)
@@ -241,7 +242,7 @@ static void trial(Rng &rng)
     std::set<std::tuple<int, int, int, int, int>> seen;
     for (const Item &it : all) {
         const int g = it.grp, chunk = g ? a.shared_kchunk : a.routed_kchunk;
-        CHECK(it.h > 0 && it.h % UNIT == 0 && it.f0 % UNIT == 0 && it.h <= most * UNIT);
+        CHECK(it.h > 0 && it.h % UNIT == 0 && it.f0 % UNIT == 0 && it.h <= most[g] * UNIT);
         CHECK(it.f0 + it.h <= a.rows[g]);
         CHECK(it.k0 % 128 == 0 && it.k0 < it.k1 && it.k1 == min(a.K[g], it.k0 + chunk));
         const int part = it.k0 / chunk;
