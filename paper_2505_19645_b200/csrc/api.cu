@@ -190,7 +190,7 @@ moe_status_t run_ffn(const moe_config_t &c, const moe_weights_t &w, const __nv_b
     else if (!gathered)
         MOE_STAGE(MOE_STAGE_GATHER, launch_gather_rows(c, x, perm, T, xs, s));
     MOE_STAGE(MOE_STAGE_GATE_UP,
-              launch_ffn_gateup(c, w, x, xs, T, plan, with_shared, h, hs, status, s));
+              launch_ffn_gateup(c, w, x, xs, T, plan, with_shared, routed_parts, h, hs, status, s));
     MOE_STAGE(MOE_STAGE_DOWN,
               launch_ffn_down(c, w, T, plan, with_shared, h, hs, y, shared_y, shared_parts,
                               routed_parts, f32_out, status, s));

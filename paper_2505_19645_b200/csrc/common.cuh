@@ -203,8 +203,8 @@ cudaError_t launch_plan(const moe_config_t &c, int T, const int32_t *offsets, in
 // down projection  -> y[row,:] and y_shared[t,:]
 cudaError_t launch_ffn_gateup(const moe_config_t &c, const moe_weights_t &w, const __nv_bfloat16 *x,
                               const __nv_bfloat16 *x_sorted, int T, PlanView plan, bool with_shared,
-                              __nv_bfloat16 *h, __nv_bfloat16 *h_shared, int32_t *status,
-                              cudaStream_t s);
+                              int routed_parts, __nv_bfloat16 *h, __nv_bfloat16 *h_shared,
+                              int32_t *status, cudaStream_t s);
 cudaError_t launch_ffn_down(const moe_config_t &c, const moe_weights_t &w, int T, PlanView plan,
                             bool with_shared, const __nv_bfloat16 *h, const __nv_bfloat16 *h_shared,
                             __nv_bfloat16 *y, __nv_bfloat16 *y_shared, int shared_parts,

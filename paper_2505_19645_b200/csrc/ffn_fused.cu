@@ -843,18 +843,6 @@ bool pairs_forced()
 
 int ffn_segment_rows(const moe_config_t &c, int T) { return segment_rows(c, T); }
 
-static int ffn_grid() { return sm_count(); }
-
-// What pulls work items: a CTA, or a pair of CTAs whose tiles are twice as high.
-struct FfnWorkers {
-    int ctas, count;
-};
-static FfnWorkers ffn_workers(const moe_config_t &c, int T)
-{
-    const int ctas = ffn_pairs(c, T) ? 2 : 1;
-    return FfnWorkers{ctas, ffn_grid() / ctas};
-}
-
 // Number of tiles the shared expert's rows are cut into.  The shared expert's work units are
 // (tile, k chunk, segment); a unit should cost about the expected per-CTA share of the whole
 // pass (or less), with the tile height within [min_tile, max_tile] rows (a weight block
@@ -877,25 +865,6 @@ static int shared_tile_count(const moe_config_t &c, int T, int rows_routed, int 
     if (tu > (max_tile >> 4))
         tu = max_tile >> 4;
     return (units + tu - 1) / tu;
-}
-
-// Weight rows of a routed tile per CTA.  Full height (128 features with their gate and up rows, or 256
-// down rows) streams best, but where that gives fewer items than workers, SMs stand idle while others
-// pull a whole tile at what a single SM takes in (about 65 GB/s: four microseconds for 256 x 512).
-// The height is halved, down to FF_MIN_TILE, while the items still fit the workers at once.
-// Tiny shape, full height -> this, us per call: T = 5 19.5 -> 18.7, 8 20.7 -> 19.4, 16 20.1 -> 19.2,
-// 32 22.3 -> 21.4, 64 24.0 -> 23.2, 128 25.6 -> 24.1, 192 to 640 equal; with 32 rows at least T = 16 21.8 and
-// T = 640 37.0 against 32.5, with 16 22.7 and 38.4 (an item's fixed costs, boxes of 2 to 4 KB).
-constexpr int FF_MIN_TILE = 64;
-static int routed_tile_rows(const moe_config_t &c, int T, int rows, int ksplit, int full)
-{
-    const FfnWorkers wk = ffn_workers(c, T);
-    const double n_act = expected_active_experts(c.n_experts, c.top_k, T);
-    const double segs = ceil(n_act) * ceil((double)T * c.top_k / n_act / segment_rows(c, T));
-    int h = full;
-    while (h > FF_MIN_TILE && segs * ksplit * ((rows + h / 2 * wk.ctas - 1) / (h / 2 * wk.ctas)) <= wk.count)
-        h /= 2;
-    return h;
 }
 
 template <bool GATED, bool PAIR>
@@ -924,15 +893,15 @@ static cudaError_t launch_ffn(FfnArgs &a, const FfnMaps &maps, cudaStream_t s)
 
 cudaError_t launch_ffn_gateup(const moe_config_t &c, const moe_weights_t &w, const __nv_bfloat16 *x,
                               const __nv_bfloat16 *x_sorted, int T, PlanView plan, bool with_shared,
-                              __nv_bfloat16 *h, __nv_bfloat16 *h_shared, int32_t *status,
-                              cudaStream_t s)
+                              int routed_parts, __nv_bfloat16 *h, __nv_bfloat16 *h_shared,
+                              int32_t *status, cudaStream_t s)
 {
     const uint64_t A = (uint64_t)T * c.top_k, H = c.hidden, E = c.n_experts;
     FfnArgs a{};
     a.rows[0] = c.inter;
     a.rows[1] = c.shared_inter;
     a.K[0] = a.K[1] = c.hidden;
-    a.max_tile = routed_tile_rows(c, T, c.inter, 1, 128);
+    a.max_tile = routed_tile_rows(c, T, routed_parts).up;
     a.shared_ksplit = 1;
     a.shared_kchunk = (c.hidden + 127) / 128 * 128;
     a.shared_tiles = with_shared ? shared_tile_count(c, T, c.inter, c.shared_inter, c.hidden, c.hidden,
@@ -1049,7 +1018,7 @@ cudaError_t launch_ffn_down(const moe_config_t &c, const moe_weights_t &w, int T
     a.rows[0] = a.rows[1] = c.hidden;
     a.K[0] = c.inter;
     a.K[1] = c.shared_inter;
-    a.max_tile = routed_tile_rows(c, T, c.hidden, routed_parts, 256);
+    a.max_tile = routed_tile_rows(c, T, routed_parts).down;
     a.shared_ksplit = with_shared ? shared_parts : 1;
     a.shared_kchunk = with_shared ? split_chunk(c.shared_inter, a.shared_ksplit) : 128;
     a.shared_part_stride = (long long)T * c.hidden;

@@ -45,8 +45,8 @@ struct FfnArgs {
     int shared_tiles;  // tiles of the shared expert's rows; (tile, k chunk, segment) units are dealt
                        // round-robin to the CTAs; the first (units % tiles) tiles have one
                        // 16-row unit more
-    int max_tile;      // most weight rows of a routed tile per CTA: 128 or 64 (gate + up stacked), 256,
-                       // 128 or 64 (down), see routed_tile_rows(); the shared expert's tiles follow from
+    int max_tile;      // most weight rows of a routed tile per CTA: 128 or 64 (gate + up stacked), 256
+                       // or 128 (down), see routed_tile_rows(); the shared expert's tiles follow from
                        // shared_tiles and may be higher
     int kboxes;        // 64-element k boxes per weight slot
     int w_slot_bytes;  // capacity of a weight slot

@@ -43,6 +43,7 @@ bool mbar_wait(uint32_t, uint32_t, volatile int *, int32_t *);
 using namespace moe;
 
 static int g_wide = -1, g_pair = 0;
+int moe::sm_count() { return 148; }
 int moe::geometry_override() { return g_wide; }
 bool moe::pairs_forced() { return g_pair; }
 

@@ -139,7 +139,7 @@ static void trial(Rng &rng)
     FfnArgs a{};
     a.seg_rows = PAIR && rng.in(0, 1) ? 256 : 128;
     const int full = down ? 256 : 128;  // rows of a full tile; the routed ones may be lower
-    a.max_tile = down ? rng.pick({64, 128, 256}) : rng.pick({64, 128});
+    a.max_tile = rng.pick({full / 2, full});
     a.rows[0] = rng.pick({32, 96, 224, 288, 544, 1088});
     a.rows[1] = down ? a.rows[0] : rng.pick({32, 96, 704, 1408});
     a.K[0] = rng.pick({32, 96, 512, 1056});
