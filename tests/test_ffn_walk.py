@@ -6,6 +6,7 @@ less than the synchronisation that stands between them.  ring_host.cc: the token
 slots and the k-step barriers in every geometry the host's rule gives.  tile_host.cc: the tile heights
 the host gives the GPU tests' cases and others."""
 import os
+import random
 import subprocess
 
 import pytest
@@ -62,6 +63,62 @@ def _tiles(exe, calls):
         cut = lambda rows, h: [min(h * ctas, rows - f) // ctas for f in range(0, rows, h * ctas)]  # noqa: E731
         out.append((ctas, cut(I, up), cut(H, down)))
     return out
+
+
+# rows per CTA of the gate/up and the down tiles of the fixed cases of test_gpu_layer.py, on pairs in
+# either ring geometry
+PAIR_TILES = {
+    "pair-tile-edges": ([64, 64, 48], [128, 16]),
+    "pair-few-rows": ([64, 48], [80]),
+    "pair-segments": ([64, 64, 64, 64, 16], [128]),
+    "pair-half-box": ([48], [128, 128, 16]),
+    "pair-mid-piece": ([64, 64, 16], [48]),
+    "pair-tile-edges-full": ([128, 48], [144]),
+    "pair-few-rows-full": ([112], [80]),
+    "pair-segments-full": ([128, 128, 16], [128]),
+    "pair-half-box-full": ([48], [256, 256, 16]),
+    "pair-mid-piece-full": ([128, 128, 16], [48]),
+    "rr-segments": ([64, 64, 64], [128]),
+    "rr-ragged": ([64, 48], [80]),
+    "rr-segments-full": ([128, 64], [128]),
+    "rr-ragged-full": ([112], [80]),
+    "rr-blocks-full": ([128, 48], [208]),
+}
+# the same on single CTAs (calls of up to 128 tokens, the host's own choice)
+SINGLE_TILES = {
+    "rr-ragged": ([64, 64, 64, 32], [128, 32]),
+    "rr-ragged-full": ([128, 96], [160]),
+    "rr-blocks-full": ([128, 128, 96], [256, 160]),
+}
+
+
+def test_gpu_cases_run_at_the_tile_heights_they_name(tmp_path):
+    """The height of a routed tile follows from the number of items, so a case reaches an edge of a
+    full-height tile, or of a cut one, only at the right number of groups."""
+    from test_gpu_idle_tiles import IDLE_TILE_CASES
+    from test_gpu_layer import PAIR_CASES, SCHEDULING_CASES
+    from test_gpu_random_shapes import FULL_TILE_CASES, draw_full_tile_case
+
+    exe = _build(tmp_path / "tile", "tile_host.cc")
+    cases = {n: (H, E, k, I, Is, B * (g + 1)) for n, H, E, k, I, Is, B, g in PAIR_CASES + SCHEDULING_CASES}
+    for wide in (0, 1):
+        got = _tiles(exe, [cases[n] + (wide, 1) for n in PAIR_TILES])
+        assert {n: (2, *t) for n, t in PAIR_TILES.items()} == dict(zip(PAIR_TILES, got))
+    got = _tiles(exe, [cases[n] + (-1, 0) for n in SINGLE_TILES])
+    assert {n: (1, *t) for n, t in SINGLE_TILES.items()} == dict(zip(SINGLE_TILES, got))
+
+    # low tiles in both passes, in one of them
+    idle = _tiles(exe, [c + (-1, 0) for c in IDLE_TILE_CASES if c[3] < 2048])
+    assert all(max(up) <= 64 and max(down) <= 128 for _, up, down in idle[:-2])
+    assert idle[-2:] == [(1, [128, 32], [128] * 4 + [32]), (2, [48], [256, 144])]
+
+    # full tiles of the random shapes: ragged second down blocks, ragged gate/up tiles
+    rng = random.Random(15)
+    full = _tiles(exe, [draw_full_tile_case(rng) + (-1, 0) for _ in range(FULL_TILE_CASES)])
+    second = [ctas for ctas, _, down in full if any(128 < h < 256 for h in down)]
+    partial = [ctas for ctas, up, _ in full if any(64 < h < 128 for h in up)]
+    assert len(second) >= 40 and second.count(2) >= 10, (len(second), second.count(2))
+    assert len(partial) >= 40 and partial.count(2) >= 10, (len(partial), partial.count(2))
 
 
 # (H, E, k, I, Is, T): rows per CTA of a tile in the two passes, where full height and low tiles were

@@ -52,10 +52,16 @@ def test_layer_parity_small_shapes(name, H, E, k, I, Is, score, renorm, sgate, B
     check_layer_against_oracle(shape, w, x, B, gamma)
 
 
+# (The tile heights of these cases and of PAIR_CASES below, which follow from the number of items:
+# test_ffn_walk.py.)
 SCHEDULING_CASES = [
     ("rr-shared", 512, 60, 4, 352, 1408, 13, 4),     # shared expert with a k-split down pass
     ("rr-segments", 256, 4, 2, 384, 256, 100, 3),    # 200 rows per expert: segment pairs, 4 shared segments
-    ("rr-ragged", 160, 6, 3, 224, 96, 11, 6),        # tiles shorter than a box, k tails
+    ("rr-ragged", 160, 6, 3, 224, 96, 11, 6),        # low tiles, tiles shorter than a box, k tails
+    # the same rows per group and edges with enough items for tiles of full height
+    ("rr-segments-full", 256, 40, 16, 384, 256, 100, 4),
+    ("rr-ragged-full", 160, 100, 16, 224, 96, 11, 6),   # a down tile of 160: blocks of 128 and 32
+    ("rr-blocks-full", 416, 60, 4, 352, 0, 40, 0),      # down tiles of 256 and 160, single CTAs
 ]
 
 
@@ -327,16 +333,28 @@ def test_grouping_and_gather_of_medium_batches(E, k, T):
 
 
 PAIR_CASES = [
-    # gate/up tiles of 256 and 96 features, a down tile of 288 (144 per CTA: blocks of 128 and 16), 300 shared rows
+    # few items, low tiles (64 and 128 rows per CTA): a last gate/up tile of 48 and down tile of 16, 300
+    # shared rows
     ("pair-tile-edges", 288, 5, 2, 352, 1408, 150, 1),
-    # groups of 1..6 rows: the second CTA's rows are all padding; tiles of 224 and 160 features
+    # groups of 1..6 rows: the second CTA's rows are all padding; gate/up tiles of 128 and 96 features
     ("pair-few-rows", 160, 6, 3, 224, 96, 1, 5),
-    # groups of about 259 rows in two or three segments; gate/up tiles of 256, 256 and 32 features (16 per CTA)
+    # groups of about 259 rows in two or three segments; a last gate/up tile of 16 rows per CTA
     ("pair-segments", 256, 2, 1, 544, 0, 259, 1),
-    # reductions that end in half a k box; groups of 33 rows: 32 in the first CTA, one in the second; down tiles 512 and 32
+    # reductions that end in half a k box; groups of 33 rows: 32 in the first CTA, one in the second
     ("pair-half-box", 544, 4, 4, 96, 32, 33, 0),
-    # groups of 41 rows: the next group begins inside the second CTA's first 16-row piece; tiles of 256 and 32
+    # groups of 41 rows: the next group begins inside the second CTA's first 16-row piece
     ("pair-mid-piece", 96, 3, 3, 288, 0, 41, 0),
+    # the same edges with enough items for tiles of full height.  Gate/up tiles of 256 and 96 features, a
+    # down tile of 288 (144 per CTA: blocks of 128 and 16), 60 rows per group, 300 shared rows
+    ("pair-tile-edges-full", 288, 40, 8, 352, 1408, 150, 1),
+    # groups of one to a few rows, gate/up tiles of 224 features, down tiles of 160
+    ("pair-few-rows-full", 160, 64, 10, 224, 96, 1, 5),
+    # groups of about 259 rows; gate/up tiles of 256, 256 and 32 features (16 per CTA), down tiles of 256
+    ("pair-segments-full", 256, 20, 4, 544, 0, 259, 4),
+    # groups of 33 rows; down tiles of 512, 512 and 32
+    ("pair-half-box-full", 1056, 16, 16, 96, 32, 33, 0),
+    # groups of 41 rows; gate/up tiles of 256, 256 and 32
+    ("pair-mid-piece-full", 96, 16, 16, 544, 0, 41, 0),
 ]
 
 

@@ -56,6 +56,37 @@ def test_random_shapes_match_the_oracle(seed):
             raise AssertionError("case %d (%s): %s" % (n, name, e)) from e
 
 
+FULL_TILE_CASES = 80
+
+
+def draw_full_tile_case(rng):
+    """A layer with more (group, tile) items than SMs, whose weight tiles keep their full height (most
+    of the shapes above have so few items that their tiles are cut), with ragged last tiles."""
+    while True:
+        H = 32 * rng.choice([5, 6, 7, 9, 12, 13, 14, 15, 22])
+        E = rng.choice([80, 100, 160, 256])
+        k = rng.choice([2, 3, 4, 8, 16])
+        I = 32 * rng.choice([3, 5, 6, 7, 7, 11, 14, 16])
+        Is = 32 * rng.choice([0, 1, 4, 13])
+        T = rng.choice([33, 64, 65, 96, 128, 129, 200, 257, rng.randint(30, 400)])
+        if T * k >= 2 * E and T * k * I * H <= 400_000_000:
+            return H, E, k, I, Is, T
+
+
+def test_random_shapes_with_full_tiles():
+    rng = random.Random(15)
+    for n in range(FULL_TILE_CASES):
+        H, E, k, I, Is, T = draw_full_tile_case(rng)
+        name = "full-H%d-E%d-k%d-I%d-Is%d-T%d" % (H, E, k, I, Is, T)
+        shape = wl.small_shape(name, H, E, k, I, Is, 0, 1, 1 if Is else 0)
+        w = wl.make_weights(shape, 16000 + n, "cuda")
+        x = wl.make_tokens(shape, T, 17000 + n, "cuda")
+        try:
+            check_layer_against_oracle(shape, w, x, T, 0)
+        except AssertionError as e:
+            raise AssertionError("case %d (%s): %s" % (n, name, e)) from e
+
+
 def test_random_shapes_of_a_few_tokens():
     """One to four tokens: the one-launch kernel (where T * top_k <= 32, else the kernel chain),
     with intermediate sizes that cut the down projection into one to three column chunks."""
