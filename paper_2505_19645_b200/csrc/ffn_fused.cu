@@ -689,7 +689,7 @@ cudaError_t launch_gather_tokens(const moe_config_t &c, const __nv_bfloat16 *x, 
 {
     const int vec = c.hidden >> 3, pieces = (vec + 32 * GATHER_UNROLL - 1) / (32 * GATHER_UNROLL);
     size_t blocks = ((size_t)T * pieces + 7) / 8;  // a piece of a row per warp, eight warps per CTA
-    const size_t cap = (size_t)sm_count() * 8;
+    const size_t cap = (size_t)sm_count() * gather_ctas_per_sm(c, T, c.shared_inter > 0);
     if (blocks > cap)
         blocks = cap;
     return launch_pdl(gather_tokens_kernel, dim3((unsigned)blocks), dim3(256), 0, s, x, inv_perm, T, c.hidden,
@@ -700,15 +700,8 @@ cudaError_t launch_gather_rows(const moe_config_t &c, const __nv_bfloat16 *x, co
                                int T, __nv_bfloat16 *x_sorted, cudaStream_t s)
 {
     const int A = T * c.top_k;
-    const size_t total = (size_t)A * (c.hidden >> 3);
-    // An FFN CTA does not start on an SM while a CTA of another kernel is resident there
-    // (measured, whatever their shared-memory and register needs), so until this kernel has
-    // finished the gate/up pass runs its shared-expert tiles only on the SMs this kernel
-    // leaves alone.  Up to 16 MB of rows the gather therefore runs as one CTA per SM at most
-    // (the hardware places them on about half of the SMs; fewer, larger CTAs made the gather
-    // itself too slow); a large gather needs every SM's full thread count.
     size_t blocks = ((size_t)A + 7) / 8;  // a row per warp, eight warps per CTA
-    const size_t cap = (size_t)sm_count() * (total * 16 <= (16u << 20) ? 1 : 8);
+    const size_t cap = (size_t)sm_count() * gather_ctas_per_sm(c, T, true);
     if (blocks > cap)
         blocks = cap;
     return launch_pdl(gather_rows_kernel, dim3((unsigned)blocks), dim3(256), 0, s, x, perm, A,

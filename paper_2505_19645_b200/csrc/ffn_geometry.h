@@ -157,4 +157,18 @@ inline TileRows routed_tile_rows(const moe_config_t &c, int T, int routed_parts)
     return TileRows{low_up ? 64 : 128, down};
 }
 
+// CTAs per SM of the row gather.  An FFN CTA does not start on an SM while a CTA of another kernel is
+// resident there (measured, whatever their shared-memory and register needs), so until the gather has
+// finished the gate/up pass runs its shared-expert tiles only on the SMs the gather leaves alone.  Up
+// to 16 MB of rows it therefore runs as one CTA per SM at most (the hardware places them on about half
+// of the SMs; fewer, larger CTAs made the gather itself too slow); a large gather needs every SM's full
+// thread count.  Layer beyond 8192 assignments, eight CTAs per SM -> one, 16 experts top-4 of 256 and a
+// shared one of 512, T = 2080, us: hidden 128 48.4 -> 45.4, 512 65.3 -> 62.8, 992 80.3 -> 77.8;
+// 64 experts top-8, T = 2048, within 1 %.  Without a shared expert nothing could start early (8 experts
+// top-2 of 512, T = 4200, hidden 768: 67.4 -> 70.3).
+inline int gather_ctas_per_sm(const moe_config_t &c, int T, bool with_shared)
+{
+    return with_shared && (size_t)T * c.top_k * c.hidden * 2 <= (16u << 20) ? 1 : 8;
+}
+
 }  // namespace moe

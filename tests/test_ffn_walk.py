@@ -59,7 +59,7 @@ def _tiles(exe, calls):
     out = []
     for (H, _, _, I, *_), line in zip(calls, r.stdout.split("\n")):
         assert I < 2048   # (from there on the down pass may split its reduction)
-        ctas, up, down = map(int, line.split())
+        ctas, up, down, _ = map(int, line.split())
         cut = lambda rows, h: [min(h * ctas, rows - f) // ctas for f in range(0, rows, h * ctas)]  # noqa: E731
         out.append((ctas, cut(I, up), cut(H, down)))
     return out
@@ -141,3 +141,13 @@ def test_low_tiles_stand_where_they_were_faster(tmp_path):
     got = _tiles(_build(tmp_path / "tile", "tile_host.cc"), [c + (-1, 0) for c in MEASURED_HEIGHTS])
     for (call, heights), (_, up, down) in zip(MEASURED_HEIGHTS.items(), got):
         assert (max(up), max(down)) == heights, call
+
+
+def test_a_small_gather_leaves_sms_to_the_shared_expert(tmp_path):
+    """Up to 16 MB of rows the gather of a layer with a shared expert runs as one CTA per SM."""
+    calls = {(512, 16, 4, 256, 512, 2080): 1, (512, 16, 4, 256, 512, 4096): 1, (512, 16, 4, 256, 512, 4097): 8,
+             (512, 16, 4, 256, 0, 2080): 8, (7168, 256, 8, 2048, 2048, 3072): 8}
+    lines = ["%d %d %d %d %d %d -1 0" % (E, k, H, I, Is, T) for H, E, k, I, Is, T in calls]
+    r = subprocess.run([_build(tmp_path / "tile", "tile_host.cc")], input="\n".join(lines) + "\n",
+                       capture_output=True, text=True, check=True)
+    assert [int(v.split()[3]) for v in r.stdout.splitlines()] == list(calls.values())

@@ -332,6 +332,19 @@ def test_grouping_and_gather_of_medium_batches(E, k, T):
     check_layer_against_oracle(shape, w, x, T, 0)
 
 
+@pytest.mark.parametrize("H,E,k,Is,T", [
+    (2080, 16, 8, 32, 1026),   # rows of one piece of 2048 columns and 32 more, from the token's side
+    (96, 40, 16, 64, 520),     # rows shorter than a warp's 512 bytes
+    (512, 16, 4, 0, 2300),     # no shared expert
+])
+def test_gather_of_large_batches(H, E, k, Is, T):
+    """Beyond 8192 assignments: the row gather that reads a token once."""
+    shape = wl.small_shape("gather", H, E, k, 64, Is, 0, 1, 1 if Is else 0)
+    w = wl.make_weights(shape, 900 + E, "cuda")
+    x = wl.make_tokens(shape, T, 1000 + T, "cuda")
+    check_layer_against_oracle(shape, w, x, T, 0)
+
+
 PAIR_CASES = [
     # few items, low tiles (64 and 128 rows per CTA): a last gate/up tile of 48 and down tile of 16, 300
     # shared rows

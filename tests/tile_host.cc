@@ -2,7 +2,7 @@
 // 148 SMs, for calls read from the standard input, one a line:
 //   experts top_k hidden inter shared_inter tokens MOE_FF_WIDE MOE_FF_PAIR   (WIDE -1: unset)
 // prints, a line each: CTAs per worker, weight rows per CTA and tile of the gate/up and of the
-// (unsplit) down pass.
+// (unsplit) down pass, CTAs per SM of a large layer call's row gather.
 #include <stdint.h>
 #include <stdio.h>
 
@@ -50,7 +50,8 @@ int main()
     while (scanf("%d %d %d %d %d %d %d %d", &c.n_experts, &c.top_k, &c.hidden, &c.inter, &c.shared_inter, &T,
                  &g_wide, &g_pair) == 8) {
         const TileRows t = routed_tile_rows(c, T, 1);
-        printf("%d %d %d\n", ffn_workers(c, T).ctas, t.up, t.down);
+        printf("%d %d %d %d\n", ffn_workers(c, T).ctas, t.up, t.down,
+               gather_ctas_per_sm(c, T, c.shared_inter > 0));
     }
     return 0;
 }
