@@ -70,21 +70,28 @@ combine_kernel(const void *__restrict__ y, int routed_parts,
     const int vec_per_row = H >> 3;
     const size_t plane = (size_t)T * k * H;
     // A thread's pieces lie gridDim x CB_THREADS apart; their (token, column) advance by additions (no
-    // 64-bit division per piece), and the positions and weights of the next piece are requested while
-    // the rows of the current one are in flight.  Bound by loads in flight: 2 CTAs of 256 threads per SM with eight
-    // 16-byte row pieces each.  Alone, inputs larger than L2, us: DeepSeek-V3 shape T = 3072 96.3 -> 90.5
-    // (4.9 TB/s), T = 1024 36.5 -> 32.6, Qwen2 T = 1280 24.1 -> 22.0, Mixtral T = 1280 9.05 -> 7.77, Qwen1.5
-    // T = 640 4.18 -> 3.93, DeepSeek-V3 T = 128 equal; three CTAs per SM spill (128 us).
-    const unsigned step = gridDim.x * CB_THREADS, step_t = step / vec_per_row, step_v = step - step_t * vec_per_row;
+    // 64-bit division per piece), and the positions of the next piece are requested while the rows of
+    // the current one are in flight; the weights too where registers are left for them (one CTA per SM:
+    // top-16 of 7168 columns, T = 3072 172.0 -> 167.4 us), else they come with the rows (their registers
+    // spilled at eight rows: top-8 of 7168 columns, T = 1280 38.8 -> 37.7).  Bound by loads in flight:
+    // 2 CTAs of 256 threads per SM with eight 16-byte row pieces each.  A division per piece and no
+    // positions ahead -> this, alone, inputs larger than L2, us: top-8 of 7168 columns T = 3072
+    // 94.7 -> 86.8 (5.1 TB/s), T = 640 23.3 -> 20.6; of 3584, T = 1280 23.3 -> 20.6; top-2 of 3584,
+    // T = 1280 9.7 -> 8.9; top-4 of 2048, T = 640 5.8 -> 5.4; three CTAs per SM at eight rows spill.
+    constexpr bool WEIGHTS_AHEAD = KP > 8 && !F32;
+    const unsigned step = gridDim.x * CB_THREADS, step_t = step / vec_per_row;
+    const unsigned step_v = step - step_t * vec_per_row;
     const unsigned first = blockIdx.x * CB_THREADS + threadIdx.x;
     int t = (int)(first / vec_per_row), v8 = (int)(first - (unsigned)t * vec_per_row);
     int rows[KP];
-    float wts[KP];
+    float wts[WEIGHTS_AHEAD ? KP : 1];
+    auto weight = [&](int tok, int j) { return j < k ? topk_w[(size_t)tok * k + j] : 0.f; };
     auto fetch = [&](int tok) {
 #pragma unroll
         for (int j = 0; j < KP; ++j) {
             rows[j] = j < k ? inv_perm[(size_t)tok * k + j] : 0;
-            wts[j] = j < k ? topk_w[(size_t)tok * k + j] : 0.f;
+            if constexpr (WEIGHTS_AHEAD)
+                wts[j] = weight(tok, j);
         }
     };
     if (t < T)
@@ -106,7 +113,7 @@ combine_kernel(const void *__restrict__ y, int routed_parts,
             acc[q] = 0.f;
 #pragma unroll
         for (int j = 0; j < KP; ++j)
-            cur_w[j] = wts[j];
+            cur_w[j] = WEIGHTS_AHEAD ? wts[WEIGHTS_AHEAD ? j : 0] : weight(cur_t, j);
         t += (int)step_t;
         v8 += (int)step_v;
         if (v8 >= vec_per_row) {
@@ -163,9 +170,10 @@ cudaError_t launch_combine(const moe_config_t &c, const __nv_bfloat16 *y, int ro
         return cudaErrorInvalidValue;
     const size_t total = (size_t)T * (c.hidden >> 3);
     size_t blocks = (total + CB_THREADS - 1) / CB_THREADS;
-    // as many CTAs as are resident at once (see the launch bounds): every thread has the same number of
-    // pieces or one less
-    const size_t cap = (size_t)sm_count() * (f32 ? 1 : c.top_k <= 2 ? 4 : c.top_k <= 4 ? 3 : c.top_k <= 8 ? 2 : 1);
+    // as many CTAs as are resident at once (see the launch bounds): every thread has the same number
+    // of pieces or one less
+    const int per_sm = f32 ? 1 : c.top_k <= 2 ? 4 : c.top_k <= 4 ? 3 : c.top_k <= 8 ? 2 : 1;
+    const size_t cap = (size_t)sm_count() * per_sm;
     if (blocks > cap)
         blocks = cap;
 #define MOE_CB_LAUNCH(KP)                                                                        \

@@ -111,3 +111,16 @@ def test_oracle_under_asan_and_ubsan(tmp_path):
                        capture_output=True, text=True, timeout=600)
     assert r.returncode == 0 and "oracle clean" in r.stdout, r.stdout[-1500:] + r.stderr[-3000:]
     assert "runtime error" not in r.stderr and "AddressSanitizer" not in r.stderr, r.stderr[-3000:]
+
+
+def test_combine_instances_keep_their_values_in_registers(tmp_path):
+    """ptxas reports no spills in any instance of the combine: it is bound by the loads in flight, and
+    its launch bounds leave the instance for eight rows no register to spare."""
+    if not os.path.exists(NVCC):
+        pytest.skip("nvcc not installed")
+    r = subprocess.run([NVCC, "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
+                        "-I", os.path.join(ROOT, "include"), "-I", CSRC, "-Xptxas", "-v", "-c",
+                        os.path.join(CSRC, "combine.cu"), "-o", str(tmp_path / "combine.o")],
+                       capture_output=True, text=True, check=True)
+    spills = [line.strip() for line in (r.stdout + r.stderr).splitlines() if "spill stores" in line]
+    assert len(spills) == 8 and all(" 0 bytes spill stores, 0 bytes spill loads" in v for v in spills), spills
