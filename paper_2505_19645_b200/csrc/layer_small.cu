@@ -78,6 +78,7 @@ struct SmallArgs {
     int logit_chunks;       // ceil(H / LS_LOGIT_CHUNK)
     int chunk_r, chunks_r;  // columns per down-projection chunk of a routed group, their number
     int chunk_s, chunks_s;  // the same for the shared expert
+    int even;               // one token: the CTAs share the output features evenly
 };
 
 // ---- loads ---------------------------------------------------------------------------------
@@ -322,8 +323,11 @@ __device__ __forceinline__ int pull(int *counter, int lane)
 
 // ---- the kernel -------------------------------------------------------------------------------
 
-// VPL: logits per lane of the top-k
-template <int VPL, bool EVEN>
+// VPL: logits per lane of the top-k.  ONE: the instance for one token, without the code and the
+// registers of more rows (122 registers and no spills, against 128 and 52 / 80 bytes of them): one
+// token of the tiny, Qwen1.5, Mixtral, DeepSeek-V3 and Qwen2 shapes 14.7 -> 13.3, 34.8 -> 33.2,
+// 117.7 -> 114.7, 133.5 -> 129.0 and 143.4 -> 140.2 us.
+template <int VPL, bool ONE>
 __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallArgs a)
 {
     extern __shared__ __align__(16) float s_slot[];        // partial sums of the CTA's down items
@@ -349,7 +353,7 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
     const int G = gridDim.x, b = blockIdx.x;
     const int n_warps = G * LS_WARPS;
     const int gwarp = warp * G + b;  // consecutive work items land on different SMs
-    const int T = a.T, H = a.H, E = a.E, K = a.K, A = a.T * a.K;
+    const int T = ONE ? 1 : a.T, H = a.H, E = a.E, K = a.K, A = T * K;
     const int n_shared_items = a.Is >> 1;  // gate/up items of the shared expert
     const int per_group = a.I >> 1;        // gate/up items of an activated expert
 
@@ -647,7 +651,7 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
             if (item >= n_items)
                 break;
             const int g = item / per_group, i0 = (item - g * per_group) * 2;
-            const int e = s_grp_expert[g], row0 = s_grp_row0[g], n = s_grp_n[g];
+            const int e = s_grp_expert[g], row0 = s_grp_row0[g], n = ONE ? 1 : s_grp_n[g];
             const __nv_bfloat16 *wg = a.w_gate + (size_t)e * a.I * H;
             const __nv_bfloat16 *wu = a.w_up + (size_t)e * a.I * H;
 #define LS_ROUTED_GATEUP(NR)                                                             \
@@ -679,12 +683,14 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
     }
 
     // ---- 4: down projection of the CTA's output features, unit by unit ------------------------
-    // Blocks of LS_DOWN_ROWS features are dealt to the CTAs in turn.  EVEN: every CTA owns consecutive features
-    // instead, the same number or one less, its last block a short one (see even_features()).
-    const int feat0 = EVEN ? (int)((long long)b * H / G) : 0;
-    const int n_feat = EVEN ? (int)((long long)(b + 1) * H / G) - feat0
+    // Blocks of LS_DOWN_ROWS features are dealt to the CTAs in turn, or every CTA owns consecutive
+    // features, the same number or one less, its last block a short one (see even_features()).
+    const bool even = ONE && a.even;
+    const int feat0 = even ? (int)((long long)b * H / G) : b * LS_DOWN_ROWS;
+    const int n_feat = even ? (int)((long long)(b + 1) * H / G) - feat0
                             : owned_below(H / LS_DOWN_ROWS, b, G) * LS_DOWN_ROWS;
-    auto block_feature = [&](int k) { return EVEN ? feat0 + k * LS_DOWN_ROWS : (b + k * G) * LS_DOWN_ROWS; };
+    const int stride = even ? LS_DOWN_ROWS : LS_DOWN_ROWS * G;  // from one of its blocks to the next
+    auto block_feature = [&](int k) { return ONE ? feat0 + k * stride : (b + k * G) * LS_DOWN_ROWS; };
     const int my_blocks = (n_feat + LS_DOWN_ROWS - 1) / LS_DOWN_ROWS;
     const int n_uc = a.chunks_s + s_n_groups * a.chunks_r;  // (unit, column chunk) pairs
     {
@@ -698,7 +704,7 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
                 break;
             const int uc = item / my_blocks, k = item - uc * my_blocks;
             const int f0 = block_feature(k);
-            const int rows = EVEN ? min(LS_DOWN_ROWS, n_feat - k * LS_DOWN_ROWS) : LS_DOWN_ROWS;
+            const int rows = ONE ? min(LS_DOWN_ROWS, n_feat - k * LS_DOWN_ROWS) : LS_DOWN_ROWS;
             int unit, c, n_done;
             if (uc < a.chunks_s) {
                 unit = 0;
@@ -751,7 +757,7 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
 #undef LS_SHARED_DOWN
             } else {
                 const int g = unit - 1;
-                const int e = s_grp_expert[g], row0 = s_grp_row0[g], n = s_grp_n[g];
+                const int e = s_grp_expert[g], row0 = s_grp_row0[g], n = ONE ? 1 : s_grp_n[g];
                 const int c0 = c * a.chunk_r;
                 const int ncols = min(a.chunk_r, a.I - c0);
                 const __nv_bfloat16 *wd = a.w_down + (size_t)e * H * a.I;
@@ -776,81 +782,50 @@ __global__ void __launch_bounds__(LS_THREADS, 1) layer_small_kernel(const SmallA
     if (s_abort)
         return;
 
-    // ---- 5: combine the CTA's features -----------------------------------------------------------
-    if constexpr (EVEN) {
-        for (int idx = tid; idx < n_feat * T; idx += LS_THREADS) {
-            const int t = idx / n_feat, f = idx - t * n_feat;
-            const int k = f / LS_DOWN_ROWS, j = f - k * LS_DOWN_ROWS;
-            // the sum of a (unit, chunk) for this feature and the unit's row r
-            auto part = [&](int uc, int r) {
-                return s_slot[((size_t)uc * my_blocks + k) * LS_SLOT_FLOATS + j * LS_MAX_TOKENS + r];
-            };
-            float o = 0.f;
-            for (int slot_j = 0; slot_j < K; ++slot_j) {
-                const int asg = t * K + slot_j;
-                float y = 0.f;
-                for (int c = 0; c < a.chunks_r; ++c)
-                    y += part(a.chunks_s + s_group_of[asg] * a.chunks_r + c, s_row_of[asg]);
-                o = fmaf(s_gate_w[asg], y, o);
-            }
-            if (a.Is > 0) {
-                float y = 0.f;
-                for (int c = 0; c < a.chunks_s; ++c)
-                    y += part(c, t);
-                o = fmaf(a.gated ? s_shared_scale[t] : 1.0f, y, o);
-            }
-            a.out[(size_t)t * H + block_feature(k) + j] = __float2bfloat16_rn(o);
+    // ---- 5: combine the CTA's features, a block per thread and token (ONE: a feature) -------------
+    constexpr int W = ONE ? 1 : LS_DOWN_ROWS;
+    for (int idx = tid; idx < (ONE ? n_feat : my_blocks) * T; idx += LS_THREADS) {
+        const int p = idx / T, t = idx - p * T;
+        const int k = ONE ? p / LS_DOWN_ROWS : p, j0 = ONE ? p - k * LS_DOWN_ROWS : 0;
+        // adds the sums of a (unit, chunk) for the unit's row r
+        auto add = [&](float (&y)[W], int uc, int r) {
+            const float *slot = s_slot + ((size_t)uc * my_blocks + k) * LS_SLOT_FLOATS + r;
+#pragma unroll
+            for (int j = 0; j < W; ++j)
+                y[j] += slot[(j0 + j) * LS_MAX_TOKENS];
+        };
+        float o[W] = {};
+        for (int slot_j = 0; slot_j < K; ++slot_j) {
+            const int asg = t * K + slot_j;
+            const int uc0 = a.chunks_s + s_group_of[asg] * a.chunks_r;
+            float y[W] = {};
+            for (int c = 0; c < a.chunks_r; ++c)
+                add(y, uc0 + c, s_row_of[asg]);
+            const float gw = s_gate_w[asg];
+#pragma unroll
+            for (int j = 0; j < W; ++j)
+                o[j] = fmaf(gw, y[j], o[j]);
         }
-    } else {
-        for (int idx = tid; idx < my_blocks * T; idx += LS_THREADS) {
-            const int k = idx / T, t = idx - k * T;
-            const int f0 = (b + k * G) * LS_DOWN_ROWS;
-            float o[LS_DOWN_ROWS];
+        if (a.Is > 0) {
+            float y[W] = {};
+            for (int c = 0; c < a.chunks_s; ++c)
+                add(y, c, t);
+            const float sc = a.gated ? s_shared_scale[t] : 1.0f;
 #pragma unroll
-            for (int j = 0; j < LS_DOWN_ROWS; ++j)
-                o[j] = 0.f;
-            for (int slot_j = 0; slot_j < K; ++slot_j) {
-                const int asg = t * K + slot_j;
-                const int uc0 = a.chunks_s + s_group_of[asg] * a.chunks_r;
-                const int r = s_row_of[asg];
-                float y[LS_DOWN_ROWS];
-#pragma unroll
-                for (int j = 0; j < LS_DOWN_ROWS; ++j)
-                    y[j] = 0.f;
-                for (int c = 0; c < a.chunks_r; ++c) {
-                    const float *slot = s_slot + ((size_t)(uc0 + c) * my_blocks + k) * LS_SLOT_FLOATS;
-#pragma unroll
-                    for (int j = 0; j < LS_DOWN_ROWS; ++j)
-                        y[j] += slot[j * LS_MAX_TOKENS + r];
-                }
-                const float gw = s_gate_w[asg];
-#pragma unroll
-                for (int j = 0; j < LS_DOWN_ROWS; ++j)
-                    o[j] = fmaf(gw, y[j], o[j]);
-            }
-            if (a.Is > 0) {
-                float y[LS_DOWN_ROWS];
-#pragma unroll
-                for (int j = 0; j < LS_DOWN_ROWS; ++j)
-                    y[j] = 0.f;
-                for (int c = 0; c < a.chunks_s; ++c) {
-                    const float *slot = s_slot + ((size_t)c * my_blocks + k) * LS_SLOT_FLOATS;
-#pragma unroll
-                    for (int j = 0; j < LS_DOWN_ROWS; ++j)
-                        y[j] += slot[j * LS_MAX_TOKENS + t];
-                }
-                const float sc = a.gated ? s_shared_scale[t] : 1.0f;
-#pragma unroll
-                for (int j = 0; j < LS_DOWN_ROWS; ++j)
-                    o[j] = fmaf(sc, y[j], o[j]);
-            }
-            static_assert(LS_DOWN_ROWS == 4, "the store below writes two bf16 pairs");
+            for (int j = 0; j < W; ++j)
+                o[j] = fmaf(sc, y[j], o[j]);
+        }
+        __nv_bfloat16 *dst = a.out + (size_t)t * H + block_feature(k) + j0;
+        if constexpr (ONE) {
+            *dst = __float2bfloat16_rn(o[0]);
+        } else {
+            static_assert(ONE || W == 4, "the store below writes two bf16 pairs");
             const __nv_bfloat162 lo = __floats2bfloat162_rn(o[0], o[1]);
             const __nv_bfloat162 hi = __floats2bfloat162_rn(o[2], o[3]);
             uint2 packed;
             packed.x = *reinterpret_cast<const uint32_t *>(&lo);
             packed.y = *reinterpret_cast<const uint32_t *>(&hi);
-            *reinterpret_cast<uint2 *>(a.out + (size_t)t * H + f0) = packed;
+            *reinterpret_cast<uint2 *>(dst) = packed;
         }
     }
 }
@@ -987,7 +962,7 @@ bool layer_small_applies(const moe_config_t &c, int T)
     return small_shape(c, T) && small_layer_override() != 0 && cooperative_ok();
 }
 
-template <int VPL, bool EVEN>
+template <int VPL, bool ONE>
 static cudaError_t launch_variant(const SmallArgs &a, size_t smem, cudaStream_t s)
 {
     static DeviceOnce configured;
@@ -996,8 +971,8 @@ static cudaError_t launch_variant(const SmallArgs &a, size_t smem, cudaStream_t 
     if (err != cudaSuccess)
         return err;
     if (!configured.done(dev)) {
-        err = cudaFuncSetAttribute(layer_small_kernel<VPL, EVEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)LS_MAX_SLOT_BYTES);
+        err = cudaFuncSetAttribute(layer_small_kernel<VPL, ONE>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LS_MAX_SLOT_BYTES);
         if (err != cudaSuccess)
             return err;
         configured.mark(dev);
@@ -1012,33 +987,36 @@ static cudaError_t launch_variant(const SmallArgs &a, size_t smem, cudaStream_t 
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, layer_small_kernel<VPL, EVEN>, a);
+    return cudaLaunchKernelEx(&cfg, layer_small_kernel<VPL, ONE>, a);
 }
 
-// Whether the CTAs share the output features evenly instead of in whole blocks.  With a handful of blocks
-// per CTA those with one more are the last to finish (Qwen1.5 shape: 4 or 3 for 2048 / 148 = 13.8 features); one
-// token 36.8 -> 35.4 us per call.  More tokens make the short blocks' idle rows cost what they level (two tokens
-// equal, four 75.0 -> 75.8); from six blocks on there is less to level (Qwen2 shape, 6.05 blocks: equal; DeepSeek-V3
-// shape, 12.1, four tokens: 447 -> 451), and up to one block per CTA nothing.
-constexpr int LS_EVEN_BLOCKS = 6;
+// Whether the CTAs of a one-token call share the output features evenly instead of in whole blocks, so
+// that none has a block more than others to finish last (Qwen1.5 shape: four or three blocks for
+// 2048 / 148 = 13.8 features).  The price is a short last block in every CTA, whose missing rows leave
+// loads unused.  Blocks -> even, us per call, hidden 256 to 7168 on six kinds of experts: Qwen1.5
+// shape 34.2 -> 32.7, between two and six blocks per CTA 0.5 % less in the mean (-4.3 to +2.0 %), below
+// that 0.3 to 5 % more (hidden 640 and 768 with 32 experts of 512 23.8 -> 24.7 and +6 %: two items
+// per CTA and unit instead of one), from six blocks on equal (Qwen2 shape 140.1 -> 140.2, DeepSeek-V3
+// shape 129.0 -> 128.6).  With two tokens equal, with four 75.0 -> 75.8.
+constexpr int LS_EVEN_MIN_BLOCKS = 2, LS_EVEN_MAX_BLOCKS = 6;
 static bool even_features(const moe_config_t &c, int T)
 {
     const int blocks = c.hidden / LS_DOWN_ROWS;
-    return T == 1 && blocks > sm_count() && blocks < LS_EVEN_BLOCKS * sm_count();
+    return T == 1 && blocks > LS_EVEN_MIN_BLOCKS * sm_count() && blocks < LS_EVEN_MAX_BLOCKS * sm_count();
 }
 
-template <bool EVEN>
-static cudaError_t launch_even(const SmallArgs &a, int E, size_t smem, cudaStream_t s)
+template <bool ONE>
+static cudaError_t launch_rows(const SmallArgs &a, size_t smem, cudaStream_t s)
 {
-    if (E <= 32)
-        return launch_variant<1, EVEN>(a, smem, s);
-    if (E <= 64)
-        return launch_variant<2, EVEN>(a, smem, s);
-    if (E <= 128)
-        return launch_variant<4, EVEN>(a, smem, s);
-    if (E <= 256)
-        return launch_variant<8, EVEN>(a, smem, s);
-    return launch_variant<16, EVEN>(a, smem, s);
+    if (a.E <= 32)
+        return launch_variant<1, ONE>(a, smem, s);
+    if (a.E <= 64)
+        return launch_variant<2, ONE>(a, smem, s);
+    if (a.E <= 128)
+        return launch_variant<4, ONE>(a, smem, s);
+    if (a.E <= 256)
+        return launch_variant<8, ONE>(a, smem, s);
+    return launch_variant<16, ONE>(a, smem, s);
 }
 
 cudaError_t launch_layer_small(const moe_config_t &c, const moe_weights_t &w, const __nv_bfloat16 *x,
@@ -1099,9 +1077,9 @@ cudaError_t launch_layer_small(const moe_config_t &c, const moe_weights_t &w, co
     a.chunk_r = down_chunk_cols(c, c.inter);
     a.chunks_s = down_chunks(c, c.shared_inter);
     a.chunk_s = down_chunk_cols(c, c.shared_inter);
+    a.even = even_features(c, T) ? 1 : 0;
     const size_t smem = slot_bytes(c, T);
-    const int E = c.n_experts;
-    return even_features(c, T) ? launch_even<true>(a, E, smem, s) : launch_even<false>(a, E, smem, s);
+    return T == 1 ? launch_rows<true>(a, smem, s) : launch_rows<false>(a, smem, s);
 }
 
 }  // namespace moe

@@ -117,6 +117,23 @@ def test_few_token_case(name, H, E, k, I, Is, score, renorm, sgate, B, gamma, zi
     check_layer_against_oracle(shape, w, x, B, gamma)
 
 
+@pytest.mark.parametrize("H,E", [
+    (32, 8),       # fewer blocks of four features than CTAs: most CTAs have none
+    (1184, 100),   # two blocks in every CTA
+    (1216, 40),    # (from here) even shares: eight or nine features, the last block of one or none
+    (2080, 300),   # fourteen or fifteen
+    (3520, 130),   # 23 or 24
+    (3552, 20),    # blocks again: six in every CTA
+])
+def test_one_token_shares_of_the_output_features(H, E):
+    """The one-token instance with whole blocks and with even shares of the features, at every width
+    of its top-k."""
+    shape = wl.small_shape("one", H, E, 3, 416, 288, 0, 1, 1)
+    w = wl.make_weights(shape, 520 + H, "cuda")
+    x = wl.make_tokens(shape, 1, 620 + H, "cuda")
+    check_layer_against_oracle(shape, w, x, 1, 0)
+
+
 def test_few_tokens_take_one_launch():
     from paper_2505_19645_b200 import api
 
