@@ -236,8 +236,8 @@ cudaError_t launch_tagged_wait_selftest(int32_t *status, int limit_us, cudaStrea
 cudaError_t launch_gather_rows(const moe_config_t &c, const __nv_bfloat16 *x, const int32_t *perm,
                                int T, __nv_bfloat16 *x_sorted, cudaStream_t s);
 // the same with the inverse permutation (a layer call's)
-cudaError_t launch_gather_tokens(const moe_config_t &c, const __nv_bfloat16 *x, const int32_t *inv_perm, int T,
-                                 __nv_bfloat16 *x_sorted, cudaStream_t s);
+cudaError_t launch_gather_tokens(const moe_config_t &c, const __nv_bfloat16 *x, const int32_t *inv_perm,
+                                 int T, __nv_bfloat16 *x_sorted, cudaStream_t s);
 // y and shared_y may hold `routed_parts` / `shared_parts` partial planes ([A,H] / [T,H]: k
 // chunks of the down pass), summed here; f32: they hold floats
 cudaError_t launch_combine(const moe_config_t &c, const __nv_bfloat16 *y, int routed_parts,

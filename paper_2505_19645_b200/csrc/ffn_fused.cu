@@ -651,13 +651,14 @@ gather_rows_kernel(const __nv_bfloat16 *__restrict__ x, const int32_t *__restric
     }
 }
 
-// The same from the token's side, where the inverse permutation is at hand (a layer call): a warp reads
-// a piece of 2048 columns once and writes it to its top_k places.  Bound by the writes; gather_rows_kernel also
-// reads every row top_k times.  Alone, us: DeepSeek-V3 shape T = 3072 96 -> 71 (5.6 TB/s of rows read and written
-// once), T = 1536 43.5 -> 35.7, Qwen2 T = 1280 and 2048 equal; layer at T = 3072 4440 -> 4410.
+// The same from the token's side, where the inverse permutation is at hand (a layer call): a warp
+// reads a piece of 2048 columns once and writes it to its top_k places.  Bound by the writes;
+// gather_rows_kernel also reads every row top_k times.  Alone, us: DeepSeek-V3 shape T = 3072 96 -> 71
+// (5.6 TB/s of rows read and written once), T = 1536 43.5 -> 35.7, Qwen2 T = 1280 and 2048 equal;
+// layer, 64 experts top-8 of 256, T = 2048: hidden 256 63.1 -> 56.7, 1024 114.1 -> 111.3.
 __global__ void __launch_bounds__(256)
-gather_tokens_kernel(const __nv_bfloat16 *__restrict__ x, const int32_t *__restrict__ inv_perm, int T, int H,
-                     int top_k, __nv_bfloat16 *__restrict__ x_sorted)
+gather_tokens_kernel(const __nv_bfloat16 *__restrict__ x, const int32_t *__restrict__ inv_perm, int T,
+                     int H, int top_k, __nv_bfloat16 *__restrict__ x_sorted)
 {
     griddep_launch();
     griddep_wait();
@@ -675,7 +676,8 @@ gather_tokens_kernel(const __nv_bfloat16 *__restrict__ x, const int32_t *__restr
             if (v0 + 32 * u < vec_per_row)
                 d[u] = src[v0 + 32 * u];
         for (int j = 0; j < top_k; ++j) {
-            uint4 *dst = reinterpret_cast<uint4 *>(x_sorted + (size_t)__shfl_sync(0xffffffffu, place, j) * H);
+            const int row = __shfl_sync(0xffffffffu, place, j);
+            uint4 *dst = reinterpret_cast<uint4 *>(x_sorted + (size_t)row * H);
 #pragma unroll
             for (int u = 0; u < GATHER_UNROLL; ++u)
                 if (v0 + 32 * u < vec_per_row)
@@ -684,16 +686,16 @@ gather_tokens_kernel(const __nv_bfloat16 *__restrict__ x, const int32_t *__restr
     }
 }
 
-cudaError_t launch_gather_tokens(const moe_config_t &c, const __nv_bfloat16 *x, const int32_t *inv_perm, int T,
-                                 __nv_bfloat16 *x_sorted, cudaStream_t s)
+cudaError_t launch_gather_tokens(const moe_config_t &c, const __nv_bfloat16 *x, const int32_t *inv_perm,
+                                 int T, __nv_bfloat16 *x_sorted, cudaStream_t s)
 {
     const int vec = c.hidden >> 3, pieces = (vec + 32 * GATHER_UNROLL - 1) / (32 * GATHER_UNROLL);
     size_t blocks = ((size_t)T * pieces + 7) / 8;  // a piece of a row per warp, eight warps per CTA
     const size_t cap = (size_t)sm_count() * gather_ctas_per_sm(c, T, c.shared_inter > 0);
     if (blocks > cap)
         blocks = cap;
-    return launch_pdl(gather_tokens_kernel, dim3((unsigned)blocks), dim3(256), 0, s, x, inv_perm, T, c.hidden,
-                      c.top_k, x_sorted);
+    return launch_pdl(gather_tokens_kernel, dim3((unsigned)blocks), dim3(256), 0, s, x, inv_perm, T,
+                      c.hidden, c.top_k, x_sorted);
 }
 
 cudaError_t launch_gather_rows(const moe_config_t &c, const __nv_bfloat16 *x, const int32_t *perm,
